@@ -94,9 +94,9 @@ typedef enum {
 } asm_local_solver;
 
 /* Orthogonalisation of the GMRES Arnoldi step (Section 2 uses modified Gram-Schmidt).  The
- * paper has no classical option; it is offered because on this GPU every projection of MGS is a
- * global reduction (a grid-wide barrier per projection), while classical Gram-Schmidt takes the
- * same FP64 work with two global reductions per step.  It rounds differently and keeps the basis
+ * paper has no classical option.  Classical Gram-Schmidt takes two global reductions per step; the
+ * modified form takes one per block of basis vectors (4, 8 or 32 of them, by the vectors' length) and
+ * one for the norm.  It rounds differently and keeps the basis
  * less orthogonal (loss ~ cond^2 eps instead of cond eps), so iteration counts may differ from
  * MGS and from the oracle; tests hold it to the solution tolerance.  It applies to single-system
  * GMRES solves with the cooperative Gram-Schmidt (ASM_TUNE_COOP_ORTHO = 1) and restart <= 62;
@@ -267,7 +267,7 @@ int asm_get_stats(asm_handle h, asm_stats* st);
  *                        3: all in shared memory (2 and 3 fall back to device memory when they do
  *                        not fit);
  *   ASM_TUNE_COOP_ORTHO  1 (default) runs the Gram-Schmidt step of a single-system solve in one
- *                        cooperative launch, 0 in one launch per projection.
+ *                        cooperative launch, 0 in one launch per block of basis vectors.
  * Errors: INVALID_ARG for an unknown key or value. */
 typedef enum {
     ASM_TUNE_APPLY_SMEM = 0,

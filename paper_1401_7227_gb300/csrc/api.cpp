@@ -776,7 +776,8 @@ void ensure_workspace(asm_ctx* h) {
     if (h->ws_m == m && h->ws_flex == flex && h->d_ws.p) return;
     const long long n3 = 3LL * h->N;
     h->n3p = (n3 + VEC_CHUNK - 1) / VEC_CHUNK * VEC_CHUNK;
-    h->nchunk = (int)(h->n3p / VEC_CHUNK);
+    const int vchunk = vec_item_len(n3), gs_block = gs_block_size(n3);
+    h->nchunk = (int)(h->n3p / vchunk);
     // GMRES: V_0..V_m (+ Z_0..Z_{m-1} when flexible); ORTHOMIN: P_0..P_k, Q_0..Q_k
     const int nslots = om ? VV0 + 2 * (m + 1) : VV0 + m + 1 + (flex ? m : 0);
     h->d_ws.alloc((size_t)nslots * h->n3p * sizeof(double));
@@ -786,9 +787,10 @@ void ensure_workspace(asm_ctx* h) {
     h->d_scal.zero(h->stream);
     h->d_ctl.alloc(C_NCTL * sizeof(int));
     h->d_ctl.zero(h->stream);
-    // chunk partials; the cooperative Gram-Schmidt's per-CTA partials (classical: kCgsMax values per
-    // CTA, at most two CTAs per SM)
-    h->d_partial.alloc(std::max<size_t>((size_t)4 * std::max(h->nchunk, 4096), (size_t)kCgsMax * 2 * 1024) *
+    // chunk partials (a dot and a Gram entry per vector of a block, and a norm); the cooperative
+    // Gram-Schmidt's per-CTA partials (classical: kCgsMax values per CTA; blocked: two sets of
+    // 2 kGsMaxBlock + 1; at most two CTAs per SM)
+    h->d_partial.alloc(std::max<size_t>((size_t)(2 * kGsMaxBlock + 1) * h->nchunk, (size_t)(4 * kGsMaxBlock + 4) * 1024) *
                        sizeof(double));
     h->ws_m = m;
     h->ws_flex = flex;
@@ -802,6 +804,8 @@ void ensure_workspace(asm_ctx* h) {
     t.krylov = om ? 1 : 0;
     t.ortho = om ? 0 : h->opt.ortho;
     t.nchunk = h->nchunk;
+    t.vchunk = vchunk;
+    t.gs_block = gs_block;
     t.scal = h->d_scal.as<double>();
     t.ctl = h->d_ctl.as<int>();
     t.partial = h->d_partial.as<double>();
@@ -1265,6 +1269,9 @@ void launch_local_solves(Batch& B, const SysTab* tab, cudaStream_t st) {
     }
 }
 
+// index of the last Gram-Schmidt pass of a system's Arnoldi step j (one per block, one for the norm)
+int gs_passes(const asm_ctx* h, int j) { return (j + h->tab.gs_block) / h->tab.gs_block; }
+
 void launch_step(Batch& B, int kmax, cudaStream_t st, StepEvents* ev) {
     const SysTab* tab = B.d_tab.as<SysTab>();
     const VecItem* vi = B.d_vec.as<VecItem>();
@@ -1283,7 +1290,7 @@ void launch_step(Batch& B, int kmax, cudaStream_t st, StepEvents* ev) {
     if (ev) ck(cudaEventRecord(ev->e[4], st));
     long long n = 4 + local_solve_launches(B);
     if (B.coop_grid > 0) {
-        ck(launch_ortho_coop(tab, B.hs[0]->d_partial.as<double>(), B.coop_grid, st));
+        ck(launch_ortho_coop(tab, B.hs[0]->d_partial.as<double>(), B.coop_grid, B.hs[0]->tab.ortho, B.hs[0]->tab.n3, st));
         n += 1;
     } else {
         for (int k = 0; k <= kmax; k++) launch_mgs(tab, vi, B.nvec, k, st);
@@ -1378,7 +1385,7 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
     for (size_t k = 0; k < hs.size(); k++) begin_solve(hs[k], b[k], on_device, rtol, max_iter);
     build_batch(B, st);
     const bool om = hs[0]->opt.krylov == ASM_KRYLOV_ORTHOMIN;
-    if (hs.size() == 1 && !hs[0]->no_coop && !om) B.coop_grid = ortho_coop_grid(hs[0]->device);
+    if (hs.size() == 1 && !hs[0]->no_coop && !om) B.coop_grid = ortho_coop_grid(hs[0]->device, hs[0]->tab.ortho, hs[0]->tab.n3);
     {
         // initial step: x = 0, r = b, beta = ||b||
         const SysTab* tab = B.d_tab.as<SysTab>();
@@ -1387,7 +1394,7 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
         if (om) {
             launch_om(tab, vi, B.nvec, 0, st);
         } else if (B.coop_grid > 0) {
-            ck(launch_ortho_coop(tab, hs[0]->d_partial.as<double>(), B.coop_grid, st));
+            ck(launch_ortho_coop(tab, hs[0]->d_partial.as<double>(), B.coop_grid, hs[0]->tab.ortho, hs[0]->tab.n3, st));
         } else {
             launch_mgs(tab, vi, B.nvec, 0, st);
             launch_finish(tab, vi, B.nvec, st);
@@ -1455,7 +1462,7 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
             const int* c = B.pinned + k * C_NCTL;
             if (c[C_PHASE] == PH_DONE) continue;
             any = true;
-            if (c[C_PHASE] == PH_ARNOLDI) kmax = std::max(kmax, c[C_J] + 1);
+            if (c[C_PHASE] == PH_ARNOLDI) kmax = std::max(kmax, gs_passes(hs[k], c[C_J]));
             else if (c[C_PHASE] == PH_OM) kmax = std::max(kmax, c[C_OM_STORED]);
             else kmax = std::max(kmax, 0);
         }
@@ -2726,7 +2733,7 @@ int asm_server_progress(asm_server_handle S, int max_steps, int* n_active, int* 
                     continue;
                 }
                 keep.push_back(S->active[k]);
-                kmax = std::max(kmax, c[C_PHASE] == PH_ARNOLDI ? c[C_J] + 1 : 0);
+                kmax = std::max(kmax, c[C_PHASE] == PH_ARNOLDI ? gs_passes(S->active[k]->h, c[C_J]) : 0);
             }
             if (S->dirty) {  // membership changed: retired systems leave, waiting ones join
                 S->active.swap(keep);
@@ -2743,7 +2750,8 @@ int asm_server_progress(asm_server_handle S, int max_steps, int* n_active, int* 
                 kmax = -1;
                 for (size_t k = 0; k < S->active.size(); k++) {
                     const int* c = S->batch.pinned + k * C_NCTL;
-                    if (c[C_PHASE] != PH_DONE) kmax = std::max(kmax, c[C_PHASE] == PH_ARNOLDI ? c[C_J] + 1 : 0);
+                    if (c[C_PHASE] != PH_DONE)
+                        kmax = std::max(kmax, c[C_PHASE] == PH_ARNOLDI ? gs_passes(S->active[k]->h, c[C_J]) : 0);
                 }
             }
             launch_step(S->batch, kmax, S->stream, nullptr);

@@ -13,7 +13,14 @@ namespace asm2 {
 // Krylov workspace layout.  Each system owns one device block of vectors of n3p doubles
 // (n3 = 3 * n_cells rounded up to VEC_CHUNK), addressed by slot number.
 // ---------------------------------------------------------------------------------------------
-constexpr int VEC_CHUNK = 4096;   // elements per vector work item (256 threads x 16)
+constexpr int VEC_CHUNK = 4096;   // vectors are padded to whole chunks of this many elements
+// Elements per vector work item (one CTA of 256 threads): a quarter of a chunk for short vectors, so
+// that a few of them fill the chip, a whole one where the partial sums of a long vector would
+// otherwise outnumber what the last CTA adds up quickly.
+inline int vec_item_len(long long n3) { return n3 <= 400000 ? VEC_CHUNK / 4 : VEC_CHUNK; }
+// Basis vectors per reduction of the blocked modified Gram-Schmidt, and per sweep over the vectors
+constexpr int kGsMaxBlock = 32, kGsGroup = 8, kGsLong = 4;
+inline int gs_block_size(long long n3) { return n3 <= 131072 ? kGsMaxBlock : kGsGroup; }
 // bytes of one factor-stream chunk (= one shared-memory ring slot of the apply): chosen per subdomain
 // so that its largest fine level fits one chunk, within [kStreamChunkMin, kStreamChunkMax]
 constexpr int kStreamChunkMin = 8192, kStreamChunkMax = 24576;
@@ -68,7 +75,7 @@ enum Ctl {
 
 // Per-system scalars (device, double) at fixed offsets; H is (m+1) x m row-major.
 struct ScalLayout {
-    int bnorm, beta, tol, w0, hn, red0, red1, H, cs, sn, g, y, om_qq, om_beta, om_alpha, n;
+    int bnorm, beta, tol, w0, hn, red0, red1, H, cs, sn, g, y, om_qq, om_beta, om_alpha, gram, n;
     __host__ __device__ static ScalLayout make(int m) {
         ScalLayout L;
         int o = 0;
@@ -94,6 +101,8 @@ struct ScalLayout {
         L.om_beta = o;  // ORTHOMIN: projection coefficients of the step in progress
         o += m;
         L.om_alpha = o++;
+        L.gram = o;  // (v_k, v_i) of the vectors i < k in k's Gram-Schmidt block, kGsMaxBlock per vector
+        o += (m + 1) * kGsMaxBlock;
         L.n = o;
         return L;
     }
@@ -110,9 +119,11 @@ struct SysTab {
     int krylov;          // asm_krylov: 0 GMRES (slots V_k, Z_k), 1 ORTHOMIN (slots P_s, then Q_s)
     int ortho;           // asm_ortho: 0 modified, 1 classical Gram-Schmidt (single-system GMRES)
     int nchunk;          // vector work items of this system
+    int vchunk;          // elements per vector work item
+    int gs_block;        // basis vectors per Gram-Schmidt reduction (kGsGroup or kGsMaxBlock)
     double* scal;        // scalars (ScalLayout)
     int* ctl;            // control words (Ctl)
-    double* partial;     // [2 * nchunk] chunk partial sums
+    double* partial;     // [nchunk * (2 gs_block + 1)] chunk partial sums
     // A in ELL form: slot w, element t of row r at ell_val[(w*9 + t) * rows_pad + r]
     const double* ell_val;
     const int* ell_col;  // [w * rows_pad + r]; padding slots point at r with zero values
@@ -137,7 +148,7 @@ struct SysTab {
 };
 
 // Work items
-struct VecItem {   // VEC_CHUNK elements [e0, e0 + VEC_CHUNK) of system sys; chunk index within system
+struct VecItem {   // elements [chunk vchunk, (chunk + 1) vchunk) of system sys
     int sys, chunk;
 };
 struct RowItem {   // rows [r0, r0 + 256) of system sys
@@ -297,7 +308,8 @@ void launch_spmv(const SysTab* st_tab, const RowItem* items, int nitems, cudaStr
 void launch_init(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);
 void launch_prep(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);
 void launch_post(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);
-void launch_mgs(const SysTab* tab, const VecItem* items, int nitems, int k, cudaStream_t st);
+// pass 0 .. number of Gram-Schmidt blocks of the step
+void launch_mgs(const SysTab* tab, const VecItem* items, int nitems, int pass, cudaStream_t st);
 void launch_finish(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);
 // ORTHOMIN(k): projection pass l of the direction in progress (l = 0 also reduces ||r|| of
 // initial systems and ||b - A x|| of finishing ones), then x += alpha p, r -= alpha q.
@@ -343,10 +355,10 @@ cudaError_t launch_coarse_invert(const long long* keys, const double* blocks, in
 void launch_coarse_apply(const SysTab* tab, const RowItem* rows, int nrows, const BoxItem* boxes, int nboxes,
                          const RowItem* grows, int ngrows, const VecItem* vecs, int nvecs, bool two_stage,
                          cudaStream_t st);
-// Whole Gram-Schmidt + state step of a single system in one cooperative launch (grid <= the
-// co-resident limit from ortho_coop_grid); part2 holds 4 * nchunk doubles.
-int ortho_coop_grid(int device);
-cudaError_t launch_ortho_coop(const SysTab* tab, double* part2, int grid, cudaStream_t st);
+// Whole Gram-Schmidt + state step of a single system of n3 unknowns in one cooperative launch of
+// ortho_coop_grid CTAs (0: the launch is not possible)
+int ortho_coop_grid(int device, int ortho, int n3);
+cudaError_t launch_ortho_coop(const SysTab* tab, double* part2, int grid, int ortho, int n3, cudaStream_t st);
 
 // Read-only view of the device matrix of a handle (used by the no-allocation residual)
 struct MatrixView {

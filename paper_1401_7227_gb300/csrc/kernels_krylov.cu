@@ -82,6 +82,20 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
     __syncthreads();
 }
 
+// single-value form of block_sum2 (the same summation order for that value)
+__device__ __forceinline__ void block_sum1(double& a) {
+    __shared__ double s0[VEC_THREADS];
+    s0[threadIdx.x] = a;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double x = 0.0;
+        for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) x += s0[i];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        a = x;
+    }
+    __syncthreads();
+}
+
 // Publish this chunk's partials; returns true in thread 0.. of the last chunk of its system,
 // with (s0, s1) = the ordered total.
 __device__ bool finish_reduction(const SysTab& st, int chunk, double& s0, double& s1) {
@@ -116,8 +130,8 @@ __global__ void __launch_bounds__(VEC_THREADS) k_init(const SysTab* __restrict__
     double* x = vec(st, VX);
     const double* b = vec(st, VB);
     double* r = vec(st, VR);
-    const long long e0 = (long long)it.chunk * VEC_CHUNK;
-    for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
+    const long long e0 = (long long)it.chunk * st.vchunk;
+    for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
         x[e0 + i] = 0.0;
         r[e0 + i] = b[e0 + i];
     }
@@ -131,9 +145,9 @@ __global__ void __launch_bounds__(VEC_THREADS) k_prep(const SysTab* __restrict__
     const int jend = st.ctl[C_JEND];
     const ScalLayout SL = ScalLayout::make(st.m);
     const double* yv = st.scal + SL.y;
-    const long long e0 = (long long)it.chunk * VEC_CHUNK;
+    const long long e0 = (long long)it.chunk * st.vchunk;
     double* dst = st.flexible ? vec(st, VX) : vec(st, VU);
-    for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
+    for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
         double acc = st.flexible ? dst[e0 + i] : 0.0;
         for (int k = 0; k < jend; k++) acc += yv[k] * vec(st, st.flexible ? zslot(st, k) : VV0 + k)[e0 + i];
         dst[e0 + i] = acc;
@@ -147,62 +161,263 @@ __global__ void __launch_bounds__(VEC_THREADS) k_post(const SysTab* __restrict__
     if (st.ctl[C_PHASE] != PH_RESTART || st.flexible) return;
     double* x = vec(st, VX);
     const double* z = vec(st, VZ);
-    const long long e0 = (long long)it.chunk * VEC_CHUNK;
-    for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) x[e0 + i] += z[e0 + i];
+    const long long e0 = (long long)it.chunk * st.vchunk;
+    for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) x[e0 + i] += z[e0 + i];
 }
 
-// MGS step k of Arnoldi column j: w -= h_{k-1,j} v_{k-1} (k >= 1), then h_{k,j} = (w, v_k)
-// (k <= j) or h_{j+1,j} = ||w|| (k = j + 1).  k = 0 also gives ||w|| before orthogonalisation.
-// Restart/init systems compute beta = ||r|| at k = 0.
-__global__ void __launch_bounds__(VEC_THREADS) k_mgs(const SysTab* __restrict__ tab, const VecItem* __restrict__ items,
-                                                     int k) {
+// ------------------------------------------------------------------------------------------
+// Blocked modified Gram-Schmidt.  Modified Gram-Schmidt takes each coefficient h_k = (w, v_k) from
+// the w that all earlier projections have already been subtracted from, so by itself it needs a
+// global reduction per basis vector.  Within a block of vectors the same coefficients follow from
+// the inner products with the block's first w and the block's Gram matrix:
+//   h_k = (w, v_k) - sum_{i in block, i < k} (v_k, v_i) h_i,
+// a forward substitution with the unit lower triangle of V^T V (the low-synchronisation form of
+// modified Gram-Schmidt of Swirydowicz, Langou, Ananthan, Yang and Thomas, 2021, whose loss of
+// orthogonality is that of modified Gram-Schmidt).  The Gram entries are of the size of the loss
+// of orthogonality; v_j's row is taken at step j, in the same sweep as (w, v_i), and kept.  One
+// reduction per block of st.gs_block vectors replaces one per vector.
+//
+// Two block sizes (gs_block_size): a whole restart cycle of up to kGsMaxBlock vectors in one
+// block costs half as many multiply-adds again (every (v_j, v_i) of the cycle), which short vectors
+// do not notice; long vectors, bound by the FP64 pipe, take blocks of kGsGroup (batches) or
+// kGsLong (the cooperative kernel).
+// ------------------------------------------------------------------------------------------
+template <int W>
+__device__ __forceinline__ void load_w(const double* p, double (&x)[W]) {
+    if constexpr (W == 2) {
+        const double2 t = *reinterpret_cast<const double2*>(p);
+        x[0] = t.x;
+        x[1] = t.y;
+    } else {
+        x[0] = p[0];
+    }
+}
+template <int W>
+__device__ __forceinline__ void store_w(double* p, const double (&x)[W]) {
+    if constexpr (W == 2)
+        *reinterpret_cast<double2*>(p) = make_double2(x[0], x[1]);
+    else
+        p[0] = x[0];
+}
+
+// One sweep over the elements [e0, e1) of this CTA (W per thread and iteration):
+//   w -= sum_{i < np} hp[i] vp_i   (vp = the vectors from slot prev on; np = 0: w is left alone)
+//   acc[d] += (w, v_{nxt + d}), d < nn <= kGsGroup
+//   acc[kGsGroup + d] += (v_j, v_{nxt + d}), d < ng   (v_j at slot jslot)
+//   ww += (w, w) when NORM
+template <int W, bool NORM>
+__device__ __forceinline__ void gs_sweep(const SysTab& st, long long e0, long long e1, int prev, int np,
+                                         const double* hp, int nxt, int nn, int ng, int jslot, double (&acc)[16],
+                                         double& ww) {
+    double* w = vec(st, VW);
+    const double* vp = vec(st, prev);
+    const double* vn = vec(st, nxt);
+    const double* vj = vec(st, jslot);
+    const long long n = st.n3p;
+    constexpr int kL = W == 2 ? 4 : kGsGroup;  // vectors loaded together (registers)
+#pragma unroll 1
+    for (long long e = e0 + W * threadIdx.x; e < e1; e += W * VEC_THREADS) {
+        double x[W], y[W];
+        load_w<W>(w + e, x);
+        if (ng > 0) load_w<W>(vj + e, y);
+#pragma unroll 1
+        for (int i0 = 0; i0 < np; i0 += kL) {
+            double c[kL][W];
+#pragma unroll
+            for (int d = 0; d < kL; d++)
+                if (i0 + d < np) load_w<W>(vp + (i0 + d) * n + e, c[d]);
+#pragma unroll
+            for (int d = 0; d < kL; d++)
+                if (i0 + d < np) {
+                    const double h = hp[i0 + d];
+#pragma unroll
+                    for (int u = 0; u < W; u++) x[u] = fma(-h, c[d][u], x[u]);
+                }
+        }
+        if (np > 0) store_w<W>(w + e, x);
+#pragma unroll
+        for (int d0 = 0; d0 < kGsGroup; d0 += kL) {
+            if (d0 >= nn) break;
+            double b[kL][W];
+#pragma unroll
+            for (int d = 0; d < kL; d++)
+                if (d0 + d < nn) load_w<W>(vn + (d0 + d) * n + e, b[d]);
+#pragma unroll
+            for (int d = 0; d < kL; d++)
+                if (d0 + d < nn)
+#pragma unroll
+                    for (int u = 0; u < W; u++) acc[d0 + d] = fma(x[u], b[d][u], acc[d0 + d]);
+#pragma unroll
+            for (int d = 0; d < kL; d++)
+                if (d0 + d < ng)
+#pragma unroll
+                    for (int u = 0; u < W; u++)
+                        acc[kGsGroup + d0 + d] = fma(y[u], b[d][u], acc[kGsGroup + d0 + d]);
+        }
+        if constexpr (NORM)
+#pragma unroll
+            for (int u = 0; u < W; u++) ww = fma(x[u], x[u], ww);
+    }
+}
+
+// The CTA's sums of N (4, 8 or 16) values per thread: value q valid in thread q < N.  Within a warp the
+// values are halved as the lanes are (N adds and one more per spare lane bit, against 5 N for a
+// shuffle tree per value: an FP64 add holds a sub-partition's FP64 unit for ~64 cycles); the eight
+// warps' results are added in index order.  All threads call it; sm holds 8 * 16 doubles.
+template <int N>
+__device__ __forceinline__ double cta_sums(double (&v)[16], double* sm) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int c = N, o = 16;
+#pragma unroll
+    for (int step = 0; step < 4; step++) {
+        if (c == 1) break;
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < N / 2; i++)
+            if (i < c / 2) {
+                const double keep = up ? v[i + c / 2] : v[i], send = up ? v[i] : v[i + c / 2];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        c >>= 1;
+        o >>= 1;
+    }
+    for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    constexpr int kRep = 32 / N;  // lanes that hold the same value
+    __syncthreads();
+    if (lane % kRep == 0) sm[16 * warp + lane / kRep] = v[0];
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x < N) {
+#pragma unroll
+        for (int k = 0; k < VEC_THREADS / 32; k++) t += sm[16 * k + threadIdx.x];
+    }
+    return t;
+}
+
+// Sums of a block's values over its nparts partials, into tot[]: values 0 .. nd - 1 (the dots) and
+// nd .. nd + ng - 1 (the Gram row, from row bs on) and, last, (w, w) (row 2 bs) when ww.  Value q's
+// partials are at part[row(q) * rs + k * ks].  A power-of-two group of lanes per value.
+__device__ __forceinline__ void gs_totals(const double* part, long long rs, long long ks, int nparts, int nd, int ng, bool ww,
+                                          int bs, double* tot) {
+    const int nv = nd + ng + (ww ? 1 : 0);
+    const int tpv = nv <= 8 ? 32 : nv <= 16 ? 16 : nv <= 32 ? 8 : 4;
+    const int per = VEC_THREADS / tpv, sub = threadIdx.x & (tpv - 1);
+    for (int q0 = 0; q0 < nv; q0 += per) {
+        const int q = q0 + (int)threadIdx.x / tpv;
+        double a = 0.0;
+        if (q < nv) {
+            const double* p = part + (q < nd ? q : q < nd + ng ? bs + q - nd : 2 * bs) * rs;
+            int k = sub;
+            for (; k + 3 * tpv < nparts; k += 4 * tpv) {
+                const double l0 = __ldcg(p + k * ks), l1 = __ldcg(p + (k + tpv) * ks), l2 = __ldcg(p + (k + 2 * tpv) * ks),
+                             l3 = __ldcg(p + (k + 3 * tpv) * ks);
+                a += (l0 + l1) + (l2 + l3);
+            }
+            for (; k < nparts; k += tpv) a += __ldcg(p + k * ks);
+        }
+        for (int o = tpv >> 1; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (sub == 0 && q < nv) tot[q] = a;
+    }
+}
+
+// h_lo .. h_{hi-1} of a block from its dots tot[0 ..] (forward substitution with the Gram rows; the
+// last block's last vector is v_j, whose row follows the dots in tot).  gram: the kept rows
+// (kGsMaxBlock per vector, entry i - lo), from row lo on.  Warp 0 of the CTA; h into hs[0 ..].
+__device__ __forceinline__ void gs_substitute(const double* tot, int nd, int ng, const double* gram, double* hs) {
+    const int lane = threadIdx.x & 31;
+    double c = lane < nd ? tot[lane] : 0.0;
+    const double* row = ng > 0 && lane == nd - 1 ? tot + nd : gram + (long long)lane * kGsMaxBlock;
+    for (int k = 0; k + 1 < nd; k++) {
+        const double h = __shfl_sync(0xffffffffu, c, k);
+        if (lane > k && lane < nd) c = fma(-row[k], h, c);
+    }
+    if (lane < nd) hs[lane] = c;
+}
+
+// Pass b of a step of the batched path: subtract block b - 1's projections, then block b's
+// coefficients (b < number of blocks) or ||w||; pass 0 also gives ||w|| before orthogonalisation.
+// Restart/init systems compute beta = ||r|| at pass 0.  The last chunk of a system to arrive adds
+// the chunks' partials up.
+__global__ void __launch_bounds__(VEC_THREADS, 2) k_mgs(const SysTab* __restrict__ tab, const VecItem* __restrict__ items,
+                                                        int b) {
     const VecItem it = items[blockIdx.x];
     const SysTab& st = tab[it.sys];
     if (st.krylov != 0) return;
     const int ph = st.ctl[C_PHASE];
-    const long long e0 = (long long)it.chunk * VEC_CHUNK;
     const ScalLayout SL = ScalLayout::make(st.m);
-    double s0 = 0.0, s1 = 0.0;
+    const long long e0 = (long long)it.chunk * st.vchunk, e1 = e0 + st.vchunk;
     if (ph == PH_ARNOLDI) {
-        const int j = st.ctl[C_J];
-        if (k > j + 1) return;
-        double* w = vec(st, VW);
-        if (k >= 1) {
-            const double h = st.scal[SL.H + (k - 1) * st.m + j];
-            const double* v = vec(st, VV0 + k - 1);
-            for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) w[e0 + i] -= h * v[e0 + i];
-        }
-        if (k <= j) {
-            const double* v = vec(st, VV0 + k);
-            for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
-                const double a = w[e0 + i];
-                s0 += a * v[e0 + i];
-                s1 += a * a;
+        __shared__ double hp[kGsMaxBlock], sm[8 * 16], tot[2 * kGsMaxBlock + 1], hs[kGsMaxBlock];
+        __shared__ bool last;
+        const int j = st.ctl[C_J], bs = st.gs_block, m = st.m;
+        const int lo = b * bs, plo = lo - bs;
+        if (plo > j) return;
+        const int np = b > 0 ? min(bs, j + 1 - plo) : 0;
+        const int nd = max(0, min(bs, j + 1 - lo));
+        const bool fin = nd == 0, lastb = lo + nd == j + 1;
+        const int ngram = !fin && lastb ? nd - 1 : 0;
+        if ((int)threadIdx.x < np) hp[threadIdx.x] = st.scal[SL.H + (plo + threadIdx.x) * m + j];
+        __syncthreads();
+        const int rows = 2 * bs + 1;
+        double* part = st.partial + (long long)it.chunk * rows;
+        for (int g0 = 0; g0 < max(1, nd); g0 += kGsGroup) {
+            double acc[16], ww = 0.0;
+#pragma unroll
+            for (int q = 0; q < 16; q++) acc[q] = 0.0;
+            const int nn = max(0, min(kGsGroup, nd - g0)), ng = max(0, min(kGsGroup, ngram - g0));
+            const int p = g0 == 0 ? np : 0;
+            if (g0 == 0 && (b == 0 || fin))
+                gs_sweep<2, true>(st, e0, e1, VV0 + max(0, plo), p, hp, VV0 + lo, nn, ng, VV0 + j, acc, ww);
+            else
+                gs_sweep<2, false>(st, e0, e1, VV0 + max(0, plo), p, hp, VV0 + lo + g0, nn, ng, VV0 + j, acc, ww);
+            if (!fin) {
+                if (ng > 0) {
+                    const double t = cta_sums<16>(acc, sm);
+                    if ((int)threadIdx.x < nn) part[g0 + threadIdx.x] = t;
+                    if ((int)threadIdx.x >= kGsGroup && (int)threadIdx.x < kGsGroup + ng)
+                        part[bs + g0 + threadIdx.x - kGsGroup] = t;
+                } else {
+                    const double t = cta_sums<8>(acc, sm);
+                    if ((int)threadIdx.x < nn) part[g0 + threadIdx.x] = t;
+                }
             }
-        } else {
-            for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
-                const double a = w[e0 + i];
-                s0 += a * a;
+            if (g0 == 0 && (b == 0 || fin)) {
+                block_sum1(ww);
+                if (threadIdx.x == 0) part[2 * bs] = ww;
             }
         }
-        if (!finish_reduction(st, it.chunk, s0, s1)) return;
+        __syncthreads();
         if (threadIdx.x == 0) {
-            if (k <= j) {
-                st.scal[SL.H + k * st.m + j] = s0;
-                if (k == 0) st.scal[SL.w0] = sqrt(s1);
-            } else {
-                const double hn = sqrt(s0);
+            __threadfence();
+            last = atomicAdd(&st.ctl[C_CNT_RED], 1) == st.nchunk - 1;
+        }
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (threadIdx.x == 0) st.ctl[C_CNT_RED] = 0;
+        gs_totals(st.partial, 1, rows, st.nchunk, nd, ngram, b == 0 || fin, bs, tot);
+        __syncthreads();
+        double* gram = st.scal + SL.gram;
+        if (fin) {
+            if (threadIdx.x == 0) {
+                const double hn = sqrt(tot[0]);
                 st.scal[SL.hn] = hn;
-                st.scal[SL.H + (j + 1) * st.m + j] = hn;
+                st.scal[SL.H + (j + 1) * m + j] = hn;
             }
+            return;
+        }
+        if (threadIdx.x < 32) {
+            gs_substitute(tot, nd, ngram, gram + (long long)lo * kGsMaxBlock, hs);
+            const int t = threadIdx.x;
+            if (t < nd) st.scal[SL.H + (lo + t) * m + j] = hs[t];
+            if (t < ngram) gram[(long long)j * kGsMaxBlock + t] = tot[nd + t];
+            if (t == 0 && b == 0) st.scal[SL.w0] = sqrt(tot[nd + ngram]);
         }
     } else if (ph == PH_RESTART || ph == PH_INIT) {
-        if (k != 0) return;
+        if (b != 0) return;
         const double* r = vec(st, VR);
-        for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
-            const double a = r[e0 + i];
-            s0 += a * a;
-        }
+        double s0 = 0.0, s1 = 0.0;
+        for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) s0 = fma(r[e0 + i], r[e0 + i], s0);
         if (!finish_reduction(st, it.chunk, s0, s1)) return;
         if (threadIdx.x == 0) st.scal[SL.beta] = sqrt(s0);
     }
@@ -228,54 +443,93 @@ __device__ void set_slots(const SysTab& st, int ph, int j) {
     }
 }
 
-// Givens rotation of column j and the GMRES state machine of one system (one thread).
+// Givens rotation of column j and the GMRES state machine of one system, by one warp (all lanes
+// call it with the same arguments).  Every FP64 operation takes ~85 cycles here and every global
+// load more, so the operands are loaded by the lanes together and only the recurrences run in order:
+// one multiply-add per earlier rotation, and in the back substitution a division and a multiply-add
+// per column.
 __device__ void step_state(const SysTab& st, int ph) {
     const ScalLayout SL = ScalLayout::make(st.m);
-    const int m = st.m;
+    const int m = st.m, lane = threadIdx.x & 31;
+    constexpr unsigned kAll = 0xffffffffu;
     int* c = st.ctl;
     double* s = st.scal;
     double* H = s + SL.H;
     if (ph == PH_ARNOLDI) {
-        const int j = c[C_J];
-        for (int k = 0; k < j; k++) {
-            const double a = H[k * m + j], b = H[(k + 1) * m + j];
-            H[k * m + j] = s[SL.cs + k] * a + s[SL.sn + k] * b;
-            H[(k + 1) * m + j] = -s[SL.sn + k] * a + s[SL.cs + k] * b;
+        const int j = c[C_J], iters = c[C_ITERS] + 1, maxit = c[C_MAXIT];
+        const double hn = s[SL.hn], w0 = s[SL.w0], tol = s[SL.tol], bnorm = s[SL.bnorm], gj = s[SL.g + j];
+        // H[k], H[k+1] <- rotation k of them: t is the running H[k]
+        double t = H[j];
+        for (int k0 = 0; k0 < j; k0 += 32) {
+            const int k = k0 + lane;
+            double ck = 1.0, sk = 0.0, hk = 0.0, tk = 0.0;
+            if (k < j) {
+                ck = s[SL.cs + k];
+                sk = s[SL.sn + k];
+                hk = H[(k + 1) * m + j];
+            }
+            const double up = ck * hk;
+            const int nk = min(32, j - k0);
+            for (int i = 0; i < nk; i++) {
+                if (lane == i) tk = t;
+                t = fma(-__shfl_sync(kAll, sk, i), t, __shfl_sync(kAll, up, i));
+            }
+            if (k < j) H[k * m + j] = fma(ck, tk, sk * hk);
         }
-        const double a = H[j * m + j], b = H[(j + 1) * m + j];
-        const double rr = hypot(a, b);
+        const double b = hn, rr = hypot(t, b);  // (t, b) = H[j], H[j+1] of this column
         double cs = 1.0, sn = 0.0;
         if (rr != 0.0) {
-            cs = a / rr;
+            cs = t / rr;
             sn = b / rr;
         }
-        s[SL.cs + j] = cs;
-        s[SL.sn + j] = sn;
-        H[j * m + j] = cs * a + sn * b;
-        H[(j + 1) * m + j] = 0.0;
-        const double gj = s[SL.g + j];
-        s[SL.g + j + 1] = -sn * gj;
-        s[SL.g + j] = cs * gj;
-        c[C_ITERS] += 1;
-        const bool breakdown = s[SL.hn] <= 1e-14 * s[SL.w0];
-        if (breakdown) c[C_BREAKDOWN] = 1;
-        const bool small = fabs(s[SL.g + j + 1]) <= s[SL.tol] * s[SL.bnorm];
-        if (small || breakdown || c[C_ITERS] >= c[C_MAXIT] || j + 1 == m) {
-            const int jend = j + 1;
-            c[C_JEND] = jend;
-            for (int k = jend - 1; k >= 0; k--) {
-                double acc = s[SL.g + k];
-                for (int l = k + 1; l < jend; l++) acc -= H[k * m + l] * s[SL.y + l];
-                s[SL.y + k] = acc / H[k * m + k];
+        const double gn = -sn * gj;
+        const bool breakdown = hn <= 1e-14 * w0;
+        const bool small = fabs(gn) <= tol * bnorm;
+        const bool stop = small || breakdown || iters >= maxit || j + 1 == m;
+        __syncwarp();
+        if (lane == 0) {
+            s[SL.cs + j] = cs;
+            s[SL.sn + j] = sn;
+            H[j * m + j] = cs * t + sn * b;
+            H[(j + 1) * m + j] = 0.0;
+            s[SL.g + j + 1] = gn;
+            s[SL.g + j] = cs * gj;
+            c[C_ITERS] = iters;
+            if (breakdown) c[C_BREAKDOWN] = 1;
+            if (stop) {
+                c[C_JEND] = j + 1;
+                c[C_PHASE] = PH_RESTART;
+                set_slots(st, PH_RESTART, 0);
+            } else {
+                c[C_J] = j + 1;
+                set_slots(st, PH_ARNOLDI, j + 1);
             }
-            c[C_PHASE] = PH_RESTART;
-            set_slots(st, PH_RESTART, 0);
-        } else {
-            c[C_J] = j + 1;
-            set_slots(st, PH_ARNOLDI, j + 1);
+        }
+        __syncwarp();
+        if (stop) {  // y = H^{-1} g, last column first; lane k holds y_k of each 32 rows
+            const int jend = j + 1;
+            for (int r0 = (jend - 1) / 32 * 32; r0 >= 0; r0 -= 32) {
+                const int r = r0 + lane, nr = min(32, jend - r0);
+                double acc = 0.0, d = 1.0;
+                if (r < jend) {
+                    acc = s[SL.g + r];
+                    d = H[r * m + r];
+                    for (int l = jend - 1; l >= r0 + 32; l--) acc = fma(-H[r * m + l], s[SL.y + l], acc);
+                }
+                for (int k = nr - 1; k >= 0; k--) {
+                    const double yk = __shfl_sync(kAll, acc / d, k);
+                    const double h = r < r0 + k ? H[r * m + r0 + k] : 0.0;
+                    if (lane == k) acc = yk;
+                    else if (lane < k) acc = fma(-h, yk, acc);
+                    if (lane == k) d = 1.0;
+                }
+                if (r < jend) s[SL.y + r] = acc;
+                __syncwarp();
+            }
         }
         return;
     }
+    if (lane != 0) return;
     const double beta = s[SL.beta];
     if (ph == PH_INIT) {
         s[SL.bnorm] = beta;
@@ -318,7 +572,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_finish(const SysTab* __restrict
     const int ph = st.ctl[C_PHASE];
     if (ph == PH_DONE || st.krylov != 0) return;
     const ScalLayout SL = ScalLayout::make(st.m);
-    const long long e0 = (long long)it.chunk * VEC_CHUNK;
+    const long long e0 = (long long)it.chunk * st.vchunk;
     if (ph == PH_ARNOLDI) {
         const int j = st.ctl[C_J];
         const double hn = st.scal[SL.hn];
@@ -326,7 +580,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_finish(const SysTab* __restrict
             const double inv = 1.0 / hn;
             const double* w = vec(st, VW);
             double* v = vec(st, VV0 + j + 1);
-            for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) v[e0 + i] = w[e0 + i] * inv;
+            for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) v[e0 + i] = w[e0 + i] * inv;
         }
     } else {
         const double beta = st.scal[SL.beta];
@@ -334,7 +588,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_finish(const SysTab* __restrict
             const double inv = 1.0 / beta;
             const double* r = vec(st, VR);
             double* v = vec(st, VV0);
-            for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) v[e0 + i] = r[e0 + i] * inv;
+            for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) v[e0 + i] = r[e0 + i] * inv;
         }
     }
     __shared__ bool last;
@@ -344,9 +598,9 @@ __global__ void __launch_bounds__(VEC_THREADS) k_finish(const SysTab* __restrict
         last = atomicAdd(&st.ctl[C_CNT_FIN], 1) == st.nchunk - 1;
     }
     __syncthreads();
-    if (!last || threadIdx.x != 0) return;
+    if (!last || threadIdx.x >= 32) return;
     __threadfence();
-    st.ctl[C_CNT_FIN] = 0;
+    if (threadIdx.x == 0) st.ctl[C_CNT_FIN] = 0;
     step_state(st, ph);
 }
 
@@ -424,7 +678,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_om(const SysTab* __restrict__ t
     const SysTab& st = tab[it.sys];
     if (st.krylov != 1) return;
     const int ph = st.ctl[C_PHASE];
-    const long long e0 = (long long)it.chunk * VEC_CHUNK;
+    const long long e0 = (long long)it.chunk * st.vchunk;
     const ScalLayout SL = ScalLayout::make(st.m);
     double s0 = 0.0, s1 = 0.0;
     if (ph == PH_OM) {
@@ -438,17 +692,17 @@ __global__ void __launch_bounds__(VEC_THREADS) k_om(const SysTab* __restrict__ t
             const double beta = st.scal[SL.om_beta + l - 1];
             const double* po = vec(st, om_p(st, os));
             const double* qo = vec(st, om_q(st, os));
-            for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
+            for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
                 p[e0 + i] -= beta * po[e0 + i];
                 q[e0 + i] -= beta * qo[e0 + i];
             }
         }
         if (l < stored) {
             const double* qo = vec(st, om_q(st, (slot - l - 1 + K1) % K1));
-            for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) s0 += q[e0 + i] * qo[e0 + i];
+            for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) s0 += q[e0 + i] * qo[e0 + i];
         } else {
             const double* r = vec(st, VR);
-            for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
+            for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
                 const double a = q[e0 + i];
                 s0 += a * a;
                 s1 += r[e0 + i] * a;
@@ -467,7 +721,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_om(const SysTab* __restrict__ t
     } else if (ph == PH_INIT || ph == PH_OM_FINAL) {
         if (l != 0) return;
         const double* r = vec(st, ph == PH_INIT ? VR : VW);
-        for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
+        for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
             const double a = r[e0 + i];
             s0 += a * a;
         }
@@ -485,7 +739,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_om_update(const SysTab* __restr
     const ScalLayout SL = ScalLayout::make(st.m);
     const int slot = st.ctl[C_OM_SLOT];
     const bool dead = st.scal[SL.om_qq + slot] == 0.0;
-    const long long e0 = (long long)it.chunk * VEC_CHUNK;
+    const long long e0 = (long long)it.chunk * st.vchunk;
     double s0 = 0.0, s1 = 0.0;
     if (!dead) {
         const double alpha = st.scal[SL.om_alpha];
@@ -493,7 +747,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_om_update(const SysTab* __restr
         const double* q = vec(st, om_q(st, slot));
         double* x = vec(st, VX);
         double* r = vec(st, VR);
-        for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
+        for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
             x[e0 + i] += alpha * p[e0 + i];
             const double a = r[e0 + i] - alpha * q[e0 + i];
             r[e0 + i] = a;
@@ -510,42 +764,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_om_update(const SysTab* __restr
     }
 }
 
-// The whole orthogonalisation of one step of one system in one cooperative launch: modified
-// Gram-Schmidt with one grid-wide barrier per projection instead of one launch.  Each CTA keeps a
-// single partial per projection (grid-stride over the elements), and every CTA reduces the G
-// partials in the same fixed order, so the result is deterministic for a given grid size.
-// w stays in L2 between projections, so each basis vector is streamed from HBM about once.
-__device__ __forceinline__ void grid_total(const double* part, int G, double& s0, double& s1) {
-    double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < G; i += blockDim.x) {
-        a += __ldcg(&part[2 * i]);
-        b += __ldcg(&part[2 * i + 1]);
-    }
-    block_sum2(a, b);
-    __shared__ double bc[2];
-    if (threadIdx.x == 0) {
-        bc[0] = a;
-        bc[1] = b;
-    }
-    __syncthreads();
-    s0 = bc[0];
-    s1 = bc[1];
-    __syncthreads();
-}
-
-// single-value forms of block_sum2 / grid_total (the same summation order for that value)
-__device__ __forceinline__ void block_sum1(double& a) {
-    __shared__ double s0[VEC_THREADS];
-    s0[threadIdx.x] = a;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double x = 0.0;
-        for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) x += s0[i];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        a = x;
-    }
-    __syncthreads();
-}
+// sum of one partial per CTA, in every CTA in the same order
 __device__ __forceinline__ double grid_total1(const double* part, int G) {
     double a = 0.0;
     for (int i = threadIdx.x; i < G; i += blockDim.x) a += __ldcg(&part[i]);
@@ -653,7 +872,7 @@ __device__ void cgs_project(const SysTab& st, double* part2, cooperative_groups:
         if (q == 0 && i < nv) htot[i] = a;
     }
     __syncthreads();
-    w0 = sqrt(htot[j + 1]);
+    w0 = htot[j + 1];
     double p[kU];
 #pragma unroll
     for (int u = 0; u < kU; u++) p[u] = 0.0;
@@ -705,161 +924,357 @@ __device__ void cgs_project(const SysTab& st, double* part2, cooperative_groups:
         for (int i = 0; i <= j; i++) st.scal[SL.H + i * m + j] = htot[i];
 }
 
-__global__ void __launch_bounds__(VEC_THREADS, 2) k_ortho_coop(const SysTab* __restrict__ tab, double* __restrict__ part2) {
-    constexpr int kU = 4;
+// ------------------------------------------------------------------------------------------
+// The whole orthogonalisation of one step of one system in one cooperative launch, every CTA on
+// its slice [e0, e1) of the vectors: one grid barrier per block of basis vectors and one for the norm.
+// ------------------------------------------------------------------------------------------
+struct GsBlock {  // the vectors v_lo .. v_{lo + nd - 1}; ngram: Gram entries taken with them
+    int lo, nd, ngram;
+};
+__device__ __forceinline__ GsBlock gs_block_at(int lo, int bs, int j) {
+    const int nd = min(bs, j + 1 - lo);
+    return GsBlock{lo, nd, lo + nd == j + 1 ? nd - 1 : 0};
+}
+
+struct GsShared {
+    double sm[8 * 16], tot[2 * kGsMaxBlock + 1], hs[kGsMaxBlock];
+    double gram[kGsMaxBlock * kGsMaxBlock];
+};
+
+// A group's CTA sums into the partials of its block: row q of the block's dots, Gram row and (row
+// 2 bs) w's norm, one value per CTA.  GP: vectors per group (dots acc[0 ..], Gram entries acc[GP ..])
+template <int GP>
+__device__ __forceinline__ void gs_store_partials(GsShared& S, double (&acc)[16], double ww, bool norm, double* part, int bs,
+                                                  int g0, int nn, int ng) {
+    const int G = gridDim.x, q = threadIdx.x;
+    const double t = ng > 0 ? cta_sums<2 * GP>(acc, S.sm) : cta_sums<GP>(acc, S.sm);
+    if (q < nn) part[(long long)(g0 + q) * G + blockIdx.x] = t;
+    if (q >= GP && q < GP + ng) part[(long long)(bs + g0 + q - GP) * G + blockIdx.x] = t;
+    if (norm) {
+        block_sum1(ww);
+        if (q == 0) part[(long long)2 * bs * G + blockIdx.x] = ww;
+    }
+}
+
+// The coefficients of a block, in S.hs of every CTA, from the partials (this is the grid barrier);
+// CTA 0 keeps them and v_j's Gram row.  Each CTA adds the CTAs' partials up itself, in the same
+// order.  Where that is many values from many CTAs (a whole cycle in one block), CTA q adds value q up
+// and a second barrier hands it round: 152 partials of 60 values in every CTA would be ~40
+// dependent FP64 adds of ~128 cycles.
+__device__ __forceinline__ void gs_coefficients(const SysTab& st, GsShared& S, cooperative_groups::grid_group& grid,
+                                                double* part, const GsBlock& B, int bs, int j, const ScalLayout& SL,
+                                                double& w0) {
+    const int G = gridDim.x, m = st.m;
+    double* gram = st.scal + SL.gram;
+    // the kept Gram rows, loaded while the barrier is waited for
+    for (int t = threadIdx.x; t < B.nd * kGsMaxBlock; t += blockDim.x)
+        S.gram[t] = t / kGsMaxBlock + B.lo < j ? gram[(long long)B.lo * kGsMaxBlock + t] : 0.0;
+    grid.sync();
+    const int nv = B.nd + B.ngram + (B.lo == 0 ? 1 : 0);
+    if (nv > 16 && G > 32) {
+        double* all = part + (long long)(2 * bs + 1) * G;
+        const int q = blockIdx.x + G * (threadIdx.x >> 5);
+        if (q < nv) {
+            const int lane = threadIdx.x & 31;
+            const double* p = part + (long long)(q < B.nd ? q : q < B.nd + B.ngram ? bs + q - B.nd : 2 * bs) * G;
+            double a = 0.0;
+            for (int k = lane; k < G; k += 32) a += __ldcg(p + k);
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (lane == 0) all[q] = a;
+        }
+        grid.sync();
+        if ((int)threadIdx.x < nv) S.tot[threadIdx.x] = __ldcg(all + threadIdx.x);
+    } else {
+        gs_totals(part, G, 1, G, B.nd, B.ngram, B.lo == 0, bs, S.tot);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) gs_substitute(S.tot, B.nd, B.ngram, S.gram, S.hs);
+    if (B.lo == 0) w0 = S.tot[B.nd + B.ngram];
+    __syncthreads();
+    if (blockIdx.x == 0) {
+        const int t = threadIdx.x;
+        if (t < B.nd) st.scal[SL.H + (B.lo + t) * m + j] = S.hs[t];
+        if (t < B.ngram) gram[(long long)j * kGsMaxBlock + t] = S.tot[B.nd + t];
+    }
+}
+
+// doubles of one of the two sets of partials (a block's are read while the next block's are written)
+__device__ __forceinline__ long long gs_part_set(int bs) { return (long long)(2 * bs + 1) * gridDim.x + 2 * kGsMaxBlock + 1; }
+
+// a sum over the CTAs, in every CTA (the other grid barrier)
+__device__ __forceinline__ double gs_grid_sum(double s, double* part, cooperative_groups::grid_group& grid) {
+    block_sum1(s);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    grid.sync();
+    return grid_total1(part, gridDim.x);
+}
+
+// End of a step: v_{j+1} = w / h_{j+1,j}, or v_0 = r / beta (scale: that norm).  The state machine takes a few
+// microseconds of dependent scalar operations: warp 0 of CTA 0 runs it while the other warps scale.
+template <int W>
+__device__ __forceinline__ void ortho_finish(const SysTab& st, int ph, int j, const ScalLayout& SL, long long e0, long long e1,
+                                             double w0, double scale) {
+    constexpr int kU = 8;
+    const double* src = vec(st, ph == PH_ARNOLDI ? VW : VR);
+    const int dst = ph == PH_ARNOLDI ? VV0 + j + 1 : VV0;
+    int first = threadIdx.x, step = VEC_THREADS;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < 32) {
+            if (threadIdx.x == 0) {
+                if (ph == PH_ARNOLDI) {
+                    st.scal[SL.w0] = sqrt(w0);
+                    st.scal[SL.hn] = scale;
+                    st.scal[SL.H + (j + 1) * st.m + j] = scale;
+                } else {
+                    st.scal[SL.beta] = scale;
+                }
+            }
+            __syncwarp();
+            step_state(st, ph);
+            return;
+        }
+        first -= 32;
+        step -= 32;
+    }
+    if (scale > 0.0) {
+        const double inv = 1.0 / scale;
+        double* v = vec(st, dst);
+        for (long long e = e0 + W * first; e < e1; e += kU * W * step) {
+            double a[kU][W];
+#pragma unroll
+            for (int u = 0; u < kU; u++)
+                if (e + u * W * step < e1) load_w<W>(src + e + u * W * step, a[u]);
+#pragma unroll
+            for (int u = 0; u < kU; u++)
+                if (e + u * W * step < e1) {
+#pragma unroll
+                    for (int k = 0; k < W; k++) a[u][k] *= inv;
+                    store_w<W>(v + e + u * W * step, a[u]);
+                }
+        }
+    }
+}
+
+// this CTA's slice of the vectors: whole 64-element pieces (the vectors are zero beyond n3)
+__device__ __forceinline__ void gs_slice(const SysTab& st, long long& e0, long long& e1) {
+    const long long n = (st.n3 + 63) & ~63;
+    const long long len = ((n + gridDim.x - 1) / gridDim.x + 63) & ~63LL;
+    e0 = min(n, len * blockIdx.x);
+    e1 = min(n, e0 + len);
+}
+
+// ||r|| of an initial or restarting system
+__device__ __forceinline__ double ortho_beta(const SysTab& st, double* part2, cooperative_groups::grid_group& grid,
+                                             long long e0, long long e1) {
+    const double* r = vec(st, VR);
+    constexpr int kU = 8;
+    double s0 = 0.0;
+    for (long long e = e0 + threadIdx.x; e < e1; e += kU * VEC_THREADS) {
+        double a[kU];
+#pragma unroll
+        for (int u = 0; u < kU; u++) a[u] = e + u * VEC_THREADS < e1 ? r[e + u * VEC_THREADS] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kU; u++) s0 = fma(a[u], a[u], s0);
+    }
+    return sqrt(gs_grid_sum(s0, part2, grid));
+}
+
+// Short vectors (st.gs_block = kGsMaxBlock: up to 862 elements per SM): a handful of elements per thread, so
+// what counts is the number of barriers and of dependent FP64 operations.
+__global__ void __launch_bounds__(VEC_THREADS, 1) k_ortho_short(const SysTab* __restrict__ tab, double* __restrict__ part2) {
+    namespace cg = cooperative_groups;
+    cg::grid_group grid = cg::this_grid();
+    __shared__ GsShared S;
+    const SysTab& st = tab[0];
+    const int ph = st.ctl[C_PHASE];
+    if (ph == PH_DONE) return;
+    const ScalLayout SL = ScalLayout::make(st.m);
+    long long e0, e1;
+    gs_slice(st, e0, e1);
+    if (ph != PH_ARNOLDI) {
+        ortho_finish<1>(st, ph, 0, SL, e0, e1, 0.0, ortho_beta(st, part2, grid, e0, e1));
+        return;
+    }
+    const int j = st.ctl[C_J], bs = st.gs_block;
+    double w0 = 0.0, norm = 0.0;
+    int turn = 0;
+    for (int lo = 0; lo <= j; lo += bs, turn ^= 1) {
+        const GsBlock B = gs_block_at(lo, bs, j);
+        double* part = part2 + turn * gs_part_set(bs);
+        for (int g0 = 0; g0 < B.nd; g0 += kGsGroup) {
+            double acc[16], ww = 0.0;
+#pragma unroll
+            for (int q = 0; q < 16; q++) acc[q] = 0.0;
+            const int nn = min(kGsGroup, B.nd - g0), ng = max(0, min(kGsGroup, B.ngram - g0));
+            const bool start = lo == 0 && g0 == 0;
+            if (start)
+                gs_sweep<1, true>(st, e0, e1, VV0, 0, S.hs, VV0, nn, ng, VV0 + j, acc, ww);
+            else
+                gs_sweep<1, false>(st, e0, e1, VV0, 0, S.hs, VV0 + lo + g0, nn, ng, VV0 + j, acc, ww);
+            gs_store_partials<kGsGroup>(S, acc, ww, start, part, bs, g0, nn, ng);
+        }
+        gs_coefficients(st, S, grid, part, B, bs, j, SL, w0);
+        double acc[16];
+        norm = 0.0;
+        gs_sweep<1, true>(st, e0, e1, VV0 + lo, B.nd, S.hs, VV0, 0, 0, VV0, acc, norm);
+    }
+    ortho_finish<1>(st, ph, j, SL, e0, e1, w0, sqrt(gs_grid_sum(norm, part2 + turn * gs_part_set(bs), grid)));
+}
+
+// gs_sweep for blocks of kGsLong vectors, with loads ahead of the arithmetic: the next vectors of an
+// iteration are requested before its subtractions, the previous block's vectors of the next iteration
+// before the products; with vectors on one side only, those of the next iteration.
+template <bool PREV, bool GRAM>
+__device__ __forceinline__ void gs_sweep_pipe(const SysTab& st, long long e0, long long e1, int prev, int np,
+                                              const double* hp, int nxt, int nn, int ng, int jslot, bool norm,
+                                              double (&acc)[16], double& ww) {
+    constexpr int W = 2;
+    const long long n = st.n3p;
+    const long long first = e0 + W * threadIdx.x, step = W * VEC_THREADS;
+    if (first >= e1) return;
+    double* w = vec(st, VW);
+    const double* vp = vec(st, prev);
+    const double* vn = vec(st, nxt);
+    const double* vj = vec(st, jslot);
+    double h[kGsLong], x[W], y[W], b[kGsLong][W], c[kGsLong][W];
+    auto load_group = [&](const double* base, int cnt, long long e, double (&v)[kGsLong][W]) {
+        // no branch around the loads: a vector past the last one reads the last one again (its products
+        // are skipped); q is opaque so that no address register per vector lives across the loop
+        const double* q = base + e;
+        asm volatile("" : "+l"(q));
+#pragma unroll
+        for (int d = 0; d < kGsLong; d++) {
+            load_w<W>(q, v[d]);
+            q += d + 1 < cnt ? n : 0;
+        }
+    };
+    load_w<W>(w + first, x);
+    if (PREV) {
+#pragma unroll
+        for (int d = 0; d < kGsLong; d++) h[d] = d < np ? hp[d] : 0.0;
+        load_group(vp, np, first, c);
+    } else {
+        load_group(vn, nn, first, b);
+        if (GRAM) load_w<W>(vj + first, y);
+    }
+#pragma unroll 1
+    for (long long e = first; e < e1; e += step) {
+        const long long en = e + step < e1 ? e + step : first;  // the last iteration's loads are not used
+        double x1[W], y1[W];
+        if (PREV) {
+            if (nn > 0) {
+                load_group(vn, nn, e, b);
+                if (GRAM) load_w<W>(vj + e, y);
+            } else {
+                load_group(vp, np, en, b);
+            }
+#pragma unroll
+            for (int d = 0; d < kGsLong; d++)
+                if (d < np)
+#pragma unroll
+                    for (int u = 0; u < W; u++) x[u] = fma(-h[d], c[d][u], x[u]);
+            store_w<W>(w + e, x);
+            if (nn > 0) {
+                load_group(vp, np, en, c);
+            } else {
+#pragma unroll
+                for (int d = 0; d < kGsLong; d++)
+#pragma unroll
+                    for (int u = 0; u < W; u++) c[d][u] = b[d][u];
+            }
+        } else {
+            load_group(vn, nn, en, c);
+            if (GRAM) load_w<W>(vj + en, y1);
+        }
+        load_w<W>(w + en, x1);
+#pragma unroll
+        for (int d = 0; d < kGsLong; d++)
+            if (d < nn)
+#pragma unroll
+                for (int u = 0; u < W; u++) acc[d] = fma(x[u], b[d][u], acc[d]);
+        if (GRAM)
+#pragma unroll
+            for (int d = 0; d < kGsLong; d++)
+                if (d < ng)
+#pragma unroll
+                    for (int u = 0; u < W; u++) acc[kGsLong + d] = fma(y[u], b[d][u], acc[kGsLong + d]);
+        if (norm)
+#pragma unroll
+            for (int u = 0; u < W; u++) ww = fma(x[u], x[u], ww);
+#pragma unroll
+        for (int u = 0; u < W; u++) {
+            x[u] = x1[u];
+            if (!PREV) {
+                if (GRAM) y[u] = y1[u];
+#pragma unroll
+                for (int d = 0; d < kGsLong; d++) b[d][u] = c[d][u];
+            }
+        }
+    }
+}
+
+// Long vectors: blocks of kGsLong, two CTAs per SM.  An FP64 multiply-add holds a sub-partition's
+// FP64 unit for 64 cycles, so what matters is that some warp always has its operands: 16 warps per SM
+// with blocks of four (18 operands in registers) do that better than eight warps with blocks of
+// eight, although those sweep w half as often (128x128x64, one solve: 21.6 against 26.9 ms; one reduction per
+// vector: 24.5 ms).
+__global__ void __launch_bounds__(VEC_THREADS, 2) k_ortho_long(const SysTab* __restrict__ tab, double* __restrict__ part2) {
+    namespace cg = cooperative_groups;
+    cg::grid_group grid = cg::this_grid();
+    __shared__ GsShared S;
+    const SysTab& st = tab[0];
+    const int ph = st.ctl[C_PHASE];
+    if (ph == PH_DONE) return;
+    const ScalLayout SL = ScalLayout::make(st.m);
+    long long e0, e1;
+    gs_slice(st, e0, e1);
+    if (ph != PH_ARNOLDI) {
+        ortho_finish<2>(st, ph, 0, SL, e0, e1, 0.0, ortho_beta(st, part2, grid, e0, e1));
+        return;
+    }
+    const int j = st.ctl[C_J], bs = kGsLong;
+    double w0 = 0.0, norm = 0.0;
+    int turn = 0, np = 0;
+    for (int lo = 0; lo <= j; lo += bs, turn ^= 1) {
+        const GsBlock B = gs_block_at(lo, bs, j);
+        double acc[16], ww = 0.0;
+#pragma unroll
+        for (int q = 0; q < 16; q++) acc[q] = 0.0;
+        if (lo == 0 && B.ngram == 0)
+            gs_sweep_pipe<false, false>(st, e0, e1, VV0, 0, S.hs, VV0, B.nd, 0, VV0 + j, true, acc, ww);
+        else if (lo == 0)
+            gs_sweep_pipe<false, true>(st, e0, e1, VV0, 0, S.hs, VV0, B.nd, B.ngram, VV0 + j, true, acc, ww);
+        else if (B.ngram == 0)
+            gs_sweep_pipe<true, false>(st, e0, e1, VV0 + lo - bs, np, S.hs, VV0 + lo, B.nd, 0, VV0 + j, false, acc, ww);
+        else
+            gs_sweep_pipe<true, true>(st, e0, e1, VV0 + lo - bs, np, S.hs, VV0 + lo, B.nd, B.ngram, VV0 + j, false, acc, ww);
+        double* part = part2 + turn * gs_part_set(bs);
+        gs_store_partials<kGsLong>(S, acc, ww, lo == 0, part, bs, 0, B.nd, B.ngram);
+        gs_coefficients(st, S, grid, part, B, bs, j, SL, w0);
+        np = B.nd;
+    }
+    double acc[16];
+    gs_sweep_pipe<true, false>(st, e0, e1, VV0 + j / bs * bs, np, S.hs, VV0, 0, 0, VV0, true, acc, norm);
+    ortho_finish<2>(st, ph, j, SL, e0, e1, w0, sqrt(gs_grid_sum(norm, part2 + turn * gs_part_set(bs), grid)));
+}
+
+__global__ void __launch_bounds__(VEC_THREADS, 2) k_ortho_cgs(const SysTab* __restrict__ tab, double* __restrict__ part2) {
     namespace cg = cooperative_groups;
     cg::grid_group grid = cg::this_grid();
     const SysTab& st = tab[0];
     const int ph = st.ctl[C_PHASE];
     if (ph == PH_DONE) return;
     const ScalLayout SL = ScalLayout::make(st.m);
-    const int m = st.m;
-    const int G = gridDim.x;
-    const long long n = st.n3p;
-    const long long stride = (long long)G * blockDim.x;
-    const long long e_begin = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    double* w = vec(st, VW);
-    if (ph == PH_ARNOLDI) {
-        const int j = st.ctl[C_J];
-        double hprev = 0.0, w0 = 0.0, hn = 0.0;
-        if (st.ortho == 1) {
-            cgs_project(st, part2, grid, j, SL, w0, hn);
-        } else {
-            // Operands of the current group of kU elements; the next group's loads are issued before
-            // the current group is computed.  The first group of pass k + 1 needs nothing from the
-            // barrier that ends pass k (its w is this thread's own result), so its loads are issued
-            // before that barrier.
-            double A[kU], B[kU], C[kU];
-            {
-                const double* v0 = vec(st, VV0);
-    #pragma unroll
-                for (int u = 0; u < kU; u++) {
-                    const long long e = e_begin + u * stride;
-                    A[u] = e < n ? w[e] : 0.0;
-                    B[u] = 0.0;
-                    C[u] = e < n ? v0[e] : 0.0;
-                }
-            }
-            for (int k = 0; k <= j + 1; k++) {
-                double* part = part2 + (size_t)(k & 1) * 2 * G;
-                double s0 = 0.0, s1 = 0.0;
-                // kU partial sums per thread, combined in a fixed order
-                double p0[kU], p1[kU];
-    #pragma unroll
-                for (int u = 0; u < kU; u++) p0[u] = p1[u] = 0.0;
-                const double* vp = k > 0 ? vec(st, VV0 + k - 1) : nullptr;
-                const double* vk = k <= j ? vec(st, VV0 + k) : nullptr;
-                for (long long e0 = e_begin; e0 < n; e0 += kU * stride) {
-                    const long long e1 = e0 + kU * stride;
-                    double An[kU], Bn[kU], Cn[kU];
-    #pragma unroll
-                    for (int u = 0; u < kU; u++) {
-                        const long long e = e1 + u * stride;
-                        const bool in = e < n;
-                        An[u] = in ? w[e] : 0.0;
-                        Bn[u] = in && vp ? vp[e] : 0.0;
-                        Cn[u] = in && vk ? vk[e] : 0.0;
-                    }
-                    if (k == 0) {  // (w, v_0) and (w, w)
-    #pragma unroll
-                        for (int u = 0; u < kU; u++) {
-                            p0[u] = fma(A[u], C[u], p0[u]);
-                            p1[u] = fma(A[u], A[u], p1[u]);
-                        }
-                    } else {  // w -= h_{k-1} v_{k-1}, then (w, v_k), or (w, w) after the last projection
-    #pragma unroll
-                        for (int u = 0; u < kU; u++) {
-                            const long long e = e0 + u * stride;
-                            const double x = fma(-hprev, B[u], A[u]);
-                            if (e < n) w[e] = x;
-                            p0[u] = fma(x, vk ? C[u] : x, p0[u]);
-                        }
-                    }
-    #pragma unroll
-                    for (int u = 0; u < kU; u++) {
-                        A[u] = An[u];
-                        B[u] = Bn[u];
-                        C[u] = Cn[u];
-                    }
-                }
-                if (k <= j) {  // the first group of pass k + 1
-                    const double* vn = k + 1 <= j ? vec(st, VV0 + k + 1) : nullptr;
-    #pragma unroll
-                    for (int u = 0; u < kU; u++) {
-                        const long long e = e_begin + u * stride;
-                        const bool in = e < n;
-                        A[u] = in ? w[e] : 0.0;
-                        B[u] = in ? vk[e] : 0.0;
-                        C[u] = in && vn ? vn[e] : 0.0;
-                    }
-                }
-                s0 = (p0[0] + p0[1]) + (p0[2] + p0[3]);
-                double t0, t1 = 0.0;
-                if (k == 0) {  // (w, v_0) and (w, w)
-                    s1 = (p1[0] + p1[1]) + (p1[2] + p1[3]);
-                    block_sum2(s0, s1);
-                    if (threadIdx.x == 0) {
-                        part[2 * blockIdx.x] = s0;
-                        part[2 * blockIdx.x + 1] = s1;
-                    }
-                    grid.sync();
-                    grid_total(part, G, t0, t1);
-                } else {  // one sum: half the FP64 adds of the two reductions (same order for s0)
-                    block_sum1(s0);
-                    if (threadIdx.x == 0) part[blockIdx.x] = s0;
-                    grid.sync();
-                    t0 = grid_total1(part, G);
-                }
-                if (k <= j) {
-                    hprev = t0;
-                    if (k == 0) w0 = sqrt(t1);
-                    if (blockIdx.x == 0 && threadIdx.x == 0) st.scal[SL.H + k * m + j] = t0;
-                } else {
-                    hn = sqrt(t0);
-                }
-            }
-        }
-        if (hn > 0.0) {
-            const double inv = 1.0 / hn;
-            double* v = vec(st, VV0 + j + 1);
-            for (long long e0 = e_begin; e0 < n; e0 += kU * stride) {
-                double a[kU];
-#pragma unroll
-                for (int u = 0; u < kU; u++) a[u] = e0 + u * stride < n ? w[e0 + u * stride] : 0.0;
-#pragma unroll
-                for (int u = 0; u < kU; u++)
-                    if (e0 + u * stride < n) v[e0 + u * stride] = a[u] * inv;
-            }
-        }
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            st.scal[SL.w0] = w0;
-            st.scal[SL.hn] = hn;
-            st.scal[SL.H + (j + 1) * m + j] = hn;
-            step_state(st, ph);
-        }
-    } else {
-        const double* r = vec(st, VR);
-        double s0 = 0.0, s1 = 0.0;
-        for (long long e = e_begin; e < n; e += stride) s0 = fma(r[e], r[e], s0);
-        block_sum2(s0, s1);
-        if (threadIdx.x == 0) {
-            part2[2 * blockIdx.x] = s0;
-            part2[2 * blockIdx.x + 1] = s1;
-        }
-        grid.sync();
-        double t0, t1;
-        grid_total(part2, G, t0, t1);
-        const double beta = sqrt(t0);
-        if (beta > 0.0) {
-            const double inv = 1.0 / beta;
-            double* v = vec(st, VV0);
-            for (long long e = e_begin; e < n; e += stride) v[e] = r[e] * inv;
-        }
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            st.scal[SL.beta] = beta;
-            step_state(st, ph);
-        }
+    long long e0, e1;
+    gs_slice(st, e0, e1);
+    if (ph != PH_ARNOLDI) {
+        ortho_finish<2>(st, ph, 0, SL, e0, e1, 0.0, ortho_beta(st, part2, grid, e0, e1));
+        return;
     }
+    const int j = st.ctl[C_J];
+    double w0 = 0.0, hn = 0.0;
+    cgs_project(st, part2, grid, j, SL, w0, hn);
+    ortho_finish<2>(st, ph, j, SL, e0, e1, w0, hn);
 }
 
 }  // namespace
@@ -877,20 +1292,32 @@ void launch_prep(const SysTab* tab, const VecItem* items, int nitems, cudaStream
 void launch_post(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st) {
     if (nitems > 0) k_post<<<nitems, VEC_THREADS, 0, st>>>(tab, items);
 }
-void launch_mgs(const SysTab* tab, const VecItem* items, int nitems, int k, cudaStream_t st) {
-    if (nitems > 0) k_mgs<<<nitems, VEC_THREADS, 0, st>>>(tab, items, k);
+void launch_mgs(const SysTab* tab, const VecItem* items, int nitems, int pass, cudaStream_t st) {
+    if (nitems > 0) k_mgs<<<nitems, VEC_THREADS, 0, st>>>(tab, items, pass);
 }
-int ortho_coop_grid(int device) {
+namespace {
+const void* ortho_kernel(int ortho, int n3) {
+    if (ortho == 1) return (const void*)k_ortho_cgs;
+    if (gs_block_size(n3) == kGsMaxBlock) return (const void*)k_ortho_short;
+    return (const void*)k_ortho_long;
+}
+}  // namespace
+
+int ortho_coop_grid(int device, int ortho, int n3) {
     int per_sm = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ortho_coop, VEC_THREADS, 0) != cudaSuccess) return 0;
+    const void* f = ortho_kernel(ortho, n3);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, VEC_THREADS, 0) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-    // two CTAs per SM: enough loads in flight, few partials to reduce and cheap grid barriers
-    return std::min(per_sm, 2) * sms;
+    // two CTAs per SM for their loads in flight; short vectors: one, for fewer partials, with 128
+    // elements per CTA (one warp per SM sub-partition) until the chip is full
+    const bool is_short = f == (const void*)k_ortho_short;
+    const int max_grid = std::min(per_sm, is_short ? 1 : 2) * sms;
+    return is_short ? std::max(1, std::min(max_grid, (n3 + 127) / 128)) : max_grid;
 }
 
-cudaError_t launch_ortho_coop(const SysTab* tab, double* part2, int grid, cudaStream_t st) {
+cudaError_t launch_ortho_coop(const SysTab* tab, double* part2, int grid, int ortho, int n3, cudaStream_t st) {
     void* args[] = {(void*)&tab, (void*)&part2};
-    return cudaLaunchCooperativeKernel((const void*)k_ortho_coop, dim3(grid), dim3(VEC_THREADS), args, 0, st);
+    return cudaLaunchCooperativeKernel(ortho_kernel(ortho, n3), dim3(grid), dim3(VEC_THREADS), args, 0, st);
 }
 
 void launch_om(const SysTab* tab, const VecItem* items, int nitems, int l, cudaStream_t st) {
