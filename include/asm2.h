@@ -260,12 +260,16 @@ int asm_get_stats(asm_handle h, asm_stats* st);
 /* Tuning switches of the kernels (none changes the arithmetic of a fine row; results are bitwise
  * the same, except where ASM_TUNE_CHUNK_KB says otherwise):
  *   ASM_TUNE_APPLY_SMEM  where the apply keeps each subdomain's local vectors.  1 (default):
- *                        all in shared memory (256-thread CTAs) when every subdomain CTA of the
+ *                        all in shared memory with the factor stream laid out by lane (512-thread
+ *                        CTAs; not for FP64 lump rows under narrower fine rows) when the launch is at
+ *                        most two waves of CTAs and every subdomain fits; else all in shared memory
+ *                        (256-thread CTAs) when every subdomain CTA of the
  *                        launch then runs at once; else the lump vector in shared memory and the
  *                        fine-row vector in device memory when that fits; else all in device memory
  *                        (256-thread CTAs).  0: all in device memory; 2: lumps in shared memory;
  *                        3: all in shared memory (2 and 3 fall back to device memory when they do
- *                        not fit);
+ *                        not fit).  The first launch of a handle that leaves the stream by lane
+ *                        uploads the other stream;
  *   ASM_TUNE_COOP_ORTHO  1 (default) runs the Gram-Schmidt step of a single-system solve in one
  *                        cooperative launch, 0 in one launch per block of basis vectors.
  * Errors: INVALID_ARG for an unknown key or value. */

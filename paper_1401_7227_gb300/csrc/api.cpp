@@ -79,6 +79,9 @@ struct DBuf {
 
 }  // namespace
 
+// whether the factor stream by lane is built for a system: a launch of its subdomains alone may take it (lane_slots)
+static bool wants_lanes(const Geom& g, int sms) { return g.n_sub() <= 2LL * sms; }
+
 struct asm_ctx {
     asm_options opt;
     cudaStream_t stream = nullptr;
@@ -105,6 +108,14 @@ struct asm_ctx {
     int n_along = 0;  // slots whose assembly lists are summed by a warp each
     DBuf d_fp;  // factor program arrays (one allocation, see upload_factor_program)
     DBuf d_stream, d_pk_off_f, d_pk_src_f, d_pk_off_c, d_pk_src_c;
+    // the factor stream by lane and its pack lists (packets.h); lanes_ok: every subdomain's chunks and
+    // local vectors fit a CTA's shared memory.  The other stream is then uploaded and packed only for
+    // a handle that is asked for one of its placements (rows_ready: uploaded; rows_packed: holds the current
+    // factors).
+    DBuf d_lanes, d_ln_off_f, d_ln_src_f, d_ln_off_c, d_ln_src_c;
+    long long ln_nf = 0, ln_nc = 0;
+    bool lanes_ok = false, rows_ready = false, rows_packed = false;
+    int lanes_cap = 0, lanes_smem = 0;  // its largest chunk; the largest local vectors and zero row
     DBuf d_lv, d_rlists, d_y, d_corr_cells, d_corr, d_dev_err, d_gsum, d_r32;
     int n_group_items = 0;  // box_items[0 .. n_group_items): the cell-group sums (kind 2)
     int apply_smem = 0;       // shared memory for all local vectors of the largest subdomain (0: none)
@@ -511,6 +522,89 @@ void choose_ring(asm_ctx* h) {
     }
 }
 
+// Ring slots of a launch of nsub subdomains with the stream by lane (0: another placement).  A 512-thread CTA
+// takes an SM's registers in FP64 and half of them in FP32: as many CTAs per SM as the launch needs while
+// each has three slots, then as many slots as fit.
+// The chain of levels of one subdomain is shorter by lane, but fewer CTAs fit an SM than with the local
+// vectors in device memory (four), so launches of more than two waves keep those: 128x128x32 in 256
+// subdomains, 1.7 waves, one apply: 490 against 612 us in FP64, 231 / 245 in FP32, 227 / 231 in FP16; 128x128x64 in
+// 512, 3.4 waves: 1055 / 957, 479 / 367, 485 / 341.
+int lane_slots(const asm_ctx* h, int nsub, int smem, int chunk) {
+    const int sms = std::max(1, h->n_sms), most = h->prec == 0 ? 1 : 2;
+    const auto fits = [&](int sl, int ctas) {
+        const size_t cta = (size_t)smem + apply_ring_bytes(sl, chunk) + 1024;
+        return ctas * cta <= (size_t)h->sm_smem && cta <= (size_t)h->dev_smem;
+    };
+    for (int c = std::min(most, (nsub + sms - 1) / sms); c >= 1; c--) {
+        if (nsub > 2LL * c * sms) break;
+        for (int sl = kMaxPacketSlots; sl >= 3; sl--)
+            if (fits(sl, c)) return sl;
+    }
+    return nsub <= 2LL * sms && fits(2, 1) ? 2 : 0;
+}
+
+// The subdomain descriptors of single-system launches, and the work items that index them
+void upload_sub_tables(asm_ctx* h) {
+    cudaStream_t st = h->stream;
+    // most expensive subdomains first: the CTAs of the last wave are then the short ones
+    const std::vector<SubDesc> ordered = longest_first({h});
+    h->d_subdesc_single.upload(ordered, st);
+    const std::vector<int2> di = dense_items(ordered);
+    h->d_ditems1.upload(di, st);
+    h->n_ditems1 = (int)di.size();
+    const std::vector<int2> ri = restrict_items(ordered);
+    h->d_ritems1.upload(ri, st);
+    h->n_ritems1 = (int)ri.size();
+    sync(h);
+}
+
+// The factor stream by rows and its pack lists onto the device, for the launches that take it (use_rows)
+void upload_rows(asm_ctx* h) {
+    const SysSym& S = *h->sym;
+    cudaStream_t st = h->stream;
+    const int K = (int)S.subs.size();
+    std::vector<long long> offf, offc;
+    std::vector<int> srcf, srcc;
+    h->d_stream.alloc((size_t)h->stream_base[K]);
+    for (int s = 0; s < K; s++) {
+        const SubSym& o = S.subs[s];
+        if (!o.stream.empty())
+            ck(cudaMemcpyAsync(h->d_stream.as<unsigned char>() + h->stream_base[s], o.stream.data(), o.stream.size(),
+                               cudaMemcpyHostToDevice, st));
+        for (size_t i = 0; i < o.pk_off_f.size(); i++) {
+            offf.push_back(h->stream_base[s] + o.pk_off_f[i]);
+            srcf.push_back((int)(h->slot_base[s] + o.pk_src_f[i]));
+        }
+        for (size_t i = 0; i < o.pk_off_c.size(); i++) {
+            offc.push_back(h->stream_base[s] + o.pk_off_c[i]);
+            srcc.push_back((int)(h->slot_base[s] + o.pk_src_c[i]));
+        }
+    }
+    h->pk_nf = (long long)offf.size();
+    h->pk_nc = (long long)offc.size();
+    h->d_pk_off_f.upload(offf, st);
+    h->d_pk_src_f.upload(srcf, st);
+    h->d_pk_off_c.upload(offc, st);
+    h->d_pk_src_c.upload(srcc, st);
+    for (int s = 0; s < K; s++) h->sub_desc[s].stream = h->d_stream.as<unsigned char>() + h->stream_base[s];
+    upload_sub_tables(h);
+    h->rows_ready = true;
+    h->rows_packed = false;
+}
+void pack_rows(asm_ctx* h) {
+    launch_pack(h->d_pk_off_f.as<long long>(), h->d_pk_src_f.as<int>(), h->pk_nf, h->prec, h->d_stream.as<unsigned char>(),
+                h->d_slot.as<double>(), h->stream);
+    launch_pack(h->d_pk_off_c.as<long long>(), h->d_pk_src_c.as<int>(), h->pk_nc, h->lump32 ? 1 : 0,
+                h->d_stream.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
+    ck(cudaGetLastError());
+    h->rows_packed = true;
+}
+// before a launch of configuration cfg: the stream it reads holds the current factors
+void use_stream(asm_ctx* h, const ApplyConfig& cfg) {
+    if (cfg.ymode == Y_PACKET || h->opt.local_solver == ASM_LOCAL_EXACT || is_nf(h)) return;
+    if (!h->rows_ready) upload_rows(h);
+    if (!h->rows_packed) pack_rows(h);
+}
 void upload_symbolic(asm_ctx* h) {
     SysSym& S = *h->sym;
     cudaStream_t st = h->stream;
@@ -519,7 +613,6 @@ void upload_symbolic(asm_ctx* h) {
     h->stream_base.assign(K + 1, 0);
     h->row_base.assign(K + 1, 0);
     std::vector<long long> aloc_base(K + 1, 0), fp_base(K + 1, 0), rl_base(K + 1, 0), lv_base(K + 1, 0);
-    long long npf = 0, npc = 0;
     for (int s = 0; s < K; s++) {
         const SubSym& o = S.subs[s];
         h->slot_base[s + 1] = h->slot_base[s] + o.nslot;
@@ -533,11 +626,10 @@ void upload_symbolic(asm_ctx* h) {
         fpi += (long long)o.pair.size() + (long long)o.ls.size();
         fp_base[s + 1] = fp_base[s] + fpi;
         long long rli = (long long)o.fcell.size() + o.rptr.size() + o.rsrc.size() + o.rbox.size() + o.rcorr.size() +
-                        o.clong.size() + o.own_pos.size() + o.own_cell.size() + 2LL * o.chunk_off.size();
+                        o.clong.size() + o.own_pos.size() + o.own_cell.size() + 2LL * o.chunk_off.size() +
+                        2LL * o.pk.chunk_off.size();
         rl_base[s + 1] = rl_base[s] + (rli + 1) / 2 * 2;  // even: each block starts 8-byte aligned
         lv_base[s + 1] = lv_base[s] + o.nlev;
-        npf += (long long)o.pk_off_f.size();
-        npc += (long long)o.pk_off_c.size();
     }
     h->total_slots = h->slot_base[K];
     if (h->total_slots >= (1LL << 31) / 9 || aloc_base[K] >= (1LL << 31)) throw CudaFail{ASM_ERR_INVALID_ARG};
@@ -617,17 +709,49 @@ void upload_symbolic(asm_ctx* h) {
         h->d_factdesc.upload(h->fact_desc, st);
     }
     // streams + pack lists + level tables + restriction lists
-    h->d_stream.alloc((size_t)h->stream_base[K]);
+    ck(cudaDeviceGetAttribute(&h->dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
+    ck(cudaDeviceGetAttribute(&h->sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device));
+    ck(cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, h->device));
+    h->lanes_cap = h->lanes_smem = 0;
+    h->rows_ready = h->rows_packed = false;
+    h->d_stream.alloc(16);
+    std::vector<long long> lane_base(K + 1, 0);
+    bool lanes = K > 0;
+    for (int s = 0; s < K; s++) {
+        const SubSym& o = S.subs[s];
+        lanes = lanes && o.pk.chunk_off.size() == o.chunk_off.size() && !o.chunk_off.empty();
+        lane_base[s + 1] = lane_base[s] + (long long)((o.pk.stream.size() + 255) / 256 * 256);
+        h->lanes_cap = std::max(h->lanes_cap, (o.pk.cap + 127) / 128 * 128);
+        h->lanes_smem = std::max(h->lanes_smem, (int)apply_smem_bytes(o.nf, o.n - o.nf, S.prec, S.lump32) + 32);
+    }
+    h->lanes_ok = lanes && lane_slots(h, 1, h->lanes_smem, h->lanes_cap) > 0;
     h->d_rlists.alloc((size_t)std::max<long long>(2, rl_base[K]) * 4);
     std::vector<BoxItem> corr_items;
     std::vector<int> corr_cells;
     int corr_base = 0;
-    std::vector<long long> offf, offc;
-    std::vector<int> srcf, srcc;
-    offf.reserve(npf);
-    srcf.reserve(npf);
-    offc.reserve(npc);
-    srcc.reserve(npc);
+    if (h->lanes_ok) {
+        h->d_lanes.alloc((size_t)lane_base[K]);
+        std::vector<long long> off;
+        std::vector<int> src;
+        for (int group = 0; group < 2; group++) {
+            off.clear();
+            src.clear();
+            for (int s = 0; s < K; s++) {
+                const Packets& k = S.subs[s].pk;
+                const std::vector<long long>& o = group == 0 ? k.off_f : k.off_c;
+                const std::vector<int>& r = group == 0 ? k.src_f : k.src_c;
+                for (const long long v : o) off.push_back(v >= 0 ? lane_base[s] + v : ~(lane_base[s] + ~v));
+                for (const int v : r) src.push_back((int)(h->slot_base[s] + v));
+                if (group == 0)
+                    ck(cudaMemcpyAsync(h->d_lanes.as<unsigned char>() + lane_base[s], k.stream.data(), k.stream.size(),
+                                       cudaMemcpyHostToDevice, st));
+            }
+            (group == 0 ? h->d_ln_off_f : h->d_ln_off_c).upload(off, st);
+            (group == 0 ? h->d_ln_src_f : h->d_ln_src_c).upload(src, st);
+            (group == 0 ? h->ln_nf : h->ln_nc) = (long long)off.size();
+            sync(h);
+        }
+    }
     h->sub_desc.assign(K, SubDesc{});
     h->sub_cost.assign(K, 0.0);
     h->apply_smem = 0;
@@ -637,17 +761,6 @@ void upload_symbolic(asm_ctx* h) {
     h->tuned_ymode = -1;
     for (int s = 0; s < K; s++) {
         const SubSym& o = S.subs[s];
-        if (!o.stream.empty())
-            ck(cudaMemcpyAsync(h->d_stream.as<unsigned char>() + h->stream_base[s], o.stream.data(), o.stream.size(),
-                               cudaMemcpyHostToDevice, st));
-        for (size_t i = 0; i < o.pk_off_f.size(); i++) {
-            offf.push_back(h->stream_base[s] + o.pk_off_f[i]);
-            srcf.push_back((int)(h->slot_base[s] + o.pk_src_f[i]));
-        }
-        for (size_t i = 0; i < o.pk_off_c.size(); i++) {
-            offc.push_back(h->stream_base[s] + o.pk_off_c[i]);
-            srcc.push_back((int)(h->slot_base[s] + o.pk_src_c[i]));
-        }
         std::vector<int> rl;
         rl.reserve(rl_base[s + 1] - rl_base[s]);
         int* base = h->d_rlists.as<int>() + rl_base[s];
@@ -673,7 +786,8 @@ void upload_symbolic(asm_ctx* h) {
         sd.corr0 = corr_base;
         sd.chunk_cap = o.chunk_cap;
         h->chunk_cap = std::max(h->chunk_cap, o.chunk_cap);
-        sd.stream = h->d_stream.as<unsigned char>() + h->stream_base[s];
+        sd.pk_cap = (o.pk.cap + 127) / 128 * 128;
+        sd.pk_stream = h->d_lanes.as<unsigned char>() + lane_base[s];
         sd.y = h->d_y.as<double>() + h->y_base[s];
         {
             const YLayout L = y_layout(o.nf, o.n - o.nf, S.prec, S.lump32);
@@ -689,6 +803,14 @@ void upload_symbolic(asm_ctx* h) {
                 ch.push_back(o.chunk_bytes[i]);
             }
             sd.chunks = reinterpret_cast<const int2*>(put(ch));
+            if (h->lanes_ok) {
+                ch.clear();
+                for (size_t i = 0; i < o.pk.chunk_off.size(); i++) {
+                    ch.push_back((int)o.pk.chunk_off[i]);
+                    ch.push_back(o.pk.chunk_bytes[i]);
+                }
+                sd.pk_chunks = reinterpret_cast<const int2*>(put(ch));
+            }
         }
         sd.fcell = put(o.fcell);
         sd.rptr = put(o.rptr);
@@ -709,12 +831,6 @@ void upload_symbolic(asm_ctx* h) {
     }
     if (h->opt.local_solver == ASM_LOCAL_EXACT) upload_dense(h, st);
     if (is_nf(h)) upload_nf(h, st);
-    h->pk_nf = (long long)offf.size();
-    h->pk_nc = (long long)offc.size();
-    h->d_pk_off_f.upload(offf, st);
-    h->d_pk_src_f.upload(srcf, st);
-    h->d_pk_off_c.upload(offc, st);
-    h->d_pk_src_c.upload(srcc, st);
     // cell-group sums (when any sum list may use them), far boxes, their near-region corrections,
     // and the coarse matrix
     h->box_items.clear();
@@ -749,21 +865,9 @@ void upload_symbolic(asm_ctx* h) {
         it.cells = h->d_corr_cells.as<int>();
         h->box_items.push_back(it);
     }
-    ck(cudaDeviceGetAttribute(&h->dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
-    ck(cudaDeviceGetAttribute(&h->sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device));
-    ck(cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, h->device));
     choose_ring(h);
-    // most expensive subdomains first: the CTAs of the last wave are then the short ones
-    {
-        const std::vector<SubDesc> ordered = longest_first({h});
-        h->d_subdesc_single.upload(ordered, st);
-        const std::vector<int2> di = dense_items(ordered);
-        h->d_ditems1.upload(di, st);
-        h->n_ditems1 = (int)di.size();
-        const std::vector<int2> ri = restrict_items(ordered);
-        h->d_ritems1.upload(ri, st);
-        h->n_ritems1 = (int)ri.size();
-    }
+    upload_sub_tables(h);
+    if (!h->lanes_ok && h->opt.local_solver != ASM_LOCAL_EXACT && !is_nf(h)) upload_rows(h);
     h->d_err.alloc(sizeof(FactErr));
     sync(h);
 }
@@ -1016,10 +1120,14 @@ int factor_numeric(asm_ctx* h) {
                          h->stream);
     } else {
         launch_factor(h->d_factdesc.as<FactDesc>(), (int)S.subs.size(), h->d_err.as<FactErr>(), nullptr, h->stream);
-        launch_pack(h->d_pk_off_f.as<long long>(), h->d_pk_src_f.as<int>(), h->pk_nf, h->prec,
-                    h->d_stream.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
-        launch_pack(h->d_pk_off_c.as<long long>(), h->d_pk_src_c.as<int>(), h->pk_nc, h->lump32 ? 1 : 0,
-                    h->d_stream.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
+        if (h->lanes_ok) {
+            launch_pack_lanes(h->d_ln_off_f.as<long long>(), h->d_ln_src_f.as<int>(), h->ln_nf, h->prec,
+                              h->d_lanes.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
+            launch_pack_lanes(h->d_ln_off_c.as<long long>(), h->d_ln_src_c.as<int>(), h->ln_nc, h->lump32 ? 1 : 0,
+                              h->d_lanes.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
+        }
+        h->rows_packed = false;
+        if (h->rows_ready) pack_rows(h);
     }
     ck(cudaGetLastError());
     ck(cudaEventRecord(e1, h->stream));
@@ -1127,6 +1235,42 @@ void build_batch(Batch& B, cudaStream_t st) {
             bi.push_back(b);
         }
     }
+    // kernel variants shared by the whole batch
+    B.prec = B.hs.empty() ? 0 : B.hs[0]->prec;
+    B.lump32 = !B.hs.empty() && B.hs[0]->lump32;
+    int all_bytes = 0, lump_bytes = 0;
+    bool all_ok = !B.hs.empty();
+    for (asm_ctx* h : B.hs) {
+        all_bytes = std::max(all_bytes, h->apply_smem);
+        lump_bytes = std::max(lump_bytes, h->apply_lump_smem);
+        all_ok = all_ok && h->apply_smem > 0;
+    }
+    if (!all_ok) all_bytes = 0;
+    B.all_bytes = all_bytes;
+    B.lump_bytes = lump_bytes;
+    B.slots = 4;
+    B.chunk = kStreamChunkMin;
+    for (asm_ctx* h : B.hs) {
+        B.slots = std::min(B.slots, h->apply_slots);
+        B.chunk = std::max(B.chunk, h->chunk_cap);
+    }
+    B.nsub = 0;
+    bool lanes = !B.hs.empty() && B.hs[0]->apply_place == 0;
+    int lanes_smem = 0, lanes_cap = 0;
+    for (const asm_ctx* h : B.hs) {
+        B.nsub += (int)h->sub_desc.size();
+        lanes = lanes && h->lanes_ok && h->slots_force == 0;
+        lanes_smem = std::max(lanes_smem, h->lanes_smem);
+        lanes_cap = std::max(lanes_cap, h->lanes_cap);
+    }
+    const int ls = lanes ? lane_slots(B.hs[0], B.nsub, lanes_smem, lanes_cap) : 0;
+    if (ls > 0)
+        B.apply = ApplyConfig{Y_PACKET, lanes_smem, ls, lanes_cap};
+    else if (!B.hs.empty())
+        B.apply = apply_local_vectors(B.nsub, all_bytes, lump_bytes, B.slots, B.chunk, B.hs[0]->sm_smem,
+                                      B.hs[0]->n_sms, B.hs[0]->apply_place, other_slots(B.hs[0]));
+    for (asm_ctx* h : B.hs) use_stream(h, B.apply);  // (may move a handle's descriptors: before they are copied)
+
     sd = longest_first(B.hs);
     B.exact = !B.hs.empty() && B.hs[0]->opt.local_solver == ASM_LOCAL_EXACT;
     B.nf = !B.hs.empty() && is_nf(B.hs[0]);
@@ -1197,28 +1341,6 @@ void build_batch(Batch& B, cudaStream_t st) {
         B.pinned_cap = npin + npin / 2;
         ck(cudaMallocHost((void**)&B.pinned, sizeof(int) * C_NCTL * B.pinned_cap));
     }
-    // kernel variants shared by the whole batch
-    B.prec = B.hs.empty() ? 0 : B.hs[0]->prec;
-    B.lump32 = !B.hs.empty() && B.hs[0]->lump32;
-    int all_bytes = 0, lump_bytes = 0;
-    bool all_ok = !B.hs.empty();
-    for (asm_ctx* h : B.hs) {
-        all_bytes = std::max(all_bytes, h->apply_smem);
-        lump_bytes = std::max(lump_bytes, h->apply_lump_smem);
-        all_ok = all_ok && h->apply_smem > 0;
-    }
-    if (!all_ok) all_bytes = 0;
-    B.all_bytes = all_bytes;
-    B.lump_bytes = lump_bytes;
-    B.slots = 4;
-    B.chunk = kStreamChunkMin;
-    for (asm_ctx* h : B.hs) {
-        B.slots = std::min(B.slots, h->apply_slots);
-        B.chunk = std::max(B.chunk, h->chunk_cap);
-    }
-    if (!B.hs.empty())
-        B.apply = apply_local_vectors(B.nsub, all_bytes, lump_bytes, B.slots, B.chunk, B.hs[0]->sm_smem,
-                                      B.hs[0]->n_sms, B.hs[0]->apply_place, other_slots(B.hs[0]));
 }
 
 // events bracketing the launch groups of one step: [prep | apply | post | spmv | mgs+finish]
@@ -1242,7 +1364,7 @@ std::vector<ApplyConfig> apply_candidates(const Batch& B) {
     std::vector<ApplyConfig> c;
     if (B.hs.empty() || B.exact || B.nf) return c;
     const asm_ctx* h = B.hs[0];
-    if (h->apply_place != 0) return {B.apply};
+    if (h->apply_place != 0 || B.apply.ymode == Y_PACKET) return {B.apply};
     for (int force : {Y_SMEM + 1, Y_LUMPS + 1, Y_DEVICE + 1}) {
         const ApplyConfig a =
             apply_local_vectors(B.nsub, B.all_bytes, B.lump_bytes, B.slots, B.chunk, h->sm_smem, h->n_sms, force,
@@ -1563,7 +1685,7 @@ size_t ctx_device_bytes(const asm_ctx* h) {
     const DBuf* bufs[] = {&h->d_ell_val, &h->d_ell_col, &h->d_ell_loc, &h->d_bsr_rp, &h->d_bsr_val, &h->d_bcell,
                           &h->d_cptr, &h->d_cloc, &h->d_cval, &h->d_boxsum, &h->d_slot, &h->d_dpiv, &h->d_aptr,
                           &h->d_aloc, &h->d_acs, &h->d_along, &h->d_fp, &h->d_stream, &h->d_pk_off_f, &h->d_pk_src_f,
-                          &h->d_pk_off_c, &h->d_pk_src_c, &h->d_lv, &h->d_rlists, &h->d_y, &h->d_corr_cells,
+                          &h->d_pk_off_c, &h->d_pk_src_c, &h->d_lanes, &h->d_ln_off_f, &h->d_ln_src_f, &h->d_ln_off_c, &h->d_ln_src_c, &h->d_lv, &h->d_rlists, &h->d_y, &h->d_corr_cells,
                           &h->d_corr, &h->d_dev_err, &h->d_gsum, &h->d_r32, &h->d_factdesc, &h->d_subdesc_single,
                           &h->d_err, &h->d_ws,
                           &h->d_scal, &h->d_ctl, &h->d_partial, &h->d_tab1, &h->d_vec1, &h->d_row1, &h->d_box1,
@@ -1611,6 +1733,7 @@ unsigned long long fnv1a(const void* p, size_t n, unsigned long long h) {
 
 struct asm_server {
     asm_server_options opt{};
+    int sms = 1;
     cudaStream_t stream = nullptr;
     size_t budget = 0, resident = 0;
     long long next_ticket = 1;
@@ -1673,7 +1796,8 @@ void sym_worker(asm_server* S) {
                 }
                 g.far_mode = q.far_mode;
                 e.sym = std::make_shared<SysSym>();
-                e.err = build_symbolic(g, e.pat, S->opt.precision, S->opt.lump_precision == ASM_LUMP_FP32 ? 1 : 0, 1, *e.sym, 0);
+                e.err = build_symbolic(g, e.pat, S->opt.precision, S->opt.lump_precision == ASM_LUMP_FP32 ? 1 : 0, 1, *e.sym, 0, 0,
+                                       wants_lanes(g, S->sms));
             }
         } catch (const std::exception& ex) {
             e.sym.reset();
@@ -2097,9 +2221,11 @@ int asm_factor(asm_handle h) {
         if (!h->sym_valid) {
             auto t0 = std::chrono::steady_clock::now();
             h->sym = std::make_shared<SysSym>();
+            if (h->n_sms <= 1) ck(cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, h->device));
             std::string e = build_symbolic(h->geom, h->pat, h->prec, h->lump32 ? 1 : 0,
                                            h->opt.local_solver == ASM_LOCAL_BILU0_COLSUM ? 1 : 0,
-                                           *h->sym, 0, h->chunk_force);
+                                           *h->sym, 0, h->chunk_force,
+                                           h->opt.local_solver <= ASM_LOCAL_BILU0 && wants_lanes(h->geom, h->n_sms));
             if (!e.empty()) {
                 h->last_error = e;
                 h->sym.reset();
@@ -2115,14 +2241,22 @@ int asm_factor(asm_handle h) {
     });
 }
 
+// the ASM_TUNE_APPLY_SMEM value of a placement
+int placement_code(int ymode) { return ymode == Y_SMEM || ymode == Y_PACKET ? 3 : (ymode == Y_LUMPS ? 2 : 0); }
+
 // the placement of a single-system apply: `place` as ASM_TUNE_APPLY_SMEM stores it (0 automatic)
 ApplyConfig single_apply_config(const asm_ctx* h, int place) {
+    if (place == 0 && h->lanes_ok && h->slots_force == 0) {
+        const int ls = lane_slots(h, (int)h->sub_desc.size(), h->lanes_smem, h->lanes_cap);
+        if (ls > 0) return ApplyConfig{Y_PACKET, h->lanes_smem, ls, h->lanes_cap};
+    }
     return apply_local_vectors((int)h->sub_desc.size(), h->apply_smem, h->apply_lump_smem, h->apply_slots,
                                h->chunk_cap, h->sm_smem, h->n_sms, place, other_slots(h));
 }
 
 // R_i r and the fused ILU sweeps of every subdomain (after k_sums), single-system tables
 void launch_ilu_local_solves(asm_ctx* h, const ApplyConfig& cfg) {
+    use_stream(h, cfg);
     launch_restrict(h->d_tab1.as<SysTab>(), h->d_subdesc_single.as<SubDesc>(), h->d_ritems1.as<int2>(), h->n_ritems1,
                     h->prec, h->lump32, h->stream);
     launch_apply(h->d_tab1.as<SysTab>(), h->d_subdesc_single.as<SubDesc>(), (int)h->sub_desc.size(), h->prec,
@@ -2185,6 +2319,7 @@ int asm_tune_tiling(asm_handle h, int reps, asm_tiling_report* out) {
             ensure_workspace(h);
             set_ctl(h, VU, VZ, -1, -1, -1);
             const ApplyConfig cfg = single_apply_config(h, place);
+            use_stream(h, cfg);
             std::vector<float> t;
             for (int k = 0; k < reps + 2; k++) {
                 ck(cudaEventRecord(e0, h->stream));
@@ -2215,6 +2350,7 @@ int asm_tune_tiling(asm_handle h, int reps, asm_tiling_report* out) {
         int stt = rebuild(0);
         if (stt != ASM_OK) return stt;
         out->rule_ms = time_apply(0);
+        bool by_lane[ASM_TILING_MAX] = {};
         std::vector<std::vector<int>> seen;
         for (int kb : {0, 8, 12, 16, 20, 24}) {
             h->slots_force = 0;
@@ -2232,6 +2368,8 @@ int asm_tune_tiling(asm_handle h, int reps, asm_tiling_report* out) {
                 int place, slots;
             };
             std::vector<Cand> cands;
+            h->slots_force = 0;
+            if (single_apply_config(h, 0).ymode == Y_PACKET) cands.push_back({0, 0});  // the stream by lane
             for (int place : {Y_SMEM + 1, Y_LUMPS + 1, Y_DEVICE + 1})
                 for (int sl = 2; sl <= 4; sl++) cands.push_back({place, sl});
             for (const Cand& c : cands) {
@@ -2239,13 +2377,14 @@ int asm_tune_tiling(asm_handle h, int reps, asm_tiling_report* out) {
                 h->slots_force = c.slots;
                 choose_ring(h);
                 const ApplyConfig cfg = single_apply_config(h, c.place);
-                if (cfg.ymode != c.place - 1) continue;  // does not fit
+                if (c.place != 0 && cfg.ymode != c.place - 1) continue;  // does not fit
                 asm_tiling_entry& e = out->e[out->n];
                 e.chunk_kb = kb;
                 e.chunk_max_kb = h->chunk_cap / 1024;
                 e.chunks = chunks;
-                e.placement = cfg.ymode == Y_SMEM ? 3 : (cfg.ymode == Y_LUMPS ? 2 : 0);
+                e.placement = placement_code(cfg.ymode);
                 e.slots = cfg.slots;
+                by_lane[out->n] = c.place == 0;
                 e.ctas_per_sm = apply_ctas_per_sm(h->prec, h->lump32, cfg);
                 e.apply_ms = time_apply(c.place);
                 out->n++;
@@ -2261,11 +2400,11 @@ int asm_tune_tiling(asm_handle h, int reps, asm_tiling_report* out) {
         for (int k = 1; k < out->n; k++)
             if (out->e[k].apply_ms < out->e[out->best].apply_ms) out->best = k;
         const asm_tiling_entry& b = out->e[out->best];
-        h->slots_force = b.slots;
+        h->slots_force = by_lane[out->best] ? 0 : b.slots;
         stt = rebuild(b.chunk_kb * 1024);
         if (stt != ASM_OK) return stt;
         choose_ring(h);
-        h->apply_place = b.placement == 3 ? Y_SMEM + 1 : (b.placement == 2 ? Y_LUMPS + 1 : Y_DEVICE + 1);
+        h->apply_place = by_lane[out->best] ? 0 : b.placement == 3 ? Y_SMEM + 1 : (b.placement == 2 ? Y_LUMPS + 1 : Y_DEVICE + 1);
         h->no_autotune = true;
         h->tuned_ymode = -1;
         return ASM_OK;
@@ -2402,7 +2541,7 @@ int asm_tune_tiling_batch(asm_handle* hs, int n, const double* const* b, double*
             e.chunk_kb = kb;
             e.chunk_max_kb = cmax / 1024;
             e.chunks = chunks;
-            e.placement = a.ymode == Y_SMEM ? 3 : (a.ymode == Y_LUMPS ? 2 : 0);
+            e.placement = placement_code(a.ymode);
             e.slots = a.slots;
             e.ctas_per_sm = apply_ctas_per_sm(h0->prec, h0->lump32, a);
             e.apply_ms = ms;
@@ -2450,10 +2589,10 @@ int asm_get_stats(asm_handle h, asm_stats* st) {
         for (const SubSym& o : h->sym->subs) st->stream_chunks += (long long)o.chunk_off.size();
         const int place = h->apply_place != 0 ? h->apply_place : (h->tuned_ymode >= 0 ? h->tuned_ymode + 1 : 0);
         const ApplyConfig cfg = single_apply_config(h, place);
-        st->apply_placement = cfg.ymode == Y_SMEM ? 3 : (cfg.ymode == Y_LUMPS ? 2 : 0);
+        st->apply_placement = placement_code(cfg.ymode);
         st->apply_slots = cfg.slots;
         const ApplyConfig& l = h->last_solve_apply;
-        st->last_solve_placement = l.ymode < 0 ? -1 : (l.ymode == Y_SMEM ? 3 : (l.ymode == Y_LUMPS ? 2 : 0));
+        st->last_solve_placement = l.ymode < 0 ? -1 : placement_code(l.ymode);
         st->last_solve_slots = l.ymode < 0 ? 0 : l.slots;
         st->last_solve_chunk_kb = l.ymode < 0 ? 0 : l.chunk / 1024;
     }
@@ -2651,6 +2790,11 @@ int asm_server_create(asm_server_handle* out, const asm_server_options* opt, voi
     S->stream = static_cast<cudaStream_t>(cuda_stream);
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+        cudaGetLastError();
+        delete S;
+        return ASM_ERR_CUDA;
+    }
+    if (cudaDeviceGetAttribute(&S->sms, cudaDevAttrMultiProcessorCount, o.device) != cudaSuccess) {
         cudaGetLastError();
         delete S;
         return ASM_ERR_CUDA;

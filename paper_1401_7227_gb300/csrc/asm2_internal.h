@@ -31,17 +31,20 @@ constexpr int kLongLumpRow = 16;     // lump rows with more stored blocks are sw
 // vector (and, for FP64 lump rows, its FP32 mirror) then stays in shared memory when four CTAs'
 // worth fit, else it goes to device memory too.
 constexpr int kApplyThreadsDev = 256;
-enum ApplyY { Y_SMEM = 0, Y_LUMPS = 1, Y_DEVICE = 2 };  // where the apply's local vectors live
+// Y_PACKET: all in shared memory and the factor stream by lane (packets.h), the automatic choice
+// where every subdomain of the launch fits.
+enum ApplyY { Y_SMEM = 0, Y_LUMPS = 1, Y_DEVICE = 2, Y_PACKET = 3 };  // where the apply's local vectors live
 struct ApplyConfig {
     int ymode;  // ApplyY
     int smem;   // dynamic shared memory of the vectors (bytes)
-    int slots;  // factor-stream ring slots (2..4; the tiling tuner measured deeper rings slower)
+    int slots;  // factor-stream ring slots: 2..4 (Y_PACKET: 2..kMaxPacketSlots)
     int chunk;  // bytes of one ring slot: the largest chunk capacity of the launch's subdomains
 };
 // Chunk header word 6: bit 0 = last chunk of its wavefront level; bits 8..11 = log2 of the entry
 // slots S of the short lump rows (each such row takes 3 S lanes: 3 output components x S slots);
 // kChunkLongLumps = the chunk holds a lump row of more than kLongLumpRow blocks.
 constexpr int kChunkLongLumps = 1 << 12;
+constexpr int kMaxPacketSlots = 8, kPkWarps = 16;  // ring slots; warps of its CTA
 constexpr int VEC_THREADS = 256;
 constexpr int kCgsMax = 64;  // classical Gram-Schmidt: at most kCgsMax - 2 basis vectors (restart)
 enum VecSlot { VX = 0, VB = 1, VR = 2, VW = 3, VZ = 4, VU = 5, VV0 = 6 };  // V_k = VV0 + k; Z_k after V
@@ -187,6 +190,9 @@ struct SubDesc {
     const double* dinv;          // exact local solves: [A_i | A_i^{-1}] (3n x 6n), fine then lump order
     const int2* chunks;          // (byte offset, bytes) of every chunk, consumption order
     const unsigned char* stream; // 16-byte aligned
+    int pk_cap;                  // the stream by lane: bytes of its largest chunk, chunks and bytes
+    const int2* pk_chunks;
+    const unsigned char* pk_stream;
     double* y;        // the local vectors in device memory (written by k_restrict, 16-byte aligned)
     int y_fine;       // byte offsets within y: fine rows, and the FP32 mirror of FP64 lumps; lumps at 0
     int y_mirror;
@@ -259,6 +265,9 @@ void launch_coarse(const int* cptr, const int* cloc, const double* bsr_val, doub
 void launch_factor(const FactDesc* fd, int nsub, FactErr* err, const int* sub_ids, cudaStream_t st);
 void launch_pack(const long long* off, const int* src, long long n, int prec, unsigned char* stream_base,
                  const double* slot_base, cudaStream_t st);
+// the same blocks into the streams by lane (packets.h: off holds ~offset for the blocks of a long lump row)
+void launch_pack_lanes(const long long* off, const int* src, long long n, int prec, unsigned char* stream_base,
+                       const double* slot_base, cudaStream_t st);
 void launch_ell_fill(const double* bsr_vals, const int* row_ptr, int n, int ell_w, double* ell_val, int rows_pad,
                      cudaStream_t st);
 

@@ -273,6 +273,40 @@ __global__ void k_pack(const long long* __restrict__ off, const int* __restrict_
     }
 }
 
+// The same blocks into the packets of the stream by lane: element (k, t) of a block lies 30 t + lane
+// values from its offset, the lanes of k = 0, 1, 2 next to each other (eight apart in the packet of a
+// long lump row); an FP16 row's record is {three halves, exponent} per lane.  Neighbouring threads hold
+// neighbouring rows of a packet.
+template <typename T>
+__global__ void k_pack_lanes(const long long* __restrict__ off, const int* __restrict__ src, long long n,
+                             unsigned char* __restrict__ base, const double* __restrict__ slot) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double* v = slot + (long long)src[i] * 9;
+    const long long o = off[i];
+    unsigned char* dst = base + (o >= 0 ? o : ~o);
+    if constexpr (sizeof(T) == 2) {
+        double mx = 0.0;
+#pragma unroll
+        for (int e = 0; e < 9; e++) mx = fmax(mx, fabs(v[e]));
+        const int ex = mx > 0.0 ? ilogb(mx) + 1 : 0;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            unsigned short h[3];
+#pragma unroll
+            for (int t = 0; t < 3; t++) h[t] = __half_as_ushort(__double2half(ldexp(v[3 * k + t], -ex)));
+            reinterpret_cast<uint2*>(dst)[k] =
+                make_uint2(h[0] | (unsigned)h[1] << 16, h[2] | (unsigned)(unsigned short)(short)ex << 16);
+        }
+    } else {
+        const int lane = o >= 0 ? 1 : 8;
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+#pragma unroll
+            for (int t = 0; t < 3; t++) reinterpret_cast<T*>(dst)[30 * t + lane * k] = (T)v[3 * k + t];
+    }
+}
+
 inline unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
 }  // namespace
@@ -316,6 +350,18 @@ void launch_pack(const long long* off, const int* src, long long n, int prec, un
         k_pack<float><<<g, 256, 0, st>>>(off, src, n, stream_base, slot_base);
     else
         k_pack<__half><<<g, 256, 0, st>>>(off, src, n, stream_base, slot_base);
+}
+
+void launch_pack_lanes(const long long* off, const int* src, long long n, int prec, unsigned char* stream_base,
+                       const double* slot_base, cudaStream_t st) {
+    if (n <= 0) return;
+    const unsigned g = blocks_for(n, 256);
+    if (prec == 0)
+        k_pack_lanes<double><<<g, 256, 0, st>>>(off, src, n, stream_base, slot_base);
+    else if (prec == 1)
+        k_pack_lanes<float><<<g, 256, 0, st>>>(off, src, n, stream_base, slot_base);
+    else
+        k_pack_lanes<__half><<<g, 256, 0, st>>>(off, src, n, stream_base, slot_base);
 }
 
 }  // namespace asm2

@@ -6,9 +6,11 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "asm2_internal.h"
 #include "f64cvt.h"
+#include "packets.h"
 #include "tma.h"
 
 namespace asm2 {
@@ -817,6 +819,235 @@ __global__ void __launch_bounds__(YM == Y_SMEM ? 256 : kApplyThreadsDev, YM == Y
     }
 }
 
+// ------------------------------------------------------------------------------------------
+// The fused local solve from the factor stream by lane (packets.h), every local vector in shared
+// memory.  The time is the chain of wavefront levels, and a level's time is the instructions one warp
+// runs between two CTA barriers: with the other layout a thread takes ~400 of them, most to find
+// its row's pointers, columns and blocks.  Here a warp takes a packet of ten rows, three lanes per row:
+// per entry a lane reads one operand offset, the operand row and its component's three values,
+// all at fixed offsets from one pointer.  The operations and their order are those of
+// sweep_chunk, so the results are the same bits.
+// ------------------------------------------------------------------------------------------
+
+// shared-memory accesses by 32-bit address: the address arithmetic of a packet is then one add per access
+// at most.  (volatile: they stay on their side of the barriers)
+__device__ __forceinline__ int lds_i(unsigned a) {
+    int v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ int lds_byte(unsigned a) {
+    int v;
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void lds(unsigned a, float& v) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a)); }
+__device__ __forceinline__ void lds(unsigned a, double& v) { asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a)); }
+__device__ __forceinline__ int4 lds_i4(unsigned a) {
+    int4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts(unsigned a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void sts(unsigned a, double v) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
+// a row of the local vectors
+__device__ __forceinline__ void lds_row(unsigned a, float (&x)[3]) {
+    [[maybe_unused]] float w;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(w) : "r"(a));
+    (void)w;
+}
+__device__ __forceinline__ void lds_row(unsigned a, double (&x)[3]) {
+    lds(a, x[0]);
+    lds(a + 8, x[1]);
+    lds(a + 16, x[2]);
+}
+
+// the three values of a lane: of a stored block row, with the power of two of an FP16 record
+template <typename T, bool HALF>
+struct LaneVal {
+    T v[3], sc;
+    static constexpr int size = HALF ? 8 : (int)sizeof(T);       // from one lane to the next
+    static constexpr int stride = (HALF ? 1 : 3) * size * kPkLanes;  // from one entry to the next
+    __device__ __forceinline__ void load(unsigned a) {
+        if constexpr (HALF) {
+            unsigned w0, w1;
+            asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(w0), "=r"(w1) : "r"(a));
+            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w0));
+            v[0] = f.x;
+            v[1] = f.y;
+            v[2] = __half2float(__ushort_as_half((unsigned short)(w1 & 0xffffu)));
+            sc = __int_as_float((127 + (int)(short)(w1 >> 16)) << 23);
+        } else {
+#pragma unroll
+            for (int t = 0; t < 3; t++) lds(a + t * kPkLanes * size, v[t]);
+        }
+    }
+};
+
+// One packet: pk, val the addresses of it and of its values; kind: its kind word (packets.h); y: address of the
+// local vectors.  TYPE: kPkFine, kPkLump, kPkLong; HALF: FP16 records (fine rows of FP16 factors).
+template <typename T, int TYPE, bool HALF>
+__device__ __forceinline__ void packet_rows(unsigned pk, unsigned val, int kind, unsigned y) {
+    constexpr bool kOwnFirst = sizeof(T) == 8 && TYPE == kPkFine;   // a row's sum starts from its own entry
+    constexpr bool kPlus = (sizeof(T) == 8 && TYPE == kPkLump) || TYPE == kPkLong;  // products summed, then subtracted
+    constexpr unsigned kAll = 0xffffffffu;
+    using LV = LaneVal<T, HALF>;
+    const int lane = threadIdx.x & 31;
+    const int ln = min(lane, TYPE == kPkLong ? 23 : kPkLanes - 1);  // the spare lanes repeat the last one
+    const int pos = TYPE == kPkLong ? ln & 7 : ln / 3, k = TYPE == kPkLong ? ln >> 3 : ln % 3;
+    const int lg = TYPE == kPkLump ? (kind >> 12) & 15 : 0;
+    const int out = lds_i(pk + 4 * pos);
+    unsigned idx = pk + kPkIdx + 4 * pos;
+    val += ln * LV::size;
+    const bool head = lane < (TYPE == kPkLong ? 24 : kPkLanes) && out >= 0 &&
+                      (TYPE == kPkLong ? pos == 0 : (pos & ((1 << lg) - 1)) == 0);
+    const unsigned yo = y + out + k * (int)sizeof(T);
+    T own = T(0), acc = T(0);
+    if (head) lds(yo, own);
+    if (kOwnFirst) acc = own;
+    const auto mac = [&](const LV& b, const T (&x)[3]) {
+        if constexpr (HALF)
+            acc = fma(-b.sc, fma(b.v[0], x[0], fma(b.v[1], x[1], b.v[2] * x[2])), acc);
+        else if constexpr (kPlus)
+            acc = fma(b.v[0], x[0], fma(b.v[1], x[1], fma(b.v[2], x[2], acc)));
+        else if constexpr (kOwnFirst)
+            acc = fma(-b.v[2], x[2], fma(-b.v[1], x[1], fma(-b.v[0], x[0], acc)));
+        else
+            acc = fma(-b.v[0], x[0], fma(-b.v[1], x[1], fma(-b.v[2], x[2], acc)));
+    };
+    // entries in groups whose loads are all issued before their multiply-adds (a 7-point fine row has three on a
+    // side)
+    const auto group = [&](auto count) {
+        constexpr int N = decltype(count)::value;
+        LV b[N];
+        T x[N][3];
+        int o[N];
+#pragma unroll
+        for (int u = 0; u < N; u++) o[u] = lds_i(idx + 4 * kPkPos * u);
+#pragma unroll
+        for (int u = 0; u < N; u++) b[u].load(val + u * LV::stride);
+#pragma unroll
+        for (int u = 0; u < N; u++) lds_row(y + o[u], x[u]);
+#pragma unroll
+        for (int u = 0; u < N; u++) mac(b[u], x[u]);
+        idx += 4 * kPkPos * N;
+        val += LV::stride * N;
+    };
+    int left = kind & 255;
+    for (; left >= 3; left -= 3) group(std::integral_constant<int, 3>());
+    if (left == 2) group(std::integral_constant<int, 2>());
+    if (left == 1) group(std::integral_constant<int, 1>());
+    LV d;
+    if (kind >> 16) d.load(val);
+    if constexpr (TYPE == kPkLump)
+        for (int o = 3; o < 3 << lg; o <<= 1) acc += __shfl_down_sync(kAll, acc, o);
+    if constexpr (TYPE == kPkLong)
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) acc += __shfl_xor_sync(kAll, acc, o);
+    T r = kOwnFirst ? acc : kPlus ? own - acc : acc + own;
+    if (kind >> 16) {  // backward: D^{-1} of the three components
+        const int l0 = TYPE == kPkLong ? 0 : lane - k, ls = TYPE == kPkLong ? 8 : 1;
+        const T r0 = __shfl_sync(kAll, r, l0), r1 = __shfl_sync(kAll, r, l0 + ls), r2 = __shfl_sync(kAll, r, l0 + 2 * ls);
+        r = fma(d.v[0], r0, fma(d.v[1], r1, d.v[2] * r2));
+        if constexpr (HALF) r *= d.sc;
+    }
+    if (head) sts(yo, r);
+}
+
+template <typename TF>
+__global__ void __launch_bounds__(32 * kPkWarps, sizeof(TF) == 8 ? 1 : 2) k_apply_packets(const SysTab* __restrict__ tab,
+                                                                                         const SubDesc* __restrict__ subs,
+                                                                                         int slots) {
+    using T = typename Compute<TF>::T;
+    constexpr bool kHalf = sizeof(TF) == 2;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const SubDesc& sd = subs[blockIdx.x];
+    const SysTab& st = tab[sd.sys];
+    if (st.ctl[C_APPLY_IN] < 0) return;
+    double* __restrict__ z = st.ws + (long long)st.ctl[C_APPLY_OUT] * st.n3p;
+    const int cap = sd.pk_cap, n_chunks = sd.n_chunks;
+    const int2* __restrict__ chunks = sd.pk_chunks;
+    const unsigned char* __restrict__ stream = sd.pk_stream;
+    unsigned char* ring = smem_raw;
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_raw + (size_t)slots * cap);
+    unsigned char* y = smem_raw + (size_t)slots * cap + kRingHeader;  // the local vectors, then a row of zeros
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const unsigned ring_a = tma::smem_u32(ring), ya = tma::smem_u32(y);
+    const long long limit = st.wait_limit;
+    if (tid == 0) {
+        for (int k = 0; k < slots; k++) mbar_init(&bar[k], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    if (tid == 0)
+        for (int k = 0; k < slots && k < n_chunks; k++) {
+            const int2 ch = chunks[k];
+            mbar_expect_tx(&bar[k], (unsigned)ch.y);
+            bulk_load(ring + (size_t)k * cap, stream + ch.x, (unsigned)ch.y, &bar[k]);
+        }
+    {
+        const int4* src = reinterpret_cast<const int4*>(sd.y);
+        const int n16 = sd.y_bytes >> 4;
+        for (int t = tid; t < n16; t += blockDim.x) reinterpret_cast<int4*>(y)[t] = src[t];
+        if (tid < 2) reinterpret_cast<int4*>(y)[n16 + tid] = make_int4(0, 0, 0, 0);
+    }
+    // The last warp (with the fewest packets) waits for the next chunk to land while the others work on this
+    // one, so that nobody waits after the barrier; its lane 0 refills the slots, and keeps the next
+    // descriptor, loaded one ahead.
+    const bool waiter = warp == kPkWarps - 1, issuer = waiter && (tid & 31) == 0;
+    int2 next_ch = make_int2(0, 0);
+    if (issuer && slots < n_chunks) next_ch = chunks[slots];
+    bool ok = true;
+    if (waiter && n_chunks > 0) ok = __all_sync(0xffffffffu, mbar_wait(&bar[0], 0u, limit));
+    bool expired = __syncthreads_or(!ok);
+    int slot = 0;
+    unsigned parity = 0;
+    for (int ci = 0; ci < n_chunks; ci++) {
+        if (expired) {
+            // a copy did not land in time: report it, wait (bounded) for the copies still in flight
+            // into this CTA's shared memory, and leave
+            if (tid == 0) {
+                atomicExch(st.dev_err, 7);
+                const int last = min(n_chunks, ci + slots);
+                for (int k = max(0, ci - 1); k < last; k++) mbar_wait(&bar[k % slots], (unsigned)(k / slots) & 1u);
+            }
+            return;
+        }
+        const unsigned base = ring_a + slot * cap;
+        const int q1 = lds_byte(base + warp);
+        for (int q = warp > 0 ? lds_byte(base + warp - 1) : 0; q < q1; q++) {
+            const int4 d = lds_i4(base + kPkWarps + 16 * q);
+            const int type = (d.z >> 8) & 15;
+            if (type == kPkFine)
+                packet_rows<T, kPkFine, kHalf>(base + d.x, base + d.y, d.z, ya);
+            else if (type == kPkLump)
+                packet_rows<T, kPkLump, false>(base + d.x, base + d.y, d.z, ya);
+            else
+                packet_rows<T, kPkLong, false>(base + d.x, base + d.y, d.z, ya);
+        }
+        const int nslot = slot + 1 == slots ? 0 : slot + 1;
+        const unsigned nparity = slot + 1 == slots ? parity ^ 1u : parity;
+        if (waiter && ci + 1 < n_chunks) ok = __all_sync(0xffffffffu, mbar_wait(&bar[nslot], nparity, limit));
+        expired = __syncthreads_or(!ok);
+        if (issuer && !expired && ci + slots < n_chunks) {
+            mbar_expect_tx(&bar[slot], (unsigned)next_ch.y);
+            bulk_load(ring + (size_t)slot * cap, stream + next_ch.x, (unsigned)next_ch.y, &bar[slot]);
+            if (ci + slots + 1 < n_chunks) next_ch = chunks[ci + slots + 1];
+        }
+        slot = nslot;
+        parity = nparity;
+    }
+    // P_i R_i^T: owned cells take this subdomain's solution; the lumps are discarded
+    constexpr int kRow = sizeof(T) == 8 ? 24 : 16;
+    for (int t = tid; t < sd.n_own; t += blockDim.x) {
+        const T* f = reinterpret_cast<const T*>(y + sd.y_fine + kRow * sd.own_pos[t]);
+        const long long c = 3LL * sd.own_cell[t];
+        z[c] = f[0];
+        z[c + 1] = f[1];
+        z[c + 2] = f[2];
+    }
+}
+
 // Exact local solves: R_i r into the subdomain's FP64 local vector, fine indices then lump indices
 // (the order of the dense A_i^{-1}); one CTA per subdomain
 __global__ void __launch_bounds__(256) k_dense_restrict(const SysTab* __restrict__ tab, const SubDesc* __restrict__ subs) {
@@ -880,6 +1111,20 @@ void launch_apply_s(const SysTab* tab, const SubDesc* subs, int nsub, int smem, 
     else
         launch_apply_t<TF, TL, YM, 4>(tab, subs, nsub, smem, st, occ);
 }
+template <typename TF>
+void launch_apply_packets(const SysTab* tab, const SubDesc* subs, int nsub, ApplyConfig cfg, cudaStream_t st, int* occ) {
+    static int configured = -1;
+    const int smem = (int)apply_ring_bytes(cfg.slots, cfg.chunk) + cfg.smem;
+    if (configured < smem) {
+        cudaFuncSetAttribute(k_apply_packets<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        configured = smem;
+    }
+    if (occ != nullptr) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k_apply_packets<TF>, 32 * kPkWarps, smem) != cudaSuccess) *occ = 0;
+        return;
+    }
+    k_apply_packets<TF><<<nsub, 32 * kPkWarps, smem, st>>>(tab, subs, cfg.slots);
+}
 template <typename TF, typename TL>
 void launch_apply_p(const SysTab* tab, const SubDesc* subs, int nsub, ApplyConfig cfg, int slots, cudaStream_t st,
                     int* occ) {
@@ -894,6 +1139,15 @@ void launch_apply_p(const SysTab* tab, const SubDesc* subs, int nsub, ApplyConfi
 // the k_apply instance of (prec, lump32, cfg): launched, or (occ != nullptr) its resident CTAs per SM
 void apply_dispatch(const SysTab* tab, const SubDesc* subs, int nsub, int prec, bool lump32, ApplyConfig cfg,
                     cudaStream_t st, int* occ) {
+    if (cfg.ymode == Y_PACKET) {
+        if (prec == 0)
+            launch_apply_packets<double>(tab, subs, nsub, cfg, st, occ);
+        else if (prec == 1)
+            launch_apply_packets<float>(tab, subs, nsub, cfg, st, occ);
+        else
+            launch_apply_packets<__half>(tab, subs, nsub, cfg, st, occ);
+        return;
+    }
     const int slots = cfg.slots < 2 ? 2 : (cfg.slots > kMaxSlots ? kMaxSlots : cfg.slots);
     if (prec == 0)
         launch_apply_p<double, double>(tab, subs, nsub, cfg, slots, st, occ);

@@ -716,7 +716,7 @@ std::string build_pattern(int n, const int* rp, const int* ci, int nnzb, Pattern
 }
 
 std::string build_symbolic(const Geom& g, const Pattern& A, int prec, int lump32, int colsum, SysSym& S,
-                           int threads, int chunk_force) {
+                           int threads, int chunk_force, bool packets) {
     const int N = g.n_cells();
     if (A.n != N) return "matrix size does not match the grid";
     if (chunk_force != 0 &&
@@ -800,7 +800,11 @@ std::string build_symbolic(const Geom& g, const Pattern& A, int prec, int lump32
         for (;;) {
             int s = next.fetch_add(1);
             if (s >= K) break;
-            err[s] = build_sub(X, s, S.subs[s]);
+            SubSym& o = S.subs[s];
+            err[s] = build_sub(X, s, o);
+            if (packets && err[s].empty() && (prec == 0 || lump32))
+                build_packets(o.stream, o.chunk_off, o.n_fwd_chunks, o.pk_src_f, o.pk_src_c, o.nf, o.n - o.nf, prec,
+                              lump32 != 0, o.pk);
         }
     };
     std::vector<std::thread> pool;

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "asm2_internal.h"
+#include "packets.h"
 
 namespace asm2 {
 
@@ -67,6 +68,7 @@ struct SubSym {
     std::vector<unsigned char> stream;  // indices filled in, values zero
     std::vector<long long> pk_off_f, pk_off_c;
     std::vector<int> pk_src_f, pk_src_c;
+    Packets pk;  // the same chunks laid out by lane (when asked for)
     // cell -> local row over the whole grid is not stored; map_region gives it for parity hooks
     std::vector<int> cells_of_row_ptr, cells_of_row;  // fine cell or lump cells, by local row
     long long apply_index_bytes = 0;
@@ -95,9 +97,10 @@ struct SysSym {
 // 2 f16 element storage of fine-row factors; lump32: lump-row factors stored in FP32 (else FP64);
 // colsum: compensation on/off.  threads <= 0: auto.  chunk_force: 0, or the stream-chunk capacity
 // in bytes (a multiple of 4096 in [kStreamChunkMin, kStreamChunkMax]) for every subdomain, raised
-// where one row needs more.
+// where one row needs more.  packets: also the factor stream by lane (not for FP64 lump rows under
+// narrower fine rows).
 std::string build_symbolic(const Geom& g, const Pattern& A, int prec, int lump32, int colsum, SysSym& out,
-                           int threads, int chunk_force = 0);
+                           int threads, int chunk_force = 0, bool packets = false);
 
 // Aligned 2 x 2 x 2 cell groups: group of a cell, group count, and a group's cells in the grid
 // (x, y, z each in {2 g, 2 g + 1} within the grid; z fastest, as cells are numbered)
