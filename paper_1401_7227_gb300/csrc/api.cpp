@@ -82,8 +82,11 @@ struct DBuf {
 // whether the factor stream by lane is built for a system: a launch of its subdomains alone may take it (lane_slots)
 static bool wants_lanes(const Geom& g, int sms) { return g.n_sub() <= 2LL * sms; }
 
+struct Batch;
+
 struct asm_ctx {
     asm_options opt;
+    std::shared_ptr<Batch> kws;  // tables of the solves this handle leads
     cudaStream_t stream = nullptr;
     int device = 0;
     int prec = 0;
@@ -1179,6 +1182,11 @@ int factor_numeric(asm_ctx* h) {
 // ---------------------------------------------------------------------------------------------
 namespace {
 
+constexpr int kCtlRing = 4;   // control-word reads in flight
+constexpr int kRunAhead = 2;  // steps launched beyond the last one whose control words were seen
+
+}  // namespace
+
 struct Batch {
     std::vector<asm_ctx*> hs;
     DBuf d_tab, d_vec, d_row, d_box, d_sub, d_gather, d_ritems;
@@ -1199,15 +1207,24 @@ struct Batch {
     DBuf d_cbox, d_cgrow;   // coarse-correction work items of the systems that have one
     int ncbox = 0, ncgrow = 0;
     bool two_stage = false;
+    bool flexible = false;  // every system keeps its Z_k (no x += B^{-1} u at a restart)
     int coop_grid = 0;  // > 0: single system, orthogonalisation in one cooperative launch
     bool has_init = false;  // a system may be in its initial phase (serving: systems join mid-flight)
-    std::vector<int> host_ctl;
+    // control words of every system, kCtlRing reads in turn: gathered on the device (d_ctls), copied to
+    // pinned memory, an event behind each copy
+    DBuf d_ctls;
     int* pinned = nullptr;
     size_t pinned_cap = 0;
+    cudaEvent_t ctl_event[kCtlRing] = {};
+    int* ctl_slot(long long read) { return pinned + (size_t)(read % kCtlRing) * hs.size() * C_NCTL; }
     ~Batch() {
         if (pinned) cudaFreeHost(pinned);
+        for (cudaEvent_t e : ctl_event)
+            if (e) cudaEventDestroy(e);
     }
 };
+
+namespace {
 
 void build_batch(Batch& B, cudaStream_t st) {
     std::vector<SysTab> tabs;
@@ -1218,6 +1235,7 @@ void build_batch(Batch& B, cudaStream_t st) {
     for (int k = 0; k < (int)B.hs.size(); k++) {
         asm_ctx* h = B.hs[k];
         tabs.push_back(h->tab);
+        B.flexible = (k == 0 || B.flexible) && h->tab.flexible;
         for (int c = 0; c < h->nchunk; c++) vi.push_back(VecItem{k, c});
         for (int r = 0; r < h->N; r += 256) ri.push_back(RowItem{k, r});
         for (int j = 0; j < h->n_group_items; j++) {
@@ -1334,13 +1352,17 @@ void build_batch(Batch& B, cudaStream_t st) {
     B.nbox = (int)bi.size();
     B.nsub = (int)sd.size();
     // pinned control words: grown, never shrunk (pinning host memory is slow)
-    const size_t npin = std::max<size_t>(1, B.hs.size());
+    const size_t npin = std::max<size_t>(1, B.hs.size()) * kCtlRing;
     if (!B.pinned || B.pinned_cap < npin) {
         if (B.pinned) cudaFreeHost(B.pinned);
         B.pinned = nullptr;
         B.pinned_cap = npin + npin / 2;
         ck(cudaMallocHost((void**)&B.pinned, sizeof(int) * C_NCTL * B.pinned_cap));
     }
+    if (B.hs.size() > 1 && B.d_ctls.bytes < sizeof(int) * C_NCTL * B.hs.size())
+        B.d_ctls.alloc(2 * sizeof(int) * C_NCTL * B.hs.size());
+    for (cudaEvent_t& e : B.ctl_event)
+        if (!e) ck(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
 }
 
 // events bracketing the launch groups of one step: [prep | apply | post | spmv | mgs+finish]
@@ -1406,11 +1428,11 @@ void launch_step(Batch& B, int kmax, cudaStream_t st, StepEvents* ev) {
     launch_coarse_apply(tab, B.d_row.as<RowItem>(), B.nrow, B.d_cbox.as<BoxItem>(), B.ncbox, B.d_cgrow.as<RowItem>(),
                         B.ncgrow, vi, B.nvec, B.two_stage, st);
     if (ev) ck(cudaEventRecord(ev->e[2], st));
-    launch_post(tab, vi, B.nvec, st);
+    if (!B.flexible) launch_post(tab, vi, B.nvec, st);
     if (ev) ck(cudaEventRecord(ev->e[3], st));
     launch_spmv(tab, B.d_row.as<RowItem>(), B.nrow, st);
     if (ev) ck(cudaEventRecord(ev->e[4], st));
-    long long n = 4 + local_solve_launches(B);
+    long long n = (B.flexible ? 3 : 4) + local_solve_launches(B);
     if (B.coop_grid > 0) {
         ck(launch_ortho_coop(tab, B.hs[0]->d_partial.as<double>(), B.coop_grid, B.hs[0]->tab.ortho, B.hs[0]->tab.n3, st));
         n += 1;
@@ -1455,10 +1477,25 @@ float elapsed(cudaEvent_t a, cudaEvent_t b) {
     return ms;
 }
 
-void read_ctl(Batch& B, cudaStream_t st) {
-    for (size_t k = 0; k < B.hs.size(); k++)
-        ck(cudaMemcpyAsync(B.pinned + k * C_NCTL, B.hs[k]->d_ctl.p, sizeof(int) * C_NCTL, cudaMemcpyDeviceToHost, st));
-    ck(cudaStreamSynchronize(st));
+// Requests the control words of every system as read number `read` (one copy: a copy per system cost the host
+// ~3 us each), and waits for them
+void request_ctl(Batch& B, cudaStream_t st, long long read) {
+    const size_t bytes = sizeof(int) * C_NCTL * B.hs.size();
+    const void* src = B.hs[0]->d_ctl.p;
+    if (B.hs.size() > 1) {
+        launch_gather_ctl(B.d_tab.as<SysTab>(), (int)B.hs.size(), B.d_ctls.as<int>(), st);
+        src = B.d_ctls.p;
+    }
+    ck(cudaMemcpyAsync(B.ctl_slot(read), src, bytes, cudaMemcpyDeviceToHost, st));
+    ck(cudaEventRecord(B.ctl_event[read % kCtlRing], st));
+}
+const int* wait_ctl(Batch& B, long long read) {
+    ck(cudaEventSynchronize(B.ctl_event[read % kCtlRing]));
+    return B.ctl_slot(read);
+}
+const int* read_ctl(Batch& B, cudaStream_t st) {
+    request_ctl(B, st, 0);
+    return wait_ctl(B, 0);
 }
 
 // b into slot VB, control words (initial phase) and tolerance of one system
@@ -1475,8 +1512,8 @@ void begin_solve(asm_ctx* h, const double* b, int on_device, double rtol, int ma
     c[C_STATUS] = ASM_ERR_NOT_CONVERGED;
     ck(cudaMemcpyAsync(h->d_ctl.p, c, sizeof(c), cudaMemcpyHostToDevice, h->stream));
     double tol = rtol;
+    // (copies from pageable memory return once the source is staged: c and tol may go out of scope)
     ck(cudaMemcpyAsync(h->d_scal.as<double>() + SL.tol, &tol, sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    ck(cudaStreamSynchronize(h->stream));
 }
 
 // x and the result of a finished (or abandoned) system; c = its control words
@@ -1485,9 +1522,8 @@ int harvest(asm_ctx* h, const int* c, double* x, int on_device, asm_solve_info* 
     double sc[2];
     ck(cudaMemcpyAsync(sc, h->d_scal.as<double>() + SL.bnorm, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     copy_out(h, x, h->d_ws.as<double>() + (long long)VX * h->n3p, sizeof(double) * 3 * (size_t)h->N, on_device);
-    ck(cudaStreamSynchronize(h->stream));
     int status = c[C_PHASE] == PH_DONE ? c[C_STATUS] : ASM_ERR_NOT_CONVERGED;
-    if (take_dev_err(h)) status = ASM_ERR_TIMEOUT;
+    if (take_dev_err(h)) status = ASM_ERR_TIMEOUT;  // (waits for the copies above too)
     if (info) {
         info->iterations = c[C_ITERS];
         info->restarts = c[C_RESTARTS];
@@ -1502,8 +1538,16 @@ int harvest(asm_ctx* h, const int* c, double* x, int on_device, asm_solve_info* 
 int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const* x, double rtol, int max_iter,
               int on_device, asm_solve_info* infos) {
     cudaStream_t st = hs[0]->stream;
-    Batch B;
+    // the tables and pinned words of the last solve that this handle led: the next one reuses the allocations
+    if (!hs[0]->kws) hs[0]->kws = std::make_shared<Batch>();
+    Batch& B = *hs[0]->kws;
+    struct Leave {  // no other handle's pointer is kept
+        Batch& B;
+        ~Leave() { B.hs.clear(); }
+    } leave{B};
     B.hs = hs;
+    B.coop_grid = 0;
+    B.has_init = false;
     for (size_t k = 0; k < hs.size(); k++) begin_solve(hs[k], b[k], on_device, rtol, max_iter);
     build_batch(B, st);
     const bool om = hs[0]->opt.krylov == ASM_KRYLOV_ORTHOMIN;
@@ -1546,7 +1590,7 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
     bool graphs_ok = hs.size() > 1 && B.coop_grid == 0 && !prof && st != nullptr && !hs[0]->no_graphs;
     std::map<int, cudaGraphExec_t> graphs;
     std::map<int, long long> graph_launches;
-    std::set<int> seen;
+    std::set<int> run_once;
     auto plain_step = [&](int kmax, StepEvents* e) {
         if (om)
             launch_step_om(B, kmax, st, e);
@@ -1556,8 +1600,20 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
     bool pending = false;
     int pending_applies = 0;
     const int guard_steps = 4 * max_iter + 64;
+    // Read number s holds the control words before step s.  Steps are launched up to kRunAhead beyond the last
+    // read seen, so that the device does not wait for the host between them: the kernels take a step's
+    // phase from the device, and what the host chooses (the number of Gram-Schmidt or projection passes) is
+    // an upper bound for every state the systems may have reached; steps after the last are empty.  The
+    // profiler and the placement tuner time single steps and wait for each.
+    request_ctl(B, st, 0);
+    const int* words = nullptr;
+    long long seen = -1;
     for (int step = 0; step < guard_steps; step++) {
-        read_ctl(B, st);
+        const int ahead = prof || tune_next < tune_total || tune_at >= 0 ? 0 : kRunAhead;
+        if (step - ahead > seen) {
+            seen = step - ahead;
+            words = wait_ctl(B, seen);
+        }
         if (pending) {
             asm_profile_info& P = hs[0]->prof;
             P.ortho_ms += elapsed(ev.e[0], ev.e[1]) + elapsed(ev.e[2], ev.e[3]) + elapsed(ev.e[4], ev.e[5]);
@@ -1580,18 +1636,22 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
         }
         int kmax = -1;
         bool any = false;
+        const int lag = words ? (int)(step - seen) : step;  // steps launched since the words were read
         for (size_t k = 0; k < hs.size(); k++) {
-            const int* c = B.pinned + k * C_NCTL;
-            if (c[C_PHASE] == PH_DONE) continue;
+            const int* c = words ? words + k * C_NCTL : nullptr;
+            if (c && c[C_PHASE] == PH_DONE) continue;
             any = true;
-            if (c[C_PHASE] == PH_ARNOLDI) kmax = std::max(kmax, gs_passes(hs[k], c[C_J]));
-            else if (c[C_PHASE] == PH_OM) kmax = std::max(kmax, c[C_OM_STORED]);
-            else kmax = std::max(kmax, 0);
+            if (om)
+                kmax = std::max(kmax, std::min(hs[k]->ws_m, (c && c[C_PHASE] == PH_OM ? c[C_OM_STORED] : 0) + lag));
+            else if (c && c[C_PHASE] == PH_ARNOLDI)
+                kmax = std::max(kmax, gs_passes(hs[k], std::min(hs[k]->ws_m - 1, c[C_J] + lag)));
+            else
+                kmax = std::max(kmax, c && lag == 0 ? 0 : gs_passes(hs[k], std::min(hs[k]->ws_m - 1, lag)));
         }
         if (!any) break;
         pending_applies = 0;
-        for (size_t k = 0; k < hs.size(); k++) {
-            const int* c = B.pinned + k * C_NCTL;
+        for (size_t k = 0; words && k < hs.size(); k++) {
+            const int* c = words + k * C_NCTL;
             if (c[C_APPLY_IN] >= 0 && c[C_PHASE] != PH_DONE) pending_applies++;
         }
         if (tune_next < tune_total && pending_applies > 0) {
@@ -1601,7 +1661,7 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
             pending = prof;
         } else if (graphs_ok && tune_next >= tune_total) {
             auto it = graphs.find(kmax);
-            if (it == graphs.end() && seen.count(kmax)) {
+            if (it == graphs.end() && run_once.count(kmax)) {
                 // capture this step's launch sequence (its kernels were all launched once before)
                 const long long before = hs[0]->prof.kernel_launches;
                 cudaGraph_t g = nullptr;
@@ -1632,18 +1692,19 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
                 for (asm_ctx* h : hs) h->prof.kernel_launches += graph_launches[kmax];
             } else {
                 plain_step(kmax, nullptr);
-                seen.insert(kmax);
+                run_once.insert(kmax);
             }
         } else {
             plain_step(kmax, prof ? &ev : nullptr);
             pending = prof;
         }
+        request_ctl(B, st, step + 1);
     }
+    const int* end = read_ctl(B, st);
     for (auto& g : graphs) cudaGraphExecDestroy(g.second);
-    read_ctl(B, st);
     int worst = ASM_OK;
     for (size_t k = 0; k < hs.size(); k++) {
-        const int status = harvest(hs[k], B.pinned + k * C_NCTL, x[k], on_device, infos ? &infos[k] : nullptr);
+        const int status = harvest(hs[k], end + k * C_NCTL, x[k], on_device, infos ? &infos[k] : nullptr);
         if (status == ASM_ERR_TIMEOUT)
             worst = ASM_ERR_TIMEOUT;
         else if (status != ASM_OK && worst != ASM_ERR_TIMEOUT)
@@ -2865,11 +2926,11 @@ int asm_server_progress(asm_server_handle S, int max_steps, int* n_active, int* 
                 S->batch.has_init = true;
                 S->dirty = false;
             }
-            read_ctl(S->batch, S->stream);
+            const int* words = read_ctl(S->batch, S->stream);
             int kmax = -1;
             std::vector<Req*> keep;
             for (size_t k = 0; k < S->active.size(); k++) {
-                const int* c = S->batch.pinned + k * C_NCTL;
+                const int* c = words + k * C_NCTL;
                 if (c[C_PHASE] == PH_DONE) {
                     retire(S, S->active[k], c);
                     S->st.completed++;
@@ -2890,10 +2951,10 @@ int asm_server_progress(asm_server_handle S, int max_steps, int* n_active, int* 
                 build_batch(S->batch, S->stream);
                 S->batch.has_init = true;
                 S->dirty = false;
-                read_ctl(S->batch, S->stream);
+                words = read_ctl(S->batch, S->stream);
                 kmax = -1;
                 for (size_t k = 0; k < S->active.size(); k++) {
-                    const int* c = S->batch.pinned + k * C_NCTL;
+                    const int* c = words + k * C_NCTL;
                     if (c[C_PHASE] != PH_DONE)
                         kmax = std::max(kmax, c[C_PHASE] == PH_ARNOLDI ? gs_passes(S->active[k]->h, c[C_J]) : 0);
                 }

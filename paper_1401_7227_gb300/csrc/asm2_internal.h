@@ -314,6 +314,8 @@ ApplyConfig apply_local_vectors(int nsub, int all_bytes, int lump_bytes, int sme
 size_t apply_ring_bytes(int slots, int chunk);
 void launch_spmv(const SysTab* st_tab, const RowItem* items, int nitems, cudaStream_t st);
 
+// the control words of n systems, C_NCTL each, into out
+void launch_gather_ctl(const SysTab* tab, int n, int* out, cudaStream_t st);
 void launch_init(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);
 void launch_prep(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);
 void launch_post(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);

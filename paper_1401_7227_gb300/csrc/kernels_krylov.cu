@@ -123,6 +123,10 @@ __device__ bool finish_reduction(const SysTab& st, int chunk, double& s0, double
     return true;
 }
 
+__global__ void k_gather_ctl(const SysTab* __restrict__ tab, int* __restrict__ out) {
+    if (threadIdx.x < C_NCTL) out[blockIdx.x * C_NCTL + threadIdx.x] = tab[blockIdx.x].ctl[threadIdx.x];
+}
+
 __global__ void __launch_bounds__(VEC_THREADS) k_init(const SysTab* __restrict__ tab, const VecItem* __restrict__ items) {
     const VecItem it = items[blockIdx.x];
     const SysTab& st = tab[it.sys];
@@ -1283,6 +1287,9 @@ void launch_spmv(const SysTab* tab, const RowItem* items, int nitems, cudaStream
     if (nitems > 0) k_spmv<<<nitems, 256, 0, st>>>(tab, items);
 }
 
+void launch_gather_ctl(const SysTab* tab, int n, int* out, cudaStream_t st) {
+    if (n > 0) k_gather_ctl<<<n, 32, 0, st>>>(tab, out);
+}
 void launch_init(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st) {
     if (nitems > 0) k_init<<<nitems, VEC_THREADS, 0, st>>>(tab, items);
 }
