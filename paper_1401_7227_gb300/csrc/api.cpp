@@ -1416,6 +1416,9 @@ void launch_local_solves(Batch& B, const SysTab* tab, cudaStream_t st) {
 // index of the last Gram-Schmidt pass of a system's Arnoldi step j (one per block, one for the norm)
 int gs_passes(const asm_ctx* h, int j) { return (j + h->tab.gs_block) / h->tab.gs_block; }
 
+// index of the last pass of an ORTHOMIN step with that many stored directions
+int om_passes(int stored) { return (stored + kGsMaxBlock - 1) / kGsMaxBlock; }
+
 void launch_step(Batch& B, int kmax, cudaStream_t st, StepEvents* ev) {
     const SysTab* tab = B.d_tab.as<SysTab>();
     const VecItem* vi = B.d_vec.as<VecItem>();
@@ -1446,7 +1449,7 @@ void launch_step(Batch& B, int kmax, cudaStream_t st, StepEvents* ev) {
     for (asm_ctx* h : B.hs) h->prof.kernel_launches += n;
 }
 
-// One ORTHOMIN step of every system: [apply | mat-vec | projections 0..kmax + update], with the
+// One ORTHOMIN step of every system: [apply | mat-vec | projection passes 0..kmax + update], with the
 // events at the same places as a GMRES step (the prep and post groups are empty)
 void launch_step_om(Batch& B, int kmax, cudaStream_t st, StepEvents* ev) {
     const SysTab* tab = B.d_tab.as<SysTab>();
@@ -1642,7 +1645,7 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
             if (c && c[C_PHASE] == PH_DONE) continue;
             any = true;
             if (om)
-                kmax = std::max(kmax, std::min(hs[k]->ws_m, (c && c[C_PHASE] == PH_OM ? c[C_OM_STORED] : 0) + lag));
+                kmax = std::max(kmax, om_passes(std::min(hs[k]->ws_m, (c && c[C_PHASE] == PH_OM ? c[C_OM_STORED] : 0) + lag)));
             else if (c && c[C_PHASE] == PH_ARNOLDI)
                 kmax = std::max(kmax, gs_passes(hs[k], std::min(hs[k]->ws_m - 1, c[C_J] + lag)));
             else

@@ -104,7 +104,8 @@ struct ScalLayout {
         L.om_beta = o;  // ORTHOMIN: projection coefficients of the step in progress
         o += m;
         L.om_alpha = o++;
-        L.gram = o;  // (v_k, v_i) of the vectors i < k in k's Gram-Schmidt block, kGsMaxBlock per vector
+        L.gram = o;  // (v_k, v_i) of the vectors i < k in k's Gram-Schmidt block, kGsMaxBlock per vector;
+                     // ORTHOMIN: (Q_s, the direction d older), kGsMaxBlock distances d per ring slot
         o += (m + 1) * kGsMaxBlock;
         L.n = o;
         return L;
@@ -322,8 +323,6 @@ void launch_post(const SysTab* tab, const VecItem* items, int nitems, cudaStream
 // pass 0 .. number of Gram-Schmidt blocks of the step
 void launch_mgs(const SysTab* tab, const VecItem* items, int nitems, int pass, cudaStream_t st);
 void launch_finish(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);
-// ORTHOMIN(k): projection pass l of the direction in progress (l = 0 also reduces ||r|| of
-// initial systems and ||b - A x|| of finishing ones), then x += alpha p, r -= alpha q.
 // Dense matrices inverted in place by Gauss-Jordan elimination with partial pivoting: aug = [A | I]
 // (n x 2n, row-major), prow / fcol scratch of 2n / n doubles.
 struct GJMat {
@@ -355,7 +354,9 @@ int nf_apply_slots(int ndesc, int bx_max, int bz_max, int prec, int sm_smem, int
 void launch_nf_factor(const NFDesc* descs, int ndesc, int nmax, int prec, FactErr* err, cudaStream_t st);
 void launch_nf_apply(const SysTab* tab, const NFDesc* descs, int ndesc, int prec, int slots, size_t smem,
                      cudaStream_t st);
-void launch_om(const SysTab* tab, const VecItem* items, int nitems, int l, cudaStream_t st);
+// ORTHOMIN(k): pass 0 .. number of projection blocks of the direction in progress (pass 0 also reduces
+// ||r|| of initial systems and ||b - A x|| of finishing ones), then x += alpha p, r -= alpha q.
+void launch_om(const SysTab* tab, const VecItem* items, int nitems, int pass, cudaStream_t st);
 void launch_om_update(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);
 // Coarse-grid correction: [A_C | I] from the box-pair blocks, then in-place Gauss-Jordan (one
 // cooperative launch; *err = 1 + column of a zero pivot); and the per-apply kernels

@@ -364,6 +364,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_mgs(const SysTab* __restrict
         __syncthreads();
         const int rows = 2 * bs + 1;
         double* part = st.partial + (long long)it.chunk * rows;
+#pragma unroll 1
         for (int g0 = 0; g0 < max(1, nd); g0 += kGsGroup) {
             double acc[16], ww = 0.0;
 #pragma unroll
@@ -673,61 +674,168 @@ __device__ void om_state(const SysTab& st, int ph, double nrm) {
     om_set_slots(st, next);
 }
 
-// Pass l of a direction step: l >= 1 first applies projection l (p -= beta_l P_os, q -= beta_l Q_os,
-// os = the l-th most recent stored direction); then either the next coefficient
-// beta_{l+1} = (q, Q_os') / (Q_os', Q_os') or, after the last projection, (q, q) and (r, q).
+// Pass b of a direction step: the projections of block b - 1 are applied (p -= beta_l P_l, q -= beta_l Q_l, l the
+// l-th most recent stored direction, block b holding l = 32 b + 1 .. 32 b + 32), then the next block's coefficients
+// or, after the last block, (q, q) and (r, q).  Each beta_l belongs to the q that the projections before it have
+// already been subtracted from; within a block it follows from the products with the block's first q,
+//   beta_l = ((q, Q_l) - sum_{l' < l in block} beta_l' (Q_l', Q_l)) / (Q_l, Q_l),
+// so a block takes one reduction instead of one per direction.  The products (Q_l', Q_l) of directions less than a
+// block apart are kept: the newest direction's are taken in pass 0 of the step after its own, in the sweep that
+// reads the same vectors.  What bounded a step was its serial launches: at 30x30x9, k = 30, up to 31 of 15 us are
+// now three, and a solve of 29 steps takes 5.1 ms instead of 9.2.
 __global__ void __launch_bounds__(VEC_THREADS) k_om(const SysTab* __restrict__ tab, const VecItem* __restrict__ items,
-                                                    int l) {
+                                                    int b) {
     const VecItem it = items[blockIdx.x];
     const SysTab& st = tab[it.sys];
     if (st.krylov != 1) return;
     const int ph = st.ctl[C_PHASE];
-    const long long e0 = (long long)it.chunk * st.vchunk;
+    const long long e0 = (long long)it.chunk * st.vchunk, e1 = e0 + st.vchunk;
     const ScalLayout SL = ScalLayout::make(st.m);
-    double s0 = 0.0, s1 = 0.0;
     if (ph == PH_OM) {
-        const int stored = st.ctl[C_OM_STORED];
-        if (l > stored) return;
-        const int K1 = st.m + 1, slot = st.ctl[C_OM_SLOT];
+        constexpr int W = 2, kB = kGsMaxBlock, kL = 4, kRows = 2 * kB + 1;
+        __shared__ double hp[kB], sm[8 * 16], tot[kRows];
+        __shared__ long long prev_at[kB], next_at[kB];  // offsets of Q_l of the previous and of the next block
+        __shared__ bool last;
+        const int stored = st.ctl[C_OM_STORED], K1 = st.m + 1, slot = st.ctl[C_OM_SLOT];
+        const int lo = 1 + kB * b, plo = lo - kB;
+        if (plo > stored) return;
+        const int np = b > 0 ? min(kB, stored + 1 - plo) : 0, nd = max(0, min(kB, stored + 1 - lo));
+        const int ngram = b == 0 ? max(0, nd - 1) : 0;  // (Q_1, Q_l), l = 2 ..
+        const bool fin = nd == 0;
+        const auto dir = [&](int l) { return (slot - l + K1) % K1; };
         double* p = vec(st, om_p(st, slot));
         double* q = vec(st, om_q(st, slot));
-        if (l >= 1) {
-            const int os = (slot - l + K1) % K1;
-            const double beta = st.scal[SL.om_beta + l - 1];
-            const double* po = vec(st, om_p(st, os));
-            const double* qo = vec(st, om_q(st, os));
-            for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
-                p[e0 + i] -= beta * po[e0 + i];
-                q[e0 + i] -= beta * qo[e0 + i];
-            }
+        const double* newest = vec(st, om_q(st, dir(1)));
+        const double* r = vec(st, VR);
+        if ((int)threadIdx.x < np) {
+            hp[threadIdx.x] = st.scal[SL.om_beta + plo - 1 + threadIdx.x];
+            prev_at[threadIdx.x] = om_q(st, dir(plo + threadIdx.x)) * st.n3p;
         }
-        if (l < stored) {
-            const double* qo = vec(st, om_q(st, (slot - l - 1 + K1) % K1));
-            for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) s0 += q[e0 + i] * qo[e0 + i];
-        } else {
-            const double* r = vec(st, VR);
-            for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
-                const double a = q[e0 + i];
-                s0 += a * a;
-                s1 += r[e0 + i] * a;
+        if ((int)threadIdx.x < nd) next_at[threadIdx.x] = om_q(st, dir(lo + threadIdx.x)) * st.n3p;
+        const double* ws = st.ws;
+        const long long p_of_q = (long long)(om_p(st, 0) - om_q(st, 0)) * st.n3p;  // from Q_s to P_s
+        __syncthreads();
+        double* part = st.partial + (long long)it.chunk * kRows;
+        // (not unrolled: nvcc 13.0's full unroll of these up to four groups lost warp 0's share of a sum
+        // once a third group had one vector; a barrier on either side of cta_sums also cured it)
+#pragma unroll 1
+        for (int g0 = 0; g0 < max(1, nd); g0 += kGsGroup) {
+            const int nn = min(kGsGroup, nd - g0), ng = max(0, min(kGsGroup, 1 + ngram - g0));  // (entry 0: (Q_1, Q_1))
+            double acc[16], qq = 0.0, rq = 0.0;
+#pragma unroll
+            for (int k = 0; k < 16; k++) acc[k] = 0.0;
+#pragma unroll 1
+            for (long long e = e0 + W * threadIdx.x; e < e1; e += W * VEC_THREADS) {
+                double x[W], y[W];
+                load_w<W>(q + e, x);
+                if (g0 == 0 && np > 0) {
+                    double t[W];
+                    load_w<W>(p + e, t);
+#pragma unroll 1
+                    for (int i0 = 0; i0 < np; i0 += kL) {
+                        double cp[kL][W], cq[kL][W];
+#pragma unroll
+                        for (int d = 0; d < kL; d++)
+                            if (i0 + d < np) {
+                                const double* qo = ws + prev_at[i0 + d] + e;
+                                load_w<W>(qo + p_of_q, cp[d]);
+                                load_w<W>(qo, cq[d]);
+                            }
+#pragma unroll
+                        for (int d = 0; d < kL; d++)
+                            if (i0 + d < np) {
+                                const double h = hp[i0 + d];
+#pragma unroll
+                                for (int u = 0; u < W; u++) {
+                                    t[u] = fma(-h, cp[d][u], t[u]);
+                                    x[u] = fma(-h, cq[d][u], x[u]);
+                                }
+                            }
+                    }
+                    store_w<W>(p + e, t);
+                    store_w<W>(q + e, x);
+                }
+                if (fin) {
+                    load_w<W>(r + e, y);
+#pragma unroll
+                    for (int u = 0; u < W; u++) {
+                        qq = fma(x[u], x[u], qq);
+                        rq = fma(y[u], x[u], rq);
+                    }
+                } else {
+                    if (ng > 0) load_w<W>(newest + e, y);
+#pragma unroll
+                    for (int d0 = 0; d0 < kGsGroup; d0 += kL) {
+                        if (d0 >= nn) break;
+                        double v[kL][W];
+#pragma unroll
+                        for (int d = 0; d < kL; d++)
+                            if (d0 + d < nn) load_w<W>(ws + next_at[g0 + d0 + d] + e, v[d]);
+#pragma unroll
+                        for (int d = 0; d < kL; d++)
+                            if (d0 + d < nn)
+#pragma unroll
+                                for (int u = 0; u < W; u++) acc[d0 + d] = fma(x[u], v[d][u], acc[d0 + d]);
+#pragma unroll
+                        for (int d = 0; d < kL; d++)
+                            if (d0 + d < ng)
+#pragma unroll
+                                for (int u = 0; u < W; u++)
+                                    acc[kGsGroup + d0 + d] = fma(y[u], v[d][u], acc[kGsGroup + d0 + d]);
+                    }
+                }
             }
-        }
-        if (!finish_reduction(st, it.chunk, s0, s1)) return;
-        if (threadIdx.x == 0) {
-            if (l < stored) {
-                const int on = (slot - l - 1 + K1) % K1;
-                st.scal[SL.om_beta + l] = s0 / st.scal[SL.om_qq + on];
+            const int t = threadIdx.x;
+            if (fin) {
+                block_sum2(qq, rq);
+                if (t == 0) {
+                    part[0] = qq;
+                    part[1] = rq;
+                }
             } else {
-                st.scal[SL.om_qq + slot] = s0;
-                st.scal[SL.om_alpha] = s0 != 0.0 ? s1 / s0 : 0.0;
+                const double v = ng > 0 ? cta_sums<16>(acc, sm) : cta_sums<8>(acc, sm);
+                if (t < nn) part[g0 + t] = v;
+                if (t >= kGsGroup && t < kGsGroup + ng) part[kB + g0 + t - kGsGroup] = v;
             }
         }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            last = atomicAdd(&st.ctl[C_CNT_RED], 1) == st.nchunk - 1;
+        }
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (threadIdx.x == 0) st.ctl[C_CNT_RED] = 0;
+        gs_totals(st.partial, 1, kRows, st.nchunk, fin ? 2 : nd, fin || b > 0 ? 0 : 1 + ngram, false, kB, tot);
+        __syncthreads();
+        if (fin) {
+            if (threadIdx.x == 0) {
+                st.scal[SL.om_qq + slot] = tot[0];
+                st.scal[SL.om_alpha] = tot[0] != 0.0 ? tot[1] / tot[0] : 0.0;
+            }
+            return;
+        }
+        if (threadIdx.x >= 32) return;
+        // lane i: beta of l = lo + i
+        const int i = threadIdx.x;
+        double* gram = st.scal + SL.gram;  // entry (slot, distance): the product with the direction that much older
+        if (b == 0 && i >= 1 && i < nd) gram[dir(1) * kB + i] = tot[nd + i];
+        __syncwarp();
+        double c = i < nd ? tot[i] : 0.0;
+        const double inv = i < nd ? 1.0 / st.scal[SL.om_qq + dir(lo + i)] : 0.0;
+        for (int k = 0; k + 1 < nd; k++) {
+            const double beta = __shfl_sync(0xffffffffu, c * inv, k);
+            if (i > k && i < nd) c = fma(-gram[dir(lo + k) * kB + i - k], beta, c);
+        }
+        if (i < nd) st.scal[SL.om_beta + lo - 1 + i] = c * inv;
     } else if (ph == PH_INIT || ph == PH_OM_FINAL) {
-        if (l != 0) return;
+        if (b != 0) return;
         const double* r = vec(st, ph == PH_INIT ? VR : VW);
+        double s0 = 0.0, s1 = 0.0;
         for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
             const double a = r[e0 + i];
-            s0 += a * a;
+            s0 = fma(a, a, s0);
         }
         if (!finish_reduction(st, it.chunk, s0, s1)) return;
         if (threadIdx.x == 0) om_state(st, ph, sqrt(s0));
@@ -1327,8 +1435,8 @@ cudaError_t launch_ortho_coop(const SysTab* tab, double* part2, int grid, int or
     return cudaLaunchCooperativeKernel(ortho_kernel(ortho, n3), dim3(grid), dim3(VEC_THREADS), args, 0, st);
 }
 
-void launch_om(const SysTab* tab, const VecItem* items, int nitems, int l, cudaStream_t st) {
-    if (nitems > 0) k_om<<<nitems, VEC_THREADS, 0, st>>>(tab, items, l);
+void launch_om(const SysTab* tab, const VecItem* items, int nitems, int pass, cudaStream_t st) {
+    if (nitems > 0) k_om<<<nitems, VEC_THREADS, 0, st>>>(tab, items, pass);
 }
 void launch_om_update(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st) {
     if (nitems > 0) k_om_update<<<nitems, VEC_THREADS, 0, st>>>(tab, items);

@@ -68,3 +68,22 @@ def test_both_sides_of_the_short_vector_limit(grid):
         assert i["converged"] and np.linalg.norm(r) <= 1e-8 * (1 + 1e-6) * np.linalg.norm(s.b)
     assert i1["iterations"] == i2["iterations"]
     assert np.linalg.norm(x1 - x2) <= 1e-8 * np.linalg.norm(x2)
+
+
+@pytest.mark.parametrize("k", [31, 32, 33, 40])
+def test_orthomin_over_block_edges(k):
+    """45 ORTHOMIN(k) steps of a slowly converging system: the ring wraps, and the stored directions fill one
+    block of 32, one more, and a second.  The iterate and the residual are the oracle's within 1e-8."""
+    g = O.Geometry(24, 24, 8, 12, 12, 4, ov=0, near_width=0, far_mode=0)
+    s = synth.grid_jacobian(24, 24, 8, 3)
+    pc = O.Precond(g, s.row_ptr, s.col_idx, s.vals)
+    xo, oi = O.orthomin(s.row_ptr, s.col_idx, s.vals, s.b, pc, k, 1e-8, 45)
+    sol = asm2.Solver(precision="fp64", restart=k, krylov="orthomin")
+    sol.set_grid(24, 24, 8)
+    sol.set_matrix(s.row_ptr, s.col_idx, s.vals)
+    sol.set_partition(12, 12, 4, 0, 0, (2, 2, 2), "none")
+    sol.factor()
+    x, info = sol.solve(s.b, 1e-8, 45)
+    assert not oi.converged and info["status"] == 4 and info["iterations"] == 45 == oi.iters
+    assert np.linalg.norm(x - xo) <= 1e-8 * np.linalg.norm(xo)
+    assert abs(info["rel_residual"] - oi.relres) <= 1e-8 * oi.relres
