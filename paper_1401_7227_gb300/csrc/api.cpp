@@ -1119,8 +1119,8 @@ int factor_numeric(asm_ctx* h) {
     } else if (is_nf(h)) {
         int nmax = 0;
         for (const NFDesc& d : h->nf_desc) nmax = std::max(nmax, d.n);
-        launch_nf_factor(h->d_nfdesc1.as<NFDesc>(), (int)h->nf_desc.size(), nmax, h->prec, h->d_err.as<FactErr>(),
-                         h->stream);
+        launch_nf_factor(h->d_nfdesc1.as<NFDesc>(), (int)h->nf_desc.size(), nmax, h->nf_bz_max, h->prec, h->dev_smem,
+                         h->d_err.as<FactErr>(), h->stream);
     } else {
         launch_factor(h->d_factdesc.as<FactDesc>(), (int)S.subs.size(), h->d_err.as<FactErr>(), nullptr, h->stream);
         if (h->lanes_ok) {

@@ -6,10 +6,11 @@
 // of L2 T^{-1} U2 and L3 P^{-1} U3 (Eq. A.7).
 //
 // Both the factorisation and the solve are sequential along the cells of a subdomain: every line
-// depends on the previous line of its plane, every plane on the previous plane.  So one warp takes
-// one subdomain.  In the factorisation its lanes share the 3x3 block algebra (lane 3 r + c holds
-// element (r, c) of a block) and the independent per-cell products.  The apply streams one packet
-// per line -- G^{-1}, G^{-1} L1, G^{-1} U1, their two-step products, L2, L3, U3, U2 of the line's
+// depends on the previous line of its plane, every plane on the previous plane.  So one CTA takes
+// one subdomain: in the factorisation one of its warps runs the recurrences of a line (FP64 and the
+// 3x3 block algebra of G: lane 3 r + c holds element (r, c) of a block), the others fetch the next
+// line's operands, and all share the independent per-cell products.  The apply (one warp) streams one
+// packet per line -- G^{-1}, G^{-1} L1, G^{-1} U1, their two-step products, L2, L3, U3, U2 of the line's
 // cells, packed after the factorisation -- through a shared-memory ring of 2-4 slots by bulk copies,
 // ahead of the line being solved.  The products that do not depend on the line recurrences run on
 // all lanes; the two recurrences of T^{-1}, with one level of recursive doubling, run from shared
@@ -71,264 +72,291 @@ __device__ __forceinline__ bool binv(TC a, TC& inv, int lane) {
     return true;
 }
 
+// Working buffers of a line: bz blocks each, a block's rows LayF<TC>::RS values apart (FP32 pads a row
+// to four values, so that it is one 16-byte access).  Fixed ones, then per stage the operands of a line.
+enum { NB_N = 0, NB_K, NB_GI, NB_RHS, NB_VT, NB_W, NB_CS2, NB_G, NB_FIXED };
+enum { ST_SRC = 0, ST_POST, ST_N, ST_K, ST_GI, ST_MX };   // of a line of a plane solve
+enum { ST_D = 2, ST_L1, ST_U1, ST_C3, ST_FIELDS };         // of a line being factorised (with ST_SRC, ST_POST)
+
 template <typename TC>
-struct NFView {
-    const NFDesc& d;
-    TC* nk;  // N_p = G_p^{-1} U1_p ([9 n]), then K_p = L1_{p+1} G_p^{-1} ([9 n])
-    __device__ const TC* band(int k, int p) const { return static_cast<const TC*>(d.fband) + 9LL * (BD_N * p + k); }
-    __device__ const double* gi(int p) const { return d.gi + 9LL * p; }
-    __device__ const TC* N(int p) const { return nk + 9LL * p; }
-    __device__ const TC* K(int p) const { return nk + 9LL * (d.n + p); }
+struct LayF {
+    static constexpr int RS = sizeof(TC) == 4 ? 4 : 3, BS = 3 * RS;
 };
 
-// element `lane` of a block (lanes 9..31: zero)
-template <typename TC, typename TS>
-__device__ __forceinline__ TC ld(const TS* p, int lane) { return lane < 9 ? (TC)p[lane] : TC(0); }
-
-// W = u T^{-1} on the line starting at cell q0: W (G + L1)(I + G^{-1} U1) = u (rows of blocks).
-// With N_q = G_q^{-1} U1_q and K_q = L1_{q+1} G_q^{-1} (formed once per line after its G), each
-// sequential step is one block product:
-//   forward   v_q = u_q - v_{q-1} N_{q-1}            (v (I + G^{-1} U1) = u)
-//   backward  W_q = v_q G_q^{-1} - W_{q+1} K_q       (W (G + L1) = v; v_q G_q^{-1} on all lanes first)
-// The operands come from device memory (L2) at ~400 cycles, against ~50 cycles of arithmetic per
-// FP32 step, so the chains take them kRowG steps at a time into one of two register buffers, the
-// next group's loads issued before the current group is computed.  An FP64 step takes ~300 cycles,
-// so four steps cover the load latency, and the smaller buffers keep k_nf_factor<double> free of
-// register spills (eight: 255 registers and 92 bytes spilled; four: 233 registers, none, and the
-// FP64 re-factor 12% faster at 1M cells).
-template <typename TC>
-__device__ void line_row_solve(const NFView<TC>& v, int q0, const TC* u, TC* vtmp, TC* W, int lane) {
-    constexpr int kRowG = sizeof(TC) == 8 ? 4 : 8;
-    const int bz = v.d.bz;
-    {
-        TC a[2][kRowG], b[2][kRowG];  // u_q, N_{q-1}
-        TC prev = 0;
-#define NF_LOAD_F(h, gs)                                                            \
-    _Pragma("unroll") for (int i = 0; i < kRowG; i++) {                             \
-        const int q = (gs) + i;                                                     \
-        a[h][i] = q < bz ? ld<TC>(u + 9 * q, lane) : TC(0);                         \
-        b[h][i] = q > 0 && q < bz ? ld<TC>(v.N(q0 + q - 1), lane) : TC(0);          \
-    }
-        NF_LOAD_F(0, 0)
-        for (int g0 = 0; g0 < bz; g0 += 2 * kRowG) {
+// Rows of blocks along a line, one block product a step: x_0 = s_0, x_i = s_i - x_{i-1} A_i, where step i is
+// cell first + dir i and A_i the block of that cell + mo.  Warp 0; dst may be src.
+// FP32: three lanes, one row each, the row in registers: a step is the four dependent operations of the
+// product (16 cycles), its operands loaded three steps ahead; with one element per lane the row has to
+// go round by shuffles (~45 cycles).
+__device__ __forceinline__ void chain_rows(const float* src, const float* A, int mo, float* dst, int bz, int first, int dir,
+                                           int lane) {
+    if (lane >= 3) return;
+    const float4* s4 = reinterpret_cast<const float4*>(src) + lane;
+    const float4* a4 = reinterpret_cast<const float4*>(A);
+    float4* d4 = reinterpret_cast<float4*>(dst) + lane;
+    float4 c[4], m[4][3];
+    // steps past the end read the last one's operands again, and step 0 multiplies a zero row: no branch in
+    // the ring, whose slots then stay in registers
+    const auto load = [&](int i, int k) {
+        const int j = min(i, bz - 1), q = first + dir * j, qa = j > 0 ? q + mo : first;
+        c[k] = s4[3 * q];
+        m[k][0] = a4[3 * qa];
+        m[k][1] = a4[3 * qa + 1];
+        m[k][2] = a4[3 * qa + 2];
+    };
 #pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int gs = g0 + h * kRowG;
-                if (gs < bz) {
-                    if (gs + kRowG < bz) {
-                        if (h == 0) {
-                            NF_LOAD_F(1, gs + kRowG)
-                        } else {
-                            NF_LOAD_F(0, gs + kRowG)
-                        }
-                    }
+    for (int i = 0; i < 3; i++) load(i, i);
+    float x0 = 0.f, x1 = 0.f, x2 = 0.f;
+#pragma unroll 1
+    for (int i0 = 0; i0 < bz; i0 += 4) {
 #pragma unroll
-                    for (int i = 0; i < kRowG; i++) {
-                        const int q = gs + i;
-                        if (q < bz) {
-                            TC x = a[h][i];
-                            if (q > 0) x -= bmul(prev, b[h][i], lane);
-                            if (lane < 9) vtmp[9 * q + lane] = x;
-                            prev = x;
-                        }
-                    }
-                }
-            }
+        for (int k = 0; k < 4; k++) {
+            load(i0 + k + 3, (k + 3) & 3);
+            const float y0 = c[k].x - (x0 * m[k][0].x + x1 * m[k][1].x + x2 * m[k][2].x);
+            const float y1 = c[k].y - (x0 * m[k][0].y + x1 * m[k][1].y + x2 * m[k][2].y);
+            const float y2 = c[k].z - (x0 * m[k][0].z + x1 * m[k][1].z + x2 * m[k][2].z);
+            x0 = y0;
+            x1 = y1;
+            x2 = y2;
+            if (i0 + k < bz) d4[3 * (first + dir * (i0 + k))] = make_float4(x0, x1, x2, 0.f);
         }
-#undef NF_LOAD_F
     }
-    __syncwarp();
-    // v_q G_q^{-1}, one block element per lane, kB elements' loads in flight per lane
-    constexpr int kB = 4;
-    for (int t0 = lane; t0 < 9 * bz; t0 += 32 * kB) {
-        TC av[kB][3], gv[kB][3];
-#pragma unroll
-        for (int j = 0; j < kB; j++) {
-            const int t = t0 + 32 * j, q = t / 9, e = t - 9 * q, r = e / 3, k = e - 3 * r;
-            const bool in = t < 9 * bz;
-            const TC* a = vtmp + 9 * (in ? q : 0);
-            const double* g = v.gi(q0 + (in ? q : 0));
-#pragma unroll
-            for (int m = 0; m < 3; m++) {
-                av[j][m] = a[3 * r + m];
-                gv[j][m] = (TC)g[3 * m + k];
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < kB; j++)
-            if (t0 + 32 * j < 9 * bz) W[t0 + 32 * j] = av[j][0] * gv[j][0] + av[j][1] * gv[j][1] + av[j][2] * gv[j][2];
-    }
-    __syncwarp();
-    {
-        TC a[2][kRowG], b[2][kRowG];  // (v G^{-1})_q, K_q, for q = bz - 1 - (step)
-        TC next = 0;
-#define NF_LOAD_B(h, gs)                                                            \
-    _Pragma("unroll") for (int i = 0; i < kRowG; i++) {                             \
-        const int q = bz - 1 - ((gs) + i);                                          \
-        a[h][i] = q >= 0 ? ld<TC>(W + 9 * q, lane) : TC(0);                         \
-        b[h][i] = q >= 0 && q < bz - 1 ? ld<TC>(v.K(q0 + q), lane) : TC(0);         \
-    }
-        NF_LOAD_B(0, 0)
-        for (int g0 = 0; g0 < bz; g0 += 2 * kRowG) {
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int gs = g0 + h * kRowG;
-                if (gs < bz) {
-                    if (gs + kRowG < bz) {
-                        if (h == 0) {
-                            NF_LOAD_B(1, gs + kRowG)
-                        } else {
-                            NF_LOAD_B(0, gs + kRowG)
-                        }
-                    }
-#pragma unroll
-                    for (int i = 0; i < kRowG; i++) {
-                        const int q = bz - 1 - (gs + i);
-                        if (q >= 0) {
-                            TC x = a[h][i];
-                            if (q < bz - 1) x -= bmul(next, b[h][i], lane);
-                            if (lane < 9) W[9 * q + lane] = x;
-                            next = x;
-                        }
-                    }
-                }
-            }
-        }
-#undef NF_LOAD_B
-    }
-    __syncwarp();
 }
-
-// Independent block operations over n cells, one block element per lane and step (all 32 lanes):
-// dst_c = src_c - A_c B_c (SUB), dst_c = A_c B_c, or dst_c = src_c (no product); src, A, B give
-// each cell's block (src may be null: zero)
-template <bool SUB, typename TC, typename FS, typename FA, typename FB>
-__device__ __forceinline__ void blocks(TC* dst, int n, FS src, FA A, FB B, int lane) {
-    for (int t = lane; t < 9 * n; t += 32) {
-        const int c = t / 9, e = t - 9 * c, r = e / 3, k = e - 3 * r;
-        const TC* a = A(c);
-        const TC* b = B(c);
-        const TC* s0 = src(c);
-        TC v = 0;
-        if (a && b) v = a[3 * r] * b[k] + a[3 * r + 1] * b[3 + k] + a[3 * r + 2] * b[6 + k];
-        if (SUB) v = (s0 ? s0[e] : TC(0)) - v;
-        dst[9 * c + e] = v;
-    }
-    __syncwarp();
-}
-
-// W = u P^{-1} on the plane starting at c0 (rows of blocks); scratch: vb (9 S), x, y, vt (9 bz each)
-template <typename TC>
-__device__ void plane_row_solve(const NFView<TC>& v, int c0, const TC* u, TC* vb, TC* x, TC* y, TC* vt, TC* W,
-                                int lane) {
-    const int bz = v.d.bz, bx = v.d.bx;
-    const auto none = [](int) -> const TC* { return nullptr; };
-    for (int l = 0; l < bx; l++) {  // vb (I + T^{-1} U2) = u: vb_l = u_l - (vb_{l-1} T_{l-1}^{-1}) U2_{l-1}
-        const int cl = l * bz;
-        if (l > 0) {
-            line_row_solve(v, c0 + cl - bz, vb + 9 * (cl - bz), vt, x, lane);
-            blocks<true>(vb + 9 * cl, bz, [&](int q) { return u + 9 * (cl + q); }, [&](int q) { return x + 9 * q; },
-                         [&](int q) { return v.band(BD_U2, c0 + cl - bz + q); }, lane);
-        } else {
-            blocks<true>(vb, bz, [&](int q) { return u + 9 * q; }, none, none, lane);
+// FP64: nine lanes, one element each (an FP64 instruction holds the unit ~64 cycles for one lane as for 32)
+__device__ __forceinline__ void chain_rows(const double* src, const double* A, int mo, double* dst, int bz, int first, int dir,
+                                           int lane) {
+    const int e = lane < 9 ? lane : 0, r = e / 3, col = e - 3 * r;
+    double x = 0.0, c = src[9 * first + e], m = 0.0;
+#pragma unroll 1
+    for (int i = 0; i < bz; i++) {
+        const int q = first + dir * i;
+        const double y = c, b = m;
+        if (i + 1 < bz) {
+            c = src[9 * (q + dir) + e];
+            m = A[9 * (q + dir + mo) + e];
         }
-    }
-    for (int l = bx - 1; l >= 0; l--) {  // W (T + L2) = vb: W_l = (vb_l - W_{l+1} L2_{l+1}) T_l^{-1}
-        const int cl = l * bz;
-        if (l < bx - 1)
-            blocks<true>(y, bz, [&](int q) { return vb + 9 * (cl + q); }, [&](int q) { return W + 9 * (cl + bz + q); },
-                         [&](int q) { return v.band(BD_L2, c0 + cl + bz + q); }, lane);
-        else
-            blocks<true>(y, bz, [&](int q) { return vb + 9 * (cl + q); }, none, none, lane);
-        line_row_solve(v, c0 + cl, y, vt, W + 9 * cl, lane);
+        const double a0 = __shfl_sync(kFull, x, 3 * r), a1 = __shfl_sync(kFull, x, 3 * r + 1),
+                     a2 = __shfl_sync(kFull, x, 3 * r + 2);
+        const double b0 = __shfl_sync(kFull, b, col), b1 = __shfl_sync(kFull, b, 3 + col), b2 = __shfl_sync(kFull, b, 6 + col);
+        x = i > 0 ? fma(-a2, b2, fma(-a1, b1, fma(-a0, b0, y))) : y;
+        if (lane < 9) dst[9 * q + e] = x;
     }
 }
 
-// Factorisation in the compute type TC: G and G^{-1} (stored in FP64) of every cell, plane by
-// plane, line by line, cell by cell
+// f(cell, row, column, padded element offset) for each element of a line's blocks, by the threads [t0, t0 + nt)
+template <typename TC, typename F>
+__device__ __forceinline__ void elements(int bz, int t0, int nt, F f) {
+#pragma unroll 2
+    for (int t = (int)threadIdx.x - t0; t < 9 * bz; t += nt) {
+        const int q = t / 9, e = t - 9 * q, r = e / 3, c = e - 3 * r;
+        f(t, q, r, c, LayF<TC>::BS * q + LayF<TC>::RS * r + c);
+    }
+}
+
+// element (r, c) of A B for blocks of working buffers
 template <typename TC>
-__global__ void __launch_bounds__(128) k_nf_factor(const NFDesc* __restrict__ descs, int ndesc, FactErr* err) {
-    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (w >= ndesc) return;
-    const NFDesc d = descs[w];  // by value: its fields stay in registers across the stores
-    const int bz = d.bz, bx = d.bx, by = d.by, S = bz * bx;
-    // scratch: cs3 (9 S), u (9 S), W (9 S), vb (9 S), x, y, vt, cs2 (9 bz each), N and K (9 n each)
+__device__ __forceinline__ TC prod(const TC* a, const TC* b, int r, int c) {
+    constexpr int RS = LayF<TC>::RS;
+    return a[RS * r] * b[c] + a[RS * r + 1] * b[RS + c] + a[RS * r + 2] * b[2 * RS + c];
+}
+
+// Factorisation in the compute type TC: G and G^{-1} (stored in FP64) of every cell, plane by plane, line by
+// line, cell by cell, and with colsum, before each plane j > 0, cs3 = the block column sums of
+// L3 P_{j-1}^{-1} U3, from W = u P^{-1} with u = L3 (a row of blocks):
+//   vb (I + T^{-1} U2) = u:  vb_l = u_l - (vb_{l-1} T_{l-1}^{-1}) U2_{l-1}
+//   W (T + L2) = vb:         W_l = (vb_l - W_{l+1} L2_{l+1}) T_l^{-1}
+// and before each line l > 0 cs2 = those of L2 T_{l-1}^{-1} U2.  W = u T^{-1} on a line
+// (W (G + L1)(I + G^{-1} U1) = u) with N_q = G_q^{-1} U1_q and K_q = L1_{q+1} G_q^{-1} is
+//   forward   v_q = u_q - v_{q-1} N_{q-1}
+//   backward  W_q = v_q G_q^{-1} - W_{q+1} K_q       (v_q G_q^{-1} for all cells first)
+//
+// Serial along the cells of a subdomain: what bounds it is the latency of a step of a line's two recurrences
+// and of G's own.  A CTA per subdomain keeps a line's operands in shared memory: warp 0 runs the
+// recurrences while the other warps fetch the next line's operands into the second stage, and the
+// products of independent cells go over all threads.  With one warp per subdomain and the operands in device
+// memory, 64 boxes of 12 x 12 x 32 cells with column sums took 8.4 ms (FP32; FP64 15.5, FP32 boxes of
+// 4 x 3 x 150 1.77), now 2.6 (9.8, 0.55), the same FP32 bits; half of what is left is G's recurrence.
+// `stages` 2, or 1 (no overlap of the fetch) for lines whose two stages do not fit.
+constexpr int kNfThreads = 256;
+
+template <typename TC>
+__global__ void __launch_bounds__(kNfThreads) k_nf_factor(const NFDesc* __restrict__ descs, int stages, FactErr* err) {
+    constexpr int BS = LayF<TC>::BS, RS = LayF<TC>::RS;
+    extern __shared__ __align__(16) unsigned char nf_smem[];
+    __shared__ bool bad;
+    const NFDesc d = descs[blockIdx.x];  // by value: its fields stay in registers across the stores
+    const int bz = d.bz, bx = d.bx, by = d.by, S = bz * bx, lane = threadIdx.x & 31;
+    const bool seq = threadIdx.x < 32;
+    // device scratch: cs3 and vb (9 S each), N, K and (FP32) G^{-1} (9 n each)
     TC* cs3 = reinterpret_cast<TC*>(d.work);
-    const NFView<TC> v{d, cs3 + 36 * S + 36 * bz};
-    TC* u = cs3 + 9 * S;
-    TC* W = u + 9 * S;
-    TC* vb = W + 9 * S;
-    TC* x = vb + 9 * S;
-    TC* y = x + 9 * bz;
-    TC* vt = y + 9 * bz;
-    TC* cs2 = vt + 9 * bz;
+    TC* vb = cs3 + 9 * S;
+    TC* gn = vb + 9 * S;
+    TC* gk = gn + 9LL * d.n;
+    TC* gg = sizeof(TC) == 8 ? reinterpret_cast<TC*>(d.gi) : gk + 9LL * d.n;
+    TC* const buf = reinterpret_cast<TC*>(nf_smem);
+    const auto fix = [&](int f) { return buf + (long long)f * BS * bz; };
+    const auto st = [&](int b, int f) { return buf + (long long)(NB_FIXED + ST_FIELDS * b + f) * BS * bz; };
+    const TC* fband = static_cast<const TC*>(d.fband);
+    const auto band = [&](int k, int q0, int t, int q) { return fband[9LL * (BD_N * (q0 + q) + k) + t - 9 * q]; };
+    if (threadIdx.x == 0) bad = false;
+
+    // operands of line solve i of the solve with plane j - 1 (forward lines 0 .. bx-1, back to 0)
+    const auto stage_plane = [&](int j, int i, int b, int t0, int nt) {
+        const int c0 = (j - 1) * S, l = i < bx ? i : 2 * bx - 2 - i, p0 = c0 + l * bz;
+        TC *sn = st(b, ST_N), *sk = st(b, ST_K), *sg = st(b, ST_GI), *ss = st(b, ST_SRC), *sm = st(b, ST_MX),
+           *sp = st(b, ST_POST);
+        elements<TC>(bz, t0, nt, [&](int t, int q, int, int, int o) {
+            const TC n = gn[9LL * p0 + t], k = gk[9LL * p0 + t], g = gg[9LL * p0 + t];
+            const TC s = i < bx ? band(BD_L3, c0 + S + l * bz, t, q) : vb[9 * l * bz + t];
+            const TC m = i == 0 ? TC(0) : i < bx ? band(BD_U2, p0 - bz, t, q) : band(BD_L2, p0 + bz, t, q);
+            const TC u = i >= bx - 1 ? band(BD_U3, p0, t, q) : TC(0);
+            sn[o] = n;
+            sk[o] = k;
+            sg[o] = g;
+            ss[o] = s;
+            sm[o] = m;
+            sp[o] = u;
+        });
+    };
+    // operands of line l of plane j
+    const auto stage_line = [&](int j, int l, int b, bool line_term, bool plane_term, int t0, int nt) {
+        const int p0 = j * S + l * bz;
+        TC *sd = st(b, ST_D), *s1 = st(b, ST_L1), *u1 = st(b, ST_U1), *ss = st(b, ST_SRC), *sp = st(b, ST_POST), *c3 = st(b, ST_C3);
+        elements<TC>(bz, t0, nt, [&](int t, int q, int, int, int o) {
+            const TC a = band(BD_D, p0, t, q), b1 = band(BD_L1, p0, t, q), c = band(BD_U1, p0, t, q);
+            const TC s = line_term ? band(BD_L2, p0, t, q) : TC(0), u = line_term ? band(BD_U2, p0 - bz, t, q) : TC(0);
+            const TC e = plane_term ? cs3[9 * l * bz + t] : TC(0);
+            sd[o] = a;
+            s1[o] = b1;
+            u1[o] = c;
+            ss[o] = s;
+            sp[o] = u;
+            c3[o] = e;
+        });
+    };
+    // NB_W = u T^{-1}; `meanwhile` runs on the other warps during the forward recurrence
+    const auto line_solve = [&](const TC* u, const TC* N, const TC* K, const TC* GI, auto meanwhile) {
+        TC *v = fix(NB_VT), *W = fix(NB_W);
+        if (seq)
+            chain_rows(u, N, -1, v, bz, 0, 1, lane);
+        else
+            meanwhile();
+        __syncthreads();
+        elements<TC>(bz, 0, kNfThreads, [&](int, int q, int r, int c, int o) { W[o] = prod(v + BS * q, GI + BS * q, r, c); });
+        __syncthreads();
+        if (seq) chain_rows(W, K, 0, W, bz, bz - 1, -1, lane);
+        __syncthreads();
+    };
+
     for (int j = 0; j < by; j++) {
-        const int c0 = j * S;
         const bool plane_term = d.colsum && j > 0;
-        const auto none = [](int) -> const TC* { return nullptr; };
-        if (plane_term) {  // block column sums of L3 P_{j-1}^{-1} U3 on plane j
-            blocks<true>(u, S, [&](int c) { return v.band(BD_L3, c0 + c); }, none, none, lane);
-            plane_row_solve(v, c0 - S, u, vb, x, y, vt, W, lane);
-            blocks<false>(cs3, S, none, [&](int c) { return W + 9 * c; }, [&](int c) { return v.band(BD_U3, c0 - S + c); },
-                          lane);
+        if (plane_term) {
+            stage_plane(j, 0, 0, 0, kNfThreads);
+            __syncthreads();
+            for (int i = 0; i < 2 * bx - 1; i++) {
+                const int b = stages == 2 ? i & 1 : 0, l = i < bx ? i : 2 * bx - 2 - i;
+                TC *rhs = fix(NB_RHS), *W = fix(NB_W);
+                const TC *src = st(b, ST_SRC), *mx = st(b, ST_MX), *post = st(b, ST_POST);
+                elements<TC>(bz, 0, kNfThreads, [&](int t, int q, int r, int c, int o) {
+                    TC v = src[o];
+                    if (i > 0) v -= prod(W + BS * q, mx + BS * q, r, c);
+                    rhs[o] = v;
+                    if (i < bx - 1) vb[9 * l * bz + t] = v;
+                });
+                __syncthreads();
+                line_solve(rhs, st(b, ST_N), st(b, ST_K), st(b, ST_GI), [&] {
+                    if (stages == 2 && i + 1 < 2 * bx - 1) stage_plane(j, i + 1, b ^ 1, 32, kNfThreads - 32);
+                });
+                if (i >= bx - 1)
+                    elements<TC>(bz, 0, kNfThreads, [&](int t, int q, int r, int c, int) {
+                        cs3[9 * l * bz + t] = prod(W + BS * q, post + BS * q, r, c);
+                    });
+                if (stages != 2 && i + 1 < 2 * bx - 1) {
+                    __syncthreads();
+                    stage_plane(j, i + 1, 0, 0, kNfThreads);
+                    __syncthreads();
+                }
+            }
+            __syncthreads();
         }
+        stage_line(j, 0, 0, false, plane_term, 0, kNfThreads);
+        __syncthreads();
         for (int l = 0; l < bx; l++) {
-            const int q0 = c0 + l * bz;
+            const int b = stages == 2 ? l & 1 : 0, p0 = j * S + l * bz;
             const bool line_term = d.colsum && l > 0;
-            if (line_term) {  // block column sums of L2 T_{l-1}^{-1} U2 on line l
-                blocks<true>(u, bz, [&](int q) { return v.band(BD_L2, q0 + q); }, none, none, lane);
-                line_row_solve(v, q0 - bz, u, vt, W, lane);
-                blocks<false>(cs2, bz, none, [&](int q) { return W + 9 * q; },
-                              [&](int q) { return v.band(BD_U2, q0 - bz + q); }, lane);
+            const auto next = [&] {
+                if (stages == 2 && l + 1 < bx) stage_line(j, l + 1, b ^ 1, d.colsum, plane_term, 32, kNfThreads - 32);
+            };
+            TC *cs2 = fix(NB_CS2), *G = fix(NB_G), *GI = fix(NB_GI);
+            if (line_term) {
+                line_solve(st(b, ST_SRC), fix(NB_N), fix(NB_K), GI, next);
+                const TC *W = fix(NB_W), *post = st(b, ST_POST);
+                elements<TC>(bz, 0, kNfThreads,
+                             [&](int, int q, int r, int c, int o) { cs2[o] = prod(W + BS * q, post + BS * q, r, c); });
+                __syncthreads();
             }
-            // G_p = D_p - L1_p G_{p-1}^{-1} U1_{p-1} - (line and plane column sums); the previous
-            // cell's G^{-1} stays in a register, the next cell's operands load early
-            TC gprev = 0;
-            TC nd = ld<TC>(v.band(BD_D, q0), lane), nl1 = 0, nu1 = 0;
-            TC nc2 = line_term ? ld<TC>(cs2, lane) : TC(0), nc3 = plane_term ? ld<TC>(cs3 + 9 * l * bz, lane) : TC(0);
-            for (int q = 0; q < bz; q++) {
-                const int p = q0 + q;
-                const TC cd = nd, cl1 = nl1, cu1 = nu1, cc2 = nc2, cc3 = nc3;
-                if (q + 1 < bz) {
-                    nd = ld<TC>(v.band(BD_D, p + 1), lane);
-                    nl1 = ld<TC>(v.band(BD_L1, p + 1), lane);
-                    nu1 = ld<TC>(v.band(BD_U1, p), lane);
-                    if (line_term) nc2 = ld<TC>(cs2 + 9 * (q + 1), lane);
-                    if (plane_term) nc3 = ld<TC>(cs3 + 9 * (l * bz + q + 1), lane);
-                }
-                TC g = cd;
-                if (q > 0) g -= bmul(bmul(cl1, gprev, lane), cu1, lane);
-                g -= cc2;
-                g -= cc3;
-                if (lane < 9) d.g[9LL * p + lane] = (double)g;
-                TC gi;
-                if (!binv(g, gi, lane)) {
-                    if (lane == 0 && atomicCAS(&err->flag, 0, 1) == 0) {
-                        err->sub = d.sub;
-                        err->row = p;
+            if (seq) {
+                // G_p = D_p - L1_p G_{p-1}^{-1} U1_{p-1} - (line and plane column sums); the previous
+                // cell's G^{-1} stays in a register, the next cell's operands load early
+                const int e = lane < 9 ? lane : 0, o = RS * (e / 3) + e % 3;
+                const TC *D = st(b, ST_D) + o, *L1 = st(b, ST_L1) + o, *U1 = st(b, ST_U1) + o, *c2 = cs2 + o, *c3 = st(b, ST_C3) + o;
+                TC gprev = 0, nd = D[0], nl1 = 0, nu1 = 0, nc2 = line_term ? c2[0] : TC(0), nc3 = plane_term ? c3[0] : TC(0);
+#pragma unroll 1
+                for (int q = 0; q < bz; q++) {
+                    const TC cd = nd, cl1 = nl1, cu1 = nu1, cc2 = nc2, cc3 = nc3;
+                    if (q + 1 < bz) {
+                        nd = D[BS * (q + 1)];
+                        nl1 = L1[BS * (q + 1)];
+                        nu1 = U1[BS * q];
+                        if (line_term) nc2 = c2[BS * (q + 1)];
+                        if (plane_term) nc3 = c3[BS * (q + 1)];
                     }
-                    return;  // the whole warp leaves together (binv's result is warp-uniform)
+                    TC g = cd;
+                    if (q > 0) g -= bmul(bmul(cl1, gprev, lane), cu1, lane);
+                    g -= cc2;
+                    g -= cc3;
+                    TC gi;
+                    if (!binv(g, gi, lane)) {  // (warp-uniform)
+                        if (lane == 0) {
+                            bad = true;
+                            if (atomicCAS(&err->flag, 0, 1) == 0) {
+                                err->sub = d.sub;
+                                err->row = p0 + q;
+                            }
+                        }
+                        break;
+                    }
+                    if (lane < 9) {
+                        G[BS * q + o] = g;
+                        GI[BS * q + o] = gi;
+                    }
+                    gprev = gi;
                 }
-                if (lane < 9) d.gi[9LL * p + lane] = (double)gi;
-                gprev = gi;
+            } else if (!line_term) {
+                next();
             }
-            __syncwarp();
-            // N_q = G_q^{-1} U1_q and K_q = L1_{q+1} G_q^{-1} of this line, for its row-vector solves
-            TC* nline = v.nk + 9LL * q0;
-            TC* kline = v.nk + 9LL * (d.n + q0);
-            for (int t = lane; t < 9 * bz; t += 32) {
-                const int q = t / 9, e = t - 9 * q, r = e / 3, k = e - 3 * r;
-                const double* g = v.gi(q0 + q);
-                const TC* u1 = v.band(BD_U1, q0 + q);
-                nline[t] = (TC)g[3 * r] * u1[k] + (TC)g[3 * r + 1] * u1[3 + k] + (TC)g[3 * r + 2] * u1[6 + k];
-                TC kv = 0;
-                if (q + 1 < bz) {
-                    const TC* l1 = v.band(BD_L1, q0 + q + 1);
-                    kv = l1[3 * r] * (TC)g[k] + l1[3 * r + 1] * (TC)g[3 + k] + l1[3 * r + 2] * (TC)g[6 + k];
-                }
-                kline[t] = kv;
+            __syncthreads();
+            if (bad) return;
+            // G, G^{-1} and, for the line and plane solves, N_q and K_q
+            TC *N = fix(NB_N), *K = fix(NB_K);
+            const TC *L1 = st(b, ST_L1), *U1 = st(b, ST_U1);
+            elements<TC>(bz, 0, kNfThreads, [&](int t, int q, int r, int c, int o) {
+                const long long at = 9LL * p0 + t;
+                const TC n = prod(GI + BS * q, U1 + BS * q, r, c);
+                const TC k = q + 1 < bz ? prod(L1 + BS * (q + 1), GI + BS * q, r, c) : TC(0), gi = GI[o];
+                d.g[at] = (double)G[o];
+                d.gi[at] = (double)gi;
+                if (sizeof(TC) == 4) gg[at] = gi;
+                N[o] = n;
+                K[o] = k;
+                gn[at] = n;
+                gk[at] = k;
+            });
+            __syncthreads();
+            if (stages != 2 && l + 1 < bx) {
+                stage_line(j, l + 1, 0, d.colsum, plane_term, 0, kNfThreads);
+                __syncthreads();
             }
-            __syncwarp();
         }
     }
 }
@@ -851,23 +879,35 @@ size_t nf_apply_smem(int bx, int bz, int prec, int slots) {
            2 * nf_plane_bytes(bx * bz, prec) + vs * (size_t)bz * t;
 }
 
-size_t nf_work_doubles(int bx, int by, int bz) {
-    return 36 * ((size_t)bx * bz + (size_t)bz) + 18 * (size_t)bx * by * bz;
+size_t nf_work_doubles(int bx, int by, int bz) { return 18 * (size_t)bx * bz + 18 * (size_t)bx * by * bz; }
+
+namespace {
+size_t nf_factor_smem(int bz, int prec, int stages) {
+    return (size_t)(NB_FIXED + ST_FIELDS * stages) * bz * (prec == 0 ? LayF<double>::BS * 8 : LayF<float>::BS * 4);
 }
 
-void launch_nf_factor(const NFDesc* descs, int ndesc, int nmax, int prec, FactErr* err, cudaStream_t st) {
-    if (ndesc <= 0) return;
+template <typename TC>
+void nf_factor_t(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec, int dev_smem, FactErr* err, cudaStream_t st) {
     const dim3 ggrid((unsigned)((BD_N * nmax + 127) / 128), (unsigned)ndesc);
     const dim3 grid((unsigned)((nmax + 127) / 128), (unsigned)ndesc);
-    if (prec == 0) {
-        k_nf_gather<double><<<ggrid, 128, 0, st>>>(descs);
-        k_nf_factor<double><<<(ndesc + 3) / 4, 128, 0, st>>>(descs, ndesc, err);
-        k_nf_pack<double><<<grid, 128, 0, st>>>(descs);
-    } else {
-        k_nf_gather<float><<<ggrid, 128, 0, st>>>(descs);
-        k_nf_factor<float><<<(ndesc + 3) / 4, 128, 0, st>>>(descs, ndesc, err);
-        k_nf_pack<float><<<grid, 128, 0, st>>>(descs);
-    }
+    // one stage always fits where the apply's two ring slots (1,056 bytes a cell in FP64 and 720 in FP32,
+    // against 1,008 and 672 here) and its plane vectors do
+    const int stages = nf_factor_smem(bz_max, prec, 2) <= (size_t)dev_smem - 1024 ? 2 : 1;
+    const size_t smem = nf_factor_smem(bz_max, prec, stages);
+    cudaFuncSetAttribute(k_nf_factor<TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_nf_gather<TC><<<ggrid, 128, 0, st>>>(descs);
+    k_nf_factor<TC><<<ndesc, kNfThreads, smem, st>>>(descs, stages, err);
+    k_nf_pack<TC><<<grid, 128, 0, st>>>(descs);
+}
+}  // namespace
+
+void launch_nf_factor(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec, int dev_smem, FactErr* err,
+                      cudaStream_t st) {
+    if (ndesc <= 0) return;
+    if (prec == 0)
+        nf_factor_t<double>(descs, ndesc, nmax, bz_max, prec, dev_smem, err, st);
+    else
+        nf_factor_t<float>(descs, ndesc, nmax, bz_max, prec, dev_smem, err, st);
 }
 
 void launch_nf_apply(const SysTab* tab, const NFDesc* descs, int ndesc, int prec, int slots, size_t smem,
