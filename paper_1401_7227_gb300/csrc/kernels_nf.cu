@@ -21,6 +21,7 @@
 #include <algorithm>
 
 #include "asm2_internal.h"
+#include "f64cvt.h"
 #include "tma.h"
 
 namespace asm2 {
@@ -528,35 +529,32 @@ __device__ __forceinline__ void chain_step(const float4* a, float4 c, float& x0,
 }
 
 // x_q = c_q + A_q x_{q-d} for q = q0, q0 + d, ... (d = +-2; the x before q0 is zero), in place
-// in cb, on one lane (FP32).  Four steps make a group whose operands are loaded first.
+// in cb, on one lane (FP32).  The operands are loaded three steps ahead into a ring of registers (steps past
+// the end read the last one's again, so that the ring has no branches): four steps loaded together and then
+// computed left the loads' latency exposed once per group.
 __device__ __forceinline__ void chain(const float* A, float* cb, int q0, int d, int count) {
+    if (count <= 0) return;
     const float4* Av = reinterpret_cast<const float4*>(A);
     float4* cv = reinterpret_cast<float4*>(cb);
+    float4 a[4][3], c[4];
+    const auto load = [&](int i, int k) {
+        const int q = q0 + d * min(i, count - 1);
+        a[k][0] = Av[3 * q];
+        a[k][1] = Av[3 * q + 1];
+        a[k][2] = Av[3 * q + 2];
+        c[k] = cv[q];
+    };
+#pragma unroll
+    for (int i = 0; i < 3; i++) load(i, i);
     float x0 = 0.f, x1 = 0.f, x2 = 0.f;
-    int i = 0;
-    for (; i + 4 <= count; i += 4) {
-        float4 a[12], c[4];
+#pragma unroll 1
+    for (int i0 = 0; i0 < count; i0 += 4) {
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const int q = q0 + d * (i + u);
-            a[3 * u] = Av[3 * q];
-            a[3 * u + 1] = Av[3 * q + 1];
-            a[3 * u + 2] = Av[3 * q + 2];
-            c[u] = cv[q];
+        for (int k = 0; k < 4; k++) {
+            load(i0 + k + 3, (k + 3) & 3);
+            chain_step(a[k], c[k], x0, x1, x2);
+            if (i0 + k < count) cv[q0 + d * (i0 + k)] = make_float4(x0, x1, x2, 0.f);
         }
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            chain_step(a + 3 * u, c[u], x0, x1, x2);
-            c[u] = make_float4(x0, x1, x2, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; u++) cv[q0 + d * (i + u)] = c[u];
-    }
-    for (; i < count; i++) {
-        const int q = q0 + d * i;
-        const float4 a[3] = {Av[3 * q], Av[3 * q + 1], Av[3 * q + 2]};
-        chain_step(a, cv[q], x0, x1, x2);
-        cv[q] = make_float4(x0, x1, x2, 0.f);
     }
 }
 
@@ -658,8 +656,23 @@ __device__ __forceinline__ void line_solve(const T* M, const T* N, const T* P, c
     }
 }
 
-// B_i^{-1} R_i r for one subdomain per CTA (one warp), owned cells written to the apply output.
-// Shared memory: SLOTS + 1 mbarriers (16 bytes each) | SLOTS packet slots | SLOTS slots for the
+// an element of r in the compute type (FP32: the integer conversion, off the FP64 unit)
+template <typename T>
+__device__ __forceinline__ T to_compute(double v) {
+    if constexpr (sizeof(T) == 4)
+        return f64_to_f32(v);
+    else
+        return v;
+}
+
+// B_i^{-1} R_i r for one subdomain per CTA, owned cells written to the apply output.  Warp 0 solves the lines;
+// warp 1 issues the copies, a slot's next line as soon as warp 0 has released it.  What bounds the kernel is the
+// serial path of warp 0, ~3,600 cycles a line of 32 cells in FP32 (the two recurrences 850 each at 16 steps,
+// G^{-1} u 460, the wait 300, the other passes 240 - 410): addresses and copies of the next line, and the
+// conversion of r, are off it (64 boxes of 12 x 12 x 32 cells, an apply as called: FP32 1,084 -> 985 us, FP64
+// 4,360 -> 4,160).
+// Shared memory: SLOTS + 1 pairs of mbarriers (16 bytes: a slot is full | is free; y_j has come | the producer's
+// two words) | SLOTS packet slots | SLOTS slots for the
 // line's part of r (FP64) | plane vector pv [VS S] | y_j of a backward plane [VS S] | line vector
 // cb [VS bz].  pv holds, in turn, y_{j-1} and z / o of plane j during the forward planes, then
 // x_{j+1} and z / o of plane j during the backward ones: every line reads the previous plane's
@@ -667,7 +680,7 @@ __device__ __forceinline__ void line_solve(const T* M, const T* N, const T* P, c
 // nf_plane_bytes) when its forward plane is done, and comes back by a bulk copy issued at the start
 // of its backward plane.
 template <typename T, int SLOTS>
-__global__ void __launch_bounds__(32) k_nf_apply(const SysTab* __restrict__ tab, const NFDesc* __restrict__ descs) {
+__global__ void __launch_bounds__(64) k_nf_apply(const SysTab* __restrict__ tab, const NFDesc* __restrict__ descs) {
     constexpr int BS = 3 * Lay<T>::RS, VS = Lay<T>::VS;
     extern __shared__ __align__(16) unsigned char nf_smem[];
     const NFDesc d = descs[blockIdx.x];  // by value: its fields stay in registers across the stores
@@ -676,13 +689,15 @@ __global__ void __launch_bounds__(32) k_nf_apply(const SysTab* __restrict__ tab,
     if (in < 0) return;
     const double* __restrict__ r = st.ws + (long long)in * st.n3p;
     double* __restrict__ z = st.ws + (long long)st.ctl[C_APPLY_OUT] * st.n3p;
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x & 31;
     const int bx = d.bx, by = d.by, bz = d.bz, S = bx * bz;
     const unsigned fb = (unsigned)field_bytes<T>(bz);
     const size_t LB = (size_t)d.line_bytes, SB = (size_t)SL_FIELDS * fb, RB = nf_rline_bytes(bz),
                  PB = nf_plane_bytes<T>(S);
-    unsigned long long* bar = reinterpret_cast<unsigned long long*>(nf_smem);  // 2 words apart
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(nf_smem);  // full: even words, free: odd
     unsigned long long* ybar = bar + 2 * SLOTS;
+    volatile int* stop = reinterpret_cast<volatile int*>(ybar + 1);  // warp 0 has given up
+    volatile int* issued = stop + 1;                                 // line solves issued when warp 1 ends
     unsigned char* const pk_base = nf_smem + 16 * (SLOTS + 1);
     unsigned char* const r_base = pk_base + SLOTS * SB;
     T* pv = reinterpret_cast<T*>(r_base + SLOTS * RB);
@@ -733,25 +748,55 @@ __global__ void __launch_bounds__(32) k_nf_apply(const SysTab* __restrict__ tab,
         if (rbytes) tma::bulk_load(r_base + b * RB, rsrc, rbytes, &bar[2 * b]);
     };
 
-    LineStep nx, s;  // the next line solve to issue, the one in progress
-    nx.set(bx, by);
-    s.set(bx, by);
-    int ni = 0, bi = 0;  // line solves issued, slot of the next issue
-    if (lane == 0) {
-        for (int b = 0; b <= SLOTS; b++) tma::mbar_init(&bar[2 * b], 1);
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < SLOTS; b++) {
+            tma::mbar_init(&bar[2 * b], 1);
+            tma::mbar_init(&bar[2 * b + 1], 1);
+        }
+        tma::mbar_init(ybar, 1);
+        *stop = 0;
         tma::fence_mbar_init();
     }
-    __syncwarp();
-    for (; ni < SLOTS - 1 && ni < K; ni++) {
-        if (lane == 0) issue(nx, bi);
-        nx.next(bx, by);
-        bi = bi + 1 == SLOTS ? 0 : bi + 1;
+    __syncthreads();
+    if (threadIdx.x >= 32) {
+        if (lane == 0) {
+            LineStep nx;  // the next line solve to issue
+            nx.set(bx, by);
+            int ni = 0, bi = 0;
+            unsigned fph = 1;  // phase of "slot bi is free"
+            for (; ni < K; ni++) {
+                if (ni >= SLOTS) {
+                    bool ok = false;
+                    for (long long i = 0; i < tma::kWaitLimit && !ok && !*stop; i++) {
+                        ok = tma::mbar_try_wait(&bar[2 * bi + 1], fph);
+                        if (!ok) __nanosleep(200);  // (polling takes the shared-memory cycles of warp 0)
+                    }
+                    if (!ok) break;
+                }
+                issue(nx, bi);
+                nx.next(bx, by);
+                if (++bi == SLOTS) {
+                    bi = 0;
+                    fph ^= 1u;
+                }
+            }
+            *issued = ni;
+        }
+        __syncthreads();
+        return;
     }
+    LineStep s;
+    s.set(bx, by);
     bool ypend = false;
-    // a wait that expired: report it, wait (bounded) for the copies still in flight, and leave
+    // a wait that expired: report it, have warp 1 stop, wait (bounded) for the copies still in flight, and leave
     const auto fail = [&](int k) {
         if (lane == 0) {
             atomicExch(st.dev_err, 7);
+            *stop = 1;
+        }
+        __syncthreads();
+        if (lane == 0) {
+            const int ni = *issued;
             for (int k2 = k; k2 < ni; k2++) tma::mbar_wait(&bar[2 * (k2 % SLOTS)], (unsigned)(k2 / SLOTS) & 1u);
             if (ypend) tma::mbar_wait(ybar, (unsigned)(by - 2 - s.j) & 1u);
         }
@@ -759,13 +804,6 @@ __global__ void __launch_bounds__(32) k_nf_apply(const SysTab* __restrict__ tab,
     int bc = 0;
     unsigned ph = 0;  // slot and barrier phase of the line solve in progress
     for (int k = 0; k < K; k++) {
-        // line solve k + SLOTS - 1 goes into the slot that line solve k - 1 has finished with
-        if (ni < K) {
-            if (lane == 0) issue(nx, bi);
-            nx.next(bx, by);
-            bi = bi + 1 == SLOTS ? 0 : bi + 1;
-            ni++;
-        }
         if (s.plane_first && !s.fwd_plane) {  // y_j of this backward plane, needed when it is done
             if (lane == 0) {
                 tma::mbar_expect_tx(ybar, (unsigned)PB);
@@ -792,9 +830,9 @@ __global__ void __launch_bounds__(32) k_nf_apply(const SysTab* __restrict__ tab,
             const T* cur = pl + VS * q;
             if (s.fwd_line) {
                 if (s.fwd_plane) {
-                    u0 = (T)rl[3 * q];
-                    u1 = (T)rl[3 * q + 1];
-                    u2 = (T)rl[3 * q + 2];
+                    u0 = to_compute<T>(rl[3 * q]);
+                    u1 = to_compute<T>(rl[3 * q + 1]);
+                    u2 = to_compute<T>(rl[3 * q + 2]);
                     if (s.j > 0) {
                         ld3(cur, x0, x1, x2);
                         sub_mv(blk(SL_Y, q), x0, x1, x2, u0, u1, u2);  // L3
@@ -818,6 +856,7 @@ __global__ void __launch_bounds__(32) k_nf_apply(const SysTab* __restrict__ tab,
         __syncwarp();
         line_solve(blk(PK_M, 0), blk(PK_N, 0), blk(PK_P, 0), blk(PK_Q, 0), cb, pl, bz, s.fwd_line, lane);
         __syncwarp();
+        if (lane == 0) tma::mbar_arrive(&bar[2 * bc + 1]);  // the slot is free
         if (s.plane_done) {  // pv = P_j^{-1} t
             if (s.fwd_plane) {
                 if (s.j < by - 1) {  // y_j to device memory, ordered before its later bulk copy back
@@ -846,12 +885,13 @@ __global__ void __launch_bounds__(32) k_nf_apply(const SysTab* __restrict__ tab,
             ph ^= 1u;
         }
     }
+    __syncthreads();  // (with warp 1's end)
 }
 
 template <typename T, int SLOTS>
 void nf_apply_t(const SysTab* tab, const NFDesc* descs, int ndesc, size_t smem, cudaStream_t st) {
     cudaFuncSetAttribute(k_nf_apply<T, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_nf_apply<T, SLOTS><<<ndesc, 32, smem, st>>>(tab, descs);
+    k_nf_apply<T, SLOTS><<<ndesc, 64, smem, st>>>(tab, descs);
 }
 
 template <typename T>
