@@ -1122,7 +1122,8 @@ int factor_numeric(asm_ctx* h) {
         launch_nf_factor(h->d_nfdesc1.as<NFDesc>(), (int)h->nf_desc.size(), nmax, h->nf_bz_max, h->prec, h->dev_smem,
                          h->d_err.as<FactErr>(), h->stream);
     } else {
-        launch_factor(h->d_factdesc.as<FactDesc>(), (int)S.subs.size(), h->d_err.as<FactErr>(), nullptr, h->stream);
+        launch_factor(h->d_factdesc.as<FactDesc>(), (int)S.subs.size(), h->n_sms, h->d_err.as<FactErr>(), nullptr,
+                      h->stream);
         if (h->lanes_ok) {
             launch_pack_lanes(h->d_ln_off_f.as<long long>(), h->d_ln_src_f.as<int>(), h->ln_nf, h->prec,
                               h->d_lanes.as<unsigned char>(), h->d_slot.as<double>(), h->stream);

@@ -263,7 +263,8 @@ constexpr int kLongAssembly = 32;
 void launch_assemble(const int* aptr, const int* aloc, const int* acs, const double* bsr_val, const double* cval,
                      double* slot, long long nslot, cudaStream_t st, const int* long_slots = nullptr, int nlong = 0);
 void launch_coarse(const int* cptr, const int* cloc, const double* bsr_val, double* cval, int nc, cudaStream_t st);
-void launch_factor(const FactDesc* fd, int nsub, FactErr* err, const int* sub_ids, cudaStream_t st);
+// sms: the device's SMs
+void launch_factor(const FactDesc* fd, int nsub, int sms, FactErr* err, const int* sub_ids, cudaStream_t st);
 void launch_pack(const long long* off, const int* src, long long n, int prec, unsigned char* stream_base,
                  const double* slot_base, cudaStream_t st);
 // the same blocks into the streams by lane (packets.h: off holds ~offset for the blocks of a long lump row)

@@ -120,41 +120,60 @@ __global__ void __launch_bounds__(256) k_assemble_long(const int* __restrict__ a
     }
 }
 
-// 3x3 inverse by Gauss-Jordan elimination with partial pivoting; false on a zero pivot.
-__device__ bool inverse3(const double* a, double* inv) {
-    double m[3][6];
-#pragma unroll
-    for (int r = 0; r < 3; r++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            m[r][c] = a[3 * r + c];
-            m[r][3 + c] = (r == c) ? 1.0 : 0.0;
-        }
+// 3x3 inverse in place by Gauss-Jordan elimination with partial pivoting; false on a zero pivot (m is then
+// undefined).  The operations on [A | I], without those on the zeros and ones of I: ~60 instructions of the
+// FP64 unit instead of ~100.
+__device__ __forceinline__ bool inverse3(double (&m)[3][3]) {
+    int piv[2] = {0, 1};
 #pragma unroll
     for (int c = 0; c < 3; c++) {
         int p = c;
+        double big = fabs(m[c][c]);
+#pragma unroll
         for (int r = c + 1; r < 3; r++)
-            if (fabs(m[r][c]) > fabs(m[p][c])) p = r;
-        if (m[p][c] == 0.0) return false;
-        if (p != c)
-            for (int k = 0; k < 6; k++) {
-                double t = m[c][k];
-                m[c][k] = m[p][k];
-                m[p][k] = t;
+            if (fabs(m[r][c]) > big) {
+                p = r;
+                big = fabs(m[r][c]);
             }
+        if (big == 0.0) return false;
+#pragma unroll
+        for (int r = c + 1; r < 3; r++)
+            if (p == r)
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    const double t = m[c][k];
+                    m[c][k] = m[r][k];
+                    m[r][k] = t;
+                }
+        if (c < 2) piv[c] = p;
         // one reciprocal per pivot column: FP64 division expands to many FP64-pipe instructions
         const double id = 1.0 / m[c][c];
-        for (int k = 0; k < 6; k++) m[c][k] *= id;
+        m[c][c] = id;
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+            if (k != c) m[c][k] *= id;
+#pragma unroll
         for (int r = 0; r < 3; r++) {
             if (r == c) continue;
             const double f = m[r][c];
-            for (int k = 0; k < 6; k++) m[r][k] -= f * m[c][k];
+#pragma unroll
+            for (int k = 0; k < 3; k++)
+                if (k != c) m[r][k] = fma(-f, m[c][k], m[r][k]);
+            m[r][c] = -(f * id);
         }
     }
+    // the inverse of the row-swapped matrix: its columns in the order of the rows
 #pragma unroll
-    for (int r = 0; r < 3; r++)
+    for (int c = 1; c >= 0; c--)
 #pragma unroll
-        for (int c = 0; c < 3; c++) inv[3 * r + c] = m[r][3 + c];
+        for (int r = 0; r < 3; r++)
+#pragma unroll
+            for (int k = c + 1; k < 3; k++)
+                if (piv[c] == k) {
+                    const double t = m[r][c];
+                    m[r][c] = m[r][k];
+                    m[r][k] = t;
+                }
     return true;
 }
 
@@ -162,88 +181,153 @@ __device__ bool inverse3(const double* a, double* inv) {
 // (A) every slot finalised at this level subtracts its (L, U) pairs in the order the
 // right-looking update would apply them (compensations of dropped fill are pairs of the
 // diagonal slots); (B) the level's pivots are inverted; (C) its L column blocks are scaled by
-// D^{-1}.  All pairs reference slots finalised at lower levels.  Four CTAs per SM (64 registers):
-// the 512 subdomains of a 1M-cell grid run in one wave, and the extra warps fill the FP64 pipe's
-// gaps (the 1M-cell re-factor 11.35 -> 10.51 ms against two CTAs per SM; three was slower).
-__global__ void __launch_bounds__(256, 4) k_factor(const FactDesc* __restrict__ fds, const int* __restrict__ ids,
-                                                FactErr* err) {
+// D^{-1}.  All pairs reference slots finalised at lower levels.
+//
+// What bounds it is latency: a level of 40-65 rows has three phases with a barrier each, and each phase is a chain
+// of dependent loads (~1,000 cycles a link) and of dependent FP64 operations (69 cycles; a level's longest
+// target has 10-100 pairs of three).  So T threads and MINB CTAs per SM fill the SM's registers for the number of
+// subdomains in the launch, a phase's first indices are loaded in the phase before, and a target's next KP pairs
+// and a thread's KC blocks of L are in flight together.  Re-factor before -> after: 64 x 64 x 16 cells
+// (64 subdomains) 1.27 -> 0.94 ms, 97 x 83 x 29 (120) 2.95 -> 2.28, 128 x 128 x 32 (256) 4.71 -> 4.07,
+// 128 x 128 x 64 (512) 8.98 -> 8.35.
+template <int T, int MINB, int KP, int KC>
+__global__ void __launch_bounds__(T, MINB) k_factor(const FactDesc* __restrict__ fds, const int* __restrict__ ids,
+                                                    FactErr* err) {
     const FactDesc fd = fds[ids ? ids[blockIdx.x] : blockIdx.x];
     double* slot = fd.slot;
     // nine lanes per 3x3 result (lane = 3 r + c within a group), three groups per warp: each FP64
     // instruction then serves three targets instead of one thread's nine elements
     const int lane = threadIdx.x & 31, grp = lane / 9, e9 = lane - 9 * grp, er = e9 / 3, ec = e9 - 3 * er;
-    const int warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5, nwarp = T >> 5;
     const bool lane_on = grp < 3;
+    // What a level reads first -- its ranges, the first target, pivot row and L block of each thread -- is
+    // requested a phase or a level ahead: those loads are links of a serial chain of ~1,000 cycles each.
+    int tl0 = fd.tgt_lv[0], lp0 = fd.lv_pos0[0], l0 = fd.ls_lv[0];
+    int tl1 = fd.tgt_lv[1], lp1 = fd.lv_pos0[1], l1 = fd.ls_lv[1];
+    int nsl = 0, nq0 = 0, nq1 = 0;
+    const auto target = [&](int t) {
+        nsl = fd.tgt[t];
+        nq0 = fd.pp[t];
+        nq1 = fd.pp[t + 1];
+    };
+    if (lane_on && tl0 + 3 * warp + grp < tl1) target(tl0 + 3 * warp + grp);
     for (int lv = 0; lv < fd.nlev; lv++) {
-        for (int t0 = fd.tgt_lv[lv] + 3 * warp; t0 < fd.tgt_lv[lv + 1]; t0 += 3 * nwarp) {
-            const int t = t0 + grp;
-            if (!lane_on || t >= fd.tgt_lv[lv + 1]) continue;
-            double* s = slot + (long long)fd.tgt[t] * 9;
+        const int lvn = min(lv + 2, fd.nlev);
+        const int tl2 = fd.tgt_lv[lvn], lp2 = fd.lv_pos0[lvn], l2 = fd.ls_lv[lvn];
+        const int p0 = lp0 + threadIdx.x;
+        const int dpos = p0 < lp1 ? fd.diag_of_pos[p0] : 0, rpos = p0 < lp1 ? fd.row_of_pos[p0] : 0;
+        int t = tl0 + 3 * warp + grp;
+        bool on = lane_on && t < tl1;
+        while (on) {
+            double* s = slot + (long long)nsl * 9;
+            const int q0 = nq0, q1 = nq1;
+            t += 3 * nwarp;
+            on = t < tl1;
+            if (on) target(t);
             double acc = s[e9];
-            // kP pairs at a time: their indices, then their blocks, are loaded before any arithmetic
-            // (the pairs are subtracted in the same order as one at a time)
-            constexpr int kP = 4;
-            const int q1 = fd.pp[t + 1];
-            for (int q0 = fd.pp[t]; q0 < q1; q0 += kP) {
-                int2 pr[kP];
+            // KP pairs at a time, in the order of one at a time: the blocks of the next ones and the indices of
+            // those after them are requested before the arithmetic
+            int2 pa[KP], pb[KP];
+            double la[KP][3], ua[KP][3], lb[KP][3], ub[KP][3];
+            const auto pairs = [&](int q, int2(&pr)[KP]) {
 #pragma unroll
-                for (int u = 0; u < kP; u++) pr[u] = q0 + u < q1 ? fd.pair[q0 + u] : make_int2(-1, -1);
-                double l[kP][3], uu[kP][3];
+                for (int u = 0; u < KP; u++) pr[u] = q + u < q1 ? fd.pair[q + u] : make_int2(0, 0);
+            };
+            const auto blocks = [&](const int2(&pr)[KP], double(&l)[KP][3], double(&uu)[KP][3]) {
 #pragma unroll
-                for (int u = 0; u < kP; u++) {
-                    const bool on = pr[u].x >= 0;
-                    const double* L = slot + (long long)(on ? pr[u].x : 0) * 9 + 3 * er;
-                    const double* U = slot + (long long)(on ? pr[u].y : 0) * 9 + ec;
-                    l[u][0] = L[0];
-                    l[u][1] = L[1];
-                    l[u][2] = L[2];
-                    uu[u][0] = U[0];
-                    uu[u][1] = U[3];
-                    uu[u][2] = U[6];
+                for (int u = 0; u < KP; u++) {
+                    const double* L = slot + (long long)pr[u].x * 9 + 3 * er;
+                    const double* U = slot + (long long)pr[u].y * 9 + ec;
+#pragma unroll
+                    for (int k = 0; k < 3; k++) {
+                        l[u][k] = L[k];
+                        uu[u][k] = U[3 * k];
+                    }
                 }
+            };
+            const auto subtract = [&](int q, const double(&l)[KP][3], const double(&uu)[KP][3]) {
 #pragma unroll
-                for (int u = 0; u < kP; u++)
-                    if (pr[u].x >= 0)  // three FMAs into the running value (not product, sum, subtract)
+                for (int u = 0; u < KP; u++)
+                    if (q + u < q1)  // three FMAs into the running value (not product, sum, subtract)
                         acc = fma(-l[u][2], uu[u][2], fma(-l[u][1], uu[u][1], fma(-l[u][0], uu[u][0], acc)));
+            };
+            pairs(q0, pa);
+            blocks(pa, la, ua);
+            pairs(q0 + KP, pb);
+            for (int q = q0; q < q1;) {
+                if (q + KP < q1) {
+                    blocks(pb, lb, ub);
+                    pairs(q + 2 * KP, pa);
+                }
+                subtract(q, la, ua);
+                q += KP;
+                if (q >= q1) break;
+                if (q + KP < q1) {
+                    blocks(pa, la, ua);
+                    pairs(q + 2 * KP, pb);
+                }
+                subtract(q, lb, ub);
+                q += KP;
             }
             s[e9] = acc;
         }
+        if (lane_on && tl1 + 3 * warp + grp < tl2) target(tl1 + 3 * warp + grp);  // of the next level
+        int2 lq[KC];
+#pragma unroll
+        for (int u = 0; u < KC; u++) {
+            const int i = l0 + 3 * (warp + nwarp * u) + grp;
+            lq[u] = lane_on && i < l1 ? fd.ls[i] : make_int2(-1, -1);
+        }
         __syncthreads();
-        for (int p = fd.lv_pos0[lv] + threadIdx.x; p < fd.lv_pos0[lv + 1]; p += blockDim.x) {
-            double* d = slot + (long long)fd.diag_of_pos[p] * 9;
-            double D[9], Di[9];
+        for (int p = p0; p < lp1; p += T) {
+            double* d = slot + (long long)(p == p0 ? dpos : fd.diag_of_pos[p]) * 9;
+            const int row = p == p0 ? rpos : fd.row_of_pos[p];
+            double D[3][3];
 #pragma unroll
-            for (int e = 0; e < 9; e++) D[e] = d[e];
-            double* dp = fd.dpiv + (long long)fd.row_of_pos[p] * 9;
+            for (int e = 0; e < 9; e++) D[e / 3][e % 3] = d[e];
+            double* dp = fd.dpiv + (long long)row * 9;
 #pragma unroll
-            for (int e = 0; e < 9; e++) dp[e] = D[e];
-            if (!inverse3(D, Di)) {
+            for (int e = 0; e < 9; e++) dp[e] = D[e / 3][e % 3];
+            if (!inverse3(D)) {
                 if (atomicCAS(&err->flag, 0, 1) == 0) {
                     err->sub = ids ? ids[blockIdx.x] : blockIdx.x;
-                    err->row = fd.row_of_pos[p];
+                    err->row = row;
                 }
 #pragma unroll
-                for (int e = 0; e < 9; e++) Di[e] = (e % 4 == 0) ? 1.0 : 0.0;
+                for (int e = 0; e < 9; e++) D[e / 3][e % 3] = (e % 4 == 0) ? 1.0 : 0.0;
             }
 #pragma unroll
-            for (int e = 0; e < 9; e++) d[e] = Di[e];
+            for (int e = 0; e < 9; e++) d[e] = D[e / 3][e % 3];
         }
         __syncthreads();
-        for (int t0 = fd.ls_lv[lv] + 3 * warp; t0 < fd.ls_lv[lv + 1]; t0 += 3 * nwarp) {
-            const int t = t0 + grp;
-            double v = 0.0;
-            int2 q = make_int2(0, 0);
-            const bool on = lane_on && t < fd.ls_lv[lv + 1];
-            if (on) {
-                q = fd.ls[t];
-                const double* A = slot + (long long)q.x * 9 + 3 * er;
-                const double* Di = slot + (long long)q.y * 9 + ec;
-                v = A[0] * Di[0] + A[1] * Di[3] + A[2] * Di[6];
+        // KC items of a lane at a time: their blocks, and the next ones' indices, are loaded before any arithmetic
+        for (int i0 = l0 + 3 * warp; i0 < l1; i0 += 3 * nwarp * KC) {
+            int2 q[KC];
+            double a[KC][3], di[KC][3];
+#pragma unroll
+            for (int u = 0; u < KC; u++) {
+                q[u] = lq[u];
+                const int i = i0 + grp + 3 * nwarp * (KC + u);
+                lq[u] = lane_on && i < l1 ? fd.ls[i] : make_int2(-1, -1);
             }
-            __syncwarp();  // every lane of the group has read its row of L before any writes
-            if (on) slot[(long long)q.x * 9 + e9] = v;
+#pragma unroll
+            for (int u = 0; u < KC; u++) {
+                const double* A = slot + (long long)max(q[u].x, 0) * 9 + 3 * er;
+                const double* Di = slot + (long long)max(q[u].y, 0) * 9 + ec;
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    a[u][k] = q[u].x >= 0 ? A[k] : 0.0;
+                    di[u][k] = q[u].x >= 0 ? Di[3 * k] : 0.0;
+                }
+            }
+            __syncwarp();  // every lane of a group has read its row of L before any writes
+#pragma unroll
+            for (int u = 0; u < KC; u++)
+                if (q[u].x >= 0)
+                    slot[(long long)q[u].x * 9 + e9] = a[u][0] * di[u][0] + a[u][1] * di[u][1] + a[u][2] * di[u][2];
         }
         __syncthreads();
+        tl0 = tl1, tl1 = tl2, lp0 = lp1, lp1 = lp2, l0 = l1, l1 = l2;
     }
 }
 
@@ -335,9 +419,18 @@ void launch_assemble(const int* aptr, const int* aloc, const int* acs, const dou
                                                          nlong);
 }
 
-void launch_factor(const FactDesc* fd, int nsub, FactErr* err, const int* sub_ids, cudaStream_t st) {
+void launch_factor(const FactDesc* fd, int nsub, int sms, FactErr* err, const int* sub_ids, cudaStream_t st) {
     if (nsub <= 0) return;
-    k_factor<<<nsub, 256, 0, st>>>(fd, sub_ids, err);
+    // As many threads as are resident with every CTA of the launch on the chip at once.  128 x 128 x 32 cells in
+    // 256 subdomains, the whole re-factor: 4.07 ms with 512 threads and two CTAs per SM, 4.60 with one, 4.34 with
+    // four of 256 threads; 64 subdomains (64 x 64 x 16): 0.94 with 512 threads of 126 registers, 0.99 with 1,024 of
+    // 64, 1.17 with 256; 512 subdomains (128 x 128 x 64): 8.35 with four of 256, 8.92 with two of 512.
+    if (nsub <= sms)
+        k_factor<512, 1, 2, 3><<<nsub, 512, 0, st>>>(fd, sub_ids, err);
+    else if (nsub <= 2 * sms)
+        k_factor<512, 2, 2, 2><<<nsub, 512, 0, st>>>(fd, sub_ids, err);
+    else
+        k_factor<256, 4, 2, 2><<<nsub, 256, 0, st>>>(fd, sub_ids, err);
 }
 
 void launch_pack(const long long* off, const int* src, long long n, int prec, unsigned char* stream_base,
