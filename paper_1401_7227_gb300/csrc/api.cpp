@@ -1398,7 +1398,7 @@ std::vector<ApplyConfig> apply_candidates(const Batch& B) {
 }
 
 // kernels launched by launch_local_solves
-int local_solve_launches(const Batch& B) { return B.nf ? 1 : 2; }
+int local_solve_launches(const Batch& B) { return B.nf || (!B.exact && B.apply.ymode == Y_PACKET) ? 1 : 2; }
 
 // the local solves of one apply: R_i r and the fused ILU sweeps, or R_i r and the owned rows of
 // A_i^{-1} R_i r, or the nested-factorisation sweeps
@@ -1409,7 +1409,8 @@ void launch_local_solves(Batch& B, const SysTab* tab, cudaStream_t st) {
         launch_dense_restrict(tab, B.d_sub.as<SubDesc>(), B.nsub, st);
         launch_dense_apply(tab, B.d_sub.as<SubDesc>(), B.d_dense.as<int2>(), B.ndense, st);
     } else {
-        launch_restrict(tab, B.d_sub.as<SubDesc>(), B.d_ritems.as<int2>(), B.nritems, B.prec, B.lump32, st);
+        if (B.apply.ymode != Y_PACKET)  // (the apply by lane forms R_i r itself)
+            launch_restrict(tab, B.d_sub.as<SubDesc>(), B.d_ritems.as<int2>(), B.nritems, B.prec, B.lump32, st);
         launch_apply(tab, B.d_sub.as<SubDesc>(), B.nsub, B.prec, B.lump32, B.apply, st);
     }
 }
@@ -2322,8 +2323,9 @@ ApplyConfig single_apply_config(const asm_ctx* h, int place) {
 // R_i r and the fused ILU sweeps of every subdomain (after k_sums), single-system tables
 void launch_ilu_local_solves(asm_ctx* h, const ApplyConfig& cfg) {
     use_stream(h, cfg);
-    launch_restrict(h->d_tab1.as<SysTab>(), h->d_subdesc_single.as<SubDesc>(), h->d_ritems1.as<int2>(), h->n_ritems1,
-                    h->prec, h->lump32, h->stream);
+    if (cfg.ymode != Y_PACKET)  // (the apply by lane forms R_i r itself)
+        launch_restrict(h->d_tab1.as<SysTab>(), h->d_subdesc_single.as<SubDesc>(), h->d_ritems1.as<int2>(), h->n_ritems1,
+                        h->prec, h->lump32, h->stream);
     launch_apply(h->d_tab1.as<SysTab>(), h->d_subdesc_single.as<SubDesc>(), (int)h->sub_desc.size(), h->prec,
                  h->lump32, cfg, h->stream);
 }
@@ -2340,6 +2342,7 @@ int asm_apply_precond(asm_handle h, const double* r, double* z, int on_device) {
         set_ctl(h, VU, VZ, -1, -1, -1);
         launch_boxsum(h->d_tab1.as<SysTab>(), h->d_box1.as<BoxItem>(), (int)h->box_items.size(), h->n_group_items,
                       h->stream);
+        bool by_lane = false;
         if (is_nf(h)) {
             launch_nf_apply(h->d_tab1.as<SysTab>(), h->d_nfdesc1.as<NFDesc>(), (int)h->nf_desc.size(), h->prec,
                             h->nf_slots, h->nf_smem, h->stream);
@@ -2349,7 +2352,9 @@ int asm_apply_precond(asm_handle h, const double* r, double* z, int on_device) {
             launch_dense_apply(h->d_tab1.as<SysTab>(), h->d_subdesc_single.as<SubDesc>(), h->d_ditems1.as<int2>(),
                                h->n_ditems1, h->stream);
         } else {
-            launch_ilu_local_solves(h, single_apply_config(h, h->apply_place));
+            const ApplyConfig cfg = single_apply_config(h, h->apply_place);
+            launch_ilu_local_solves(h, cfg);
+            by_lane = cfg.ymode == Y_PACKET;
         }
         if (h->tab.cmode != 0)
             launch_coarse_apply(h->d_tab1.as<SysTab>(), h->d_row1.as<RowItem>(), h->n_row1,
@@ -2357,7 +2362,7 @@ int asm_apply_precond(asm_handle h, const double* r, double* z, int on_device) {
                                 (int)h->cgrow_items.size(), h->d_vec1.as<VecItem>(), h->n_vec1, h->tab.cmode == 2,
                                 h->stream);
         ck(cudaGetLastError());
-        h->prof.kernel_launches += is_nf(h) ? 2 : 3;
+        h->prof.kernel_launches += is_nf(h) || by_lane ? 2 : 3;
         copy_out(h, z, out, bytes, on_device);
         sync(h);
         return take_dev_err(h) ? ASM_ERR_TIMEOUT : ASM_OK;

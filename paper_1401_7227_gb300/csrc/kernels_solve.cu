@@ -618,23 +618,14 @@ __device__ __forceinline__ void restrict_local(const SysTab& st, const SubDesc& 
     }
 }
 
-// R_i r (Eqs. 4.1, B.2) of every subdomain into its device-memory local vectors, in the layout of
+// Row q of R_i r (Eqs. 4.1, B.2) into a subdomain's local vectors y, in the layout of
 // y_layout(): a fine row copies its cell's entries (rounded to the fine rows' compute type), a
 // lump row sums its cells in FP64 -- a far lump as the far box's sum minus its near-region cells
 // -- and is rounded to the lump type TL (with an FP32 mirror of FP64 lumps under FP32 fine rows;
 // with FP32 lumps every row is four floats, the last zero).
-// One thread per local row; items are (subdomain, first row of 256).
 template <typename TC, typename TL>
-__global__ void __launch_bounds__(256) k_restrict(const SysTab* __restrict__ tab, const SubDesc* __restrict__ subs,
-                                                  const int2* __restrict__ items) {
-    const int2 it = items[blockIdx.x];
-    const SubDesc& sd = subs[it.x];
-    const SysTab& st = tab[sd.sys];
-    const int in = st.ctl[C_APPLY_IN];
-    if (in < 0) return;
-    const double* __restrict__ r = st.ws + (long long)in * st.n3p;
-    unsigned char* y = reinterpret_cast<unsigned char*>(sd.y);
-    const int q = it.y + threadIdx.x;
+__device__ __forceinline__ void restrict_row(const SysTab& st, const SubDesc& sd, const double* __restrict__ r, int q,
+                                             unsigned char* y) {
     constexpr bool kRow16 = sizeof(TL) == 4;  // FP32 lumps: rows of four floats (16 bytes)
     if (q < sd.nf) {
         if constexpr (kRow16) {
@@ -705,6 +696,19 @@ __global__ void __launch_bounds__(256) k_restrict(const SysTab* __restrict__ tab
         ycf[1] = narrow<TC>(a1);
         ycf[2] = narrow<TC>(a2);
     }
+}
+
+// R_i r of every subdomain into its device-memory local vectors, for the applies that read them there.
+// One thread per local row; items are (subdomain, first row of 256).
+template <typename TC, typename TL>
+__global__ void __launch_bounds__(256) k_restrict(const SysTab* __restrict__ tab, const SubDesc* __restrict__ subs,
+                                                  const int2* __restrict__ items) {
+    const int2 it = items[blockIdx.x];
+    const SubDesc& sd = subs[it.x];
+    const SysTab& st = tab[sd.sys];
+    const int in = st.ctl[C_APPLY_IN];
+    if (in < 0) return;
+    restrict_row<TC, TL>(st, sd, st.ws + (long long)in * st.n3p, it.y + threadIdx.x, reinterpret_cast<unsigned char*>(sd.y));
 }
 
 // Fused local solve of one subdomain (one CTA): y = R_i r; y = L^{-1} y; y = U^{-1} y;
@@ -963,7 +967,8 @@ __global__ void __launch_bounds__(32 * kPkWarps, sizeof(TF) == 8 ? 1 : 2) k_appl
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const SubDesc& sd = subs[blockIdx.x];
     const SysTab& st = tab[sd.sys];
-    if (st.ctl[C_APPLY_IN] < 0) return;
+    const int in = st.ctl[C_APPLY_IN];
+    if (in < 0) return;
     double* __restrict__ z = st.ws + (long long)st.ctl[C_APPLY_OUT] * st.n3p;
     const int cap = sd.pk_cap, n_chunks = sd.n_chunks;
     const int2* __restrict__ chunks = sd.pk_chunks;
@@ -985,12 +990,11 @@ __global__ void __launch_bounds__(32 * kPkWarps, sizeof(TF) == 8 ? 1 : 2) k_appl
             mbar_expect_tx(&bar[k], (unsigned)ch.y);
             bulk_load(ring + (size_t)k * cap, stream + ch.x, (unsigned)ch.y, &bar[k]);
         }
-    {
-        const int4* src = reinterpret_cast<const int4*>(sd.y);
-        const int n16 = sd.y_bytes >> 4;
-        for (int t = tid; t < n16; t += blockDim.x) reinterpret_cast<int4*>(y)[t] = src[t];
-        if (tid < 2) reinterpret_cast<int4*>(y)[n16 + tid] = make_int4(0, 0, 0, 0);
-    }
+    // R_i r, formed here while the first chunks are on their way (a launch of its own, through device memory,
+    // took 7 - 10 us)
+    const double* r = st.ws + (long long)in * st.n3p;
+    for (int q = tid; q < sd.nf + sd.nc; q += blockDim.x) restrict_row<T, T>(st, sd, r, q, y);
+    if (tid < 2) reinterpret_cast<int4*>(y)[(sd.y_bytes >> 4) + tid] = make_int4(0, 0, 0, 0);
     // The last warp (with the fewest packets) waits for the next chunk to land while the others work on this
     // one, so that nobody waits after the barrier; its lane 0 refills the slots, and keeps the next
     // descriptor, loaded one ahead.
