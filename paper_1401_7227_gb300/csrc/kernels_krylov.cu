@@ -12,31 +12,66 @@ namespace asm2 {
 namespace {
 
 // ------------------------------------------------------------------------------------------
-// SpMV y = A x or y = b - A x (ELL, one thread per block row, 3x3 blocks); four CTAs per SM
-// (64 registers) hide the gathers of x better than three at 80 registers
+// SpMV y = A x or y = b - A x (ELL, one thread per block row, 3x3 blocks).  Bound by the FP64 unit (63 FMAs a
+// row of seven blocks: 105 us at a million rows) and by HBM (85 us) at once, so the next block's values and x are
+// requested before the arithmetic of this one, and the column after that; the values are read once (streaming
+// loads).  With the loads of a block after the arithmetic of the last, 256 threads and 64 registers: 148.9 us a
+// launch at 128 x 128 x 64 (0.71 of the FP64 rate), now 129.5 (0.81); 97 x 83 x 29 46 -> 38 us, 64 x 64 x 16
+// 22 -> 16.4, 10 x 10 x 5 12.3 -> 10.2 (with the gaps between events).  256 threads and three CTAs per SM: 133.7.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 4) k_spmv(const SysTab* __restrict__ tab, const RowItem* __restrict__ items) {
-    const RowItem it = items[blockIdx.x];
+constexpr int kSpmvThreads = 128;
+
+__global__ void __launch_bounds__(kSpmvThreads, 6) k_spmv(const SysTab* __restrict__ tab, const RowItem* __restrict__ items) {
+    constexpr int per = 256 / kSpmvThreads;  // CTAs per item of 256 rows
+    const RowItem it = items[blockIdx.x / per];
     const SysTab& st = tab[it.sys];
     const int in = st.ctl[C_SPMV_IN];
     if (in < 0) return;
-    const int row = it.r0 + threadIdx.x;
+    const int row = it.r0 + kSpmvThreads * (blockIdx.x % per) + threadIdx.x;
     if (row >= st.n_cells) return;
     const int out = st.ctl[C_SPMV_OUT];
     const int bs = st.ctl[C_SPMV_B];
     const double* __restrict__ x = st.ws + (long long)in * st.n3p;
     double* __restrict__ y = st.ws + (long long)out * st.n3p;
     const long long rp = st.rows_pad;
+    const int W = st.ell_w;
+    const int* __restrict__ cp = st.ell_col + row;
+    const double* __restrict__ vp = st.ell_val + row;
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    for (int w = 0; w < st.ell_w; w++) {
-        const int c = st.ell_col[(long long)w * rp + row];
-        const double x0 = x[3LL * c], x1 = x[3LL * c + 1], x2 = x[3LL * c + 2];
-        const double* v = st.ell_val + (long long)w * 9 * rp + row;
-        // one FMA per product into the running sums: an FP64 instruction costs a warp ~64 cycles
-        // here, and a separate product-then-add form would take four per three products
-        a0 = fma(v[2 * rp], x2, fma(v[rp], x1, fma(v[0], x0, a0)));
-        a1 = fma(v[5 * rp], x2, fma(v[4 * rp], x1, fma(v[3 * rp], x0, a1)));
-        a2 = fma(v[8 * rp], x2, fma(v[7 * rp], x1, fma(v[6 * rp], x0, a2)));
+    double v[2][9], xx[2][3];
+    int c1 = 0;
+    const auto load = [&](int h, int c, const double* q) {
+#pragma unroll
+        for (int k = 0; k < 9; k++) v[h][k] = __ldcs(q + k * rp);
+        xx[h][0] = x[3LL * c], xx[h][1] = x[3LL * c + 1], xx[h][2] = x[3LL * c + 2];
+    };
+    // one FMA per product into the running sums: an FP64 instruction costs a warp ~64 cycles
+    // here, and a separate product-then-add form would take four per three products
+    const auto mac = [&](int h) {
+        a0 = fma(v[h][2], xx[h][2], fma(v[h][1], xx[h][1], fma(v[h][0], xx[h][0], a0)));
+        a1 = fma(v[h][5], xx[h][2], fma(v[h][4], xx[h][1], fma(v[h][3], xx[h][0], a1)));
+        a2 = fma(v[h][8], xx[h][2], fma(v[h][7], xx[h][1], fma(v[h][6], xx[h][0], a2)));
+    };
+    if (W > 0) {
+        const int c0 = cp[0];
+        c1 = W > 1 ? cp[rp] : 0;
+        load(0, c0, vp);
+    }
+    for (int w = 0; w < W; w += 2) {
+        if (w + 1 < W) {
+            const int c = c1;
+            if (w + 2 < W) c1 = cp[(w + 2) * rp];
+            load(1, c, vp + (w + 1) * 9 * rp);
+        }
+        mac(0);
+        if (w + 1 < W) {
+            if (w + 2 < W) {
+                const int c = c1;
+                if (w + 3 < W) c1 = cp[(w + 3) * rp];
+                load(0, c, vp + (w + 2) * 9 * rp);
+            }
+            mac(1);
+        }
     }
     if (bs >= 0) {
         const double* b = st.ws + (long long)bs * st.n3p;
@@ -1392,7 +1427,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_ortho_cgs(const SysTab* __re
 }  // namespace
 
 void launch_spmv(const SysTab* tab, const RowItem* items, int nitems, cudaStream_t st) {
-    if (nitems > 0) k_spmv<<<nitems, 256, 0, st>>>(tab, items);
+    if (nitems > 0) k_spmv<<<256 / kSpmvThreads * nitems, kSpmvThreads, 0, st>>>(tab, items);
 }
 
 void launch_gather_ctl(const SysTab* tab, int n, int* out, cudaStream_t st) {
