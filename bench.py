@@ -592,7 +592,7 @@ def spmv_roofline(res, system, steps: int):
 
 
 def ortho_roofline(res, system, steps: int, m: int):
-    """Modified Gram-Schmidt (k_ortho_coop, one cooperative launch per Arnoldi step; the timer also
+    """Modified Gram-Schmidt (k_ortho_long, one cooperative launch per Arnoldi step; the timer also
     holds the small per-step control kernels).  Step j of a cycle makes j + 2 fused passes over
     the 3N-vector w, each 2 FP64 FMAs per element (w -= h v_prev; dot with the next v, or the
     norm), and one scaling pass: 4 * 3N * (j + 2) + 3N flops.  It reads v_0..v_j, w once and writes
@@ -607,7 +607,7 @@ def ortho_roofline(res, system, steps: int, m: int):
             byt += 8.0 * n3 * (j + 3)
     sec = res["prof"]["ortho_ms"] / steps * 1e-3
     ach = flops / sec / 1e12
-    return {"kernel": "k_ortho_coop", "bound": "alu", "achieved": ach, "peak": FP64_NOMINAL_TFLOPS,
+    return {"kernel": "k_ortho_long", "bound": "alu", "achieved": ach, "peak": FP64_NOMINAL_TFLOPS,
             "unit": "TFLOP/s", "frac": ach / FP64_NOMINAL_TFLOPS, "peak_kind": "nominal FP64",
             "ms_per_solve": sec * 1e3, "launch_ms": sec * 1e3 / max(1, info["iterations"]),
             "hbm_frac": byt / sec / 1e9 / peaks()[0]}

@@ -342,9 +342,9 @@ void launch_dense_scatter(const double* slot, const long long* off, const int* m
 // (items: (subdomain work item, first of 8 owned rows)) written to the apply output
 void launch_dense_restrict(const SysTab* tab, const SubDesc* subs, int nsub, cudaStream_t st);
 void launch_dense_apply(const SysTab* tab, const SubDesc* subs, const int2* items, int nitems, cudaStream_t st);
-// Nested factorisation: G and G^{-1} of every subdomain (one warp each; *err gets the first
+// Nested factorisation: G and G^{-1} of every subdomain (one CTA each; *err gets the first
 // singular G) and the line packets of the apply (nmax: largest n; prec 0 FP64, else FP32); the
-// apply z[owned] = (B_i^{-1} R_i r)[owned], one CTA of one warp per subdomain, smem = the largest
+// apply z[owned] = (B_i^{-1} R_i r)[owned], one CTA of two warps per subdomain, smem = the largest
 // nf_apply_smem of the descriptors at that ring depth
 size_t nf_work_doubles(int bx, int by, int bz);
 size_t nf_line_bytes(int bz, int prec);
