@@ -895,9 +895,10 @@ void ensure_workspace(asm_ctx* h) {
     h->d_ctl.alloc(C_NCTL * sizeof(int));
     h->d_ctl.zero(h->stream);
     // chunk partials (a dot and a Gram entry per vector of a block, and a norm); the cooperative
-    // Gram-Schmidt's per-CTA partials (classical: kCgsMax values per CTA; blocked: two sets of
-    // 2 kGsMaxBlock + 1; at most two CTAs per SM)
-    h->d_partial.alloc(std::max<size_t>((size_t)(2 * kGsMaxBlock + 1) * h->nchunk, (size_t)(4 * kGsMaxBlock + 4) * 1024) *
+    // Gram-Schmidt's per-CTA partials (classical: kCgsMax values per CTA, at most two CTAs per SM; blocked: two
+    // sets of 2 kGsMaxBlock + 1 with one CTA per SM, of 2 kGsLong + 1 with two).  1 MiB: a larger allocation is
+    // mapped by itself, which costs every second new handle 55 us in its first call.
+    h->d_partial.alloc(std::max<size_t>((size_t)(2 * kGsMaxBlock + 1) * h->nchunk, (size_t)kCgsMax * 2 * 1024) *
                        sizeof(double));
     h->ws_m = m;
     h->ws_flex = flex;
