@@ -25,6 +25,7 @@ namespace asm2 {
 
 // kind word of a packet: entries | type << 8 | log2(slots per row) << 12 | backward << 16
 enum { kPkFine = 0, kPkLump = 1, kPkLong = 2 };
+constexpr int kPkMaxEntries = 255;  // longer rows (a cell coupled to hundreds of others) are not laid out by lane
 constexpr int kPkPos = 10, kPkLanes = 30;  // positions and lanes of a packet
 constexpr int kPkIdx = 48;  // byte offset of idx in a packet (out[10], padded)
 
@@ -42,7 +43,8 @@ struct Packets {
 };
 
 // stream, chunk_off, src_f, src_c: a subdomain's chunks and the slots of its value blocks in stream order
-// (SubSym).  prec / lump32 as in build_symbolic; not for FP64 lump rows under narrower fine rows.
+// (SubSym).  prec / lump32 as in build_symbolic; not for FP64 lump rows under narrower fine rows.  P is left
+// empty where a chunk does not fit the format.
 inline void build_packets(const std::vector<unsigned char>& stream, const std::vector<long long>& chunk_off, int n_fwd,
                           const std::vector<int>& src_f, const std::vector<int>& src_c, int nf_all, int nc_all, int prec,
                           bool lump32, Packets& P) {
@@ -133,7 +135,9 @@ inline void build_packets(const std::vector<unsigned char>& stream, const std::v
                 if (warp_of[q] == w) by_warp.push_back(pks[q]);
             end[w] = (unsigned char)by_warp.size();
         }
-        if (by_warp.size() > 255) {  // (a chunk of at most 24 KB holds fewer)
+        bool fits = by_warp.size() <= 255;  // (a chunk of at most 24 KB holds fewer)
+        for (const Pk& k : by_warp) fits = fits && k.entries <= kPkMaxEntries;
+        if (!fits) {
             P = Packets();
             return;
         }

@@ -11,6 +11,7 @@ import numpy as np
 import pytest
 
 import oracle as O
+from hub_rows import hub_system
 from paper_1401_7227_gb300 import synth
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -52,3 +53,16 @@ def test_same_rows_by_lane(lib, name, prec, chunk):
     bad = lib.pk_check(geo.ctypes.data_as(C.c_void_p), s.n_cells, s.nnzb, rp.ctypes.data_as(C.c_void_p),
                        ci.ctypes.data_as(C.c_void_p), prec, chunk, err, 256)
     assert bad == 0, err.value.decode()
+
+
+@pytest.mark.parametrize("lower,prec", [(n, p) for n in (254, 255, 256, 300) for p in (0, 1, 2)] + [(512, 1), (512, 2)])
+def test_rows_of_more_entries_than_a_packet_counts(lib, lower, prec):
+    """A packet's kind word has eight bits for its entries: up to 255 the rows are there by lane, beyond it there is
+    no stream by lane and the handle applies by rows."""
+    s = hub_system(10, 10, 6, 3, lower)
+    geo = np.array([10, 10, 6, 1, 1, 1, 0, 0, 1, 1, 1, 0, 1, 1, 1], dtype=np.int32)
+    rp, ci = (np.ascontiguousarray(a, dtype=np.int32) for a in (s.row_ptr, s.col_idx))
+    err = C.create_string_buffer(256)
+    bad = lib.pk_check(geo.ctypes.data_as(C.c_void_p), s.n_cells, s.nnzb, rp.ctypes.data_as(C.c_void_p),
+                       ci.ctypes.data_as(C.c_void_p), prec, 0, err, 256)
+    assert (bad, err.value.decode()) == ((0, "") if lower <= 255 else (1, "chunk count"))
