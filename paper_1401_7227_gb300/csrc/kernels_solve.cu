@@ -1012,8 +1012,8 @@ __global__ void __launch_bounds__(32 * kPkWarps, sizeof(TF) == 8 ? 1 : 2) k_appl
             // into this CTA's shared memory, and leave
             if (tid == 0) {
                 atomicExch(st.dev_err, 7);
-                const int last = min(n_chunks, ci + slots);
-                for (int k = max(0, ci - 1); k < last; k++) mbar_wait(&bar[k % slots], (unsigned)(k / slots) & 1u);
+                const int last = pk_issued_end(ci, slots, n_chunks);
+                for (int k = ci; k < last; k++) mbar_wait(&bar[k % slots], (unsigned)(k / slots) & 1u);
             }
             return;
         }

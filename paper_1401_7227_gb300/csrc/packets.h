@@ -31,6 +31,13 @@ constexpr int kPkIdx = 48;  // byte offset of idx in a packet (out[10], padded)
 
 inline int pk_val_offset(int entries) { return (kPkIdx + 4 * kPkPos * entries + 15) & ~15; }
 
+// End of the chunks whose copies are in flight when the apply gives up at chunk ci of n: the first `slots` are issued
+// ahead, and after chunk c the copy of chunk c + slots, but not after chunk ci - 1, where the wait for ci ran out.
+__host__ __device__ inline int pk_issued_end(int ci, int slots, int n) {
+    const int end = ci > 0 ? ci - 1 + slots : slots;
+    return end < n ? end : n;
+}
+
 struct Packets {
     std::vector<unsigned char> stream;  // out and idx filled in, values zero
     std::vector<long long> chunk_off;

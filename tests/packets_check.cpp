@@ -148,3 +148,18 @@ extern "C" int pk_check(const int* geo, int n, int nnzb, const int* rp, const in
     err[errlen - 1] = 0;
     return e.empty() ? 0 : 1;
 }
+
+// The ring of k_apply_packets step by step: the wait for chunk `expire` runs out.  0 if the chunks expire ..
+// pk_issued_end - 1 are just those whose copies were issued and not waited for.
+extern "C" int pk_drain_check(int slots, int n, int expire) {
+    std::set<int> flying;
+    for (int k = 0; k < slots && k < n; k++) flying.insert(k);
+    for (int ci = 0; ci < expire; ci++) {
+        flying.erase(ci);                               // landed before chunk ci was worked on
+        const bool expired = ci + 1 == expire;          // the wait for the next one, before the refill
+        if (!expired && ci + slots < n) flying.insert(ci + slots);
+    }
+    std::set<int> drained;
+    for (int k = expire; k < pk_issued_end(expire, slots, n); k++) drained.insert(k);
+    return drained == flying ? 0 : 1;
+}

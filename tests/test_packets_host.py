@@ -66,3 +66,11 @@ def test_rows_of_more_entries_than_a_packet_counts(lib, lower, prec):
     bad = lib.pk_check(geo.ctypes.data_as(C.c_void_p), s.n_cells, s.nnzb, rp.ctypes.data_as(C.c_void_p),
                        ci.ctypes.data_as(C.c_void_p), prec, 0, err, 256)
     assert (bad, err.value.decode()) == ((0, "") if lower <= 255 else (1, "chunk count"))
+
+
+@pytest.mark.parametrize("slots", [2, 3, 5, 8])
+def test_an_expired_wait_drains_the_copies_in_flight_and_no_others(lib, slots):
+    """A wait for a copy that was never issued would poll until its own limit."""
+    for n in (1, 2, 3, 7, 20):
+        for expire in range(n):
+            assert lib.pk_drain_check(slots, n, expire) == 0, (n, expire)
