@@ -303,6 +303,8 @@ __device__ __forceinline__ void gs_sweep(const SysTab& st, long long e0, long lo
 // values are halved as the lanes are (N adds and one more per spare lane bit, against 5 N for a
 // shuffle tree per value: an FP64 add holds a sub-partition's FP64 unit for ~64 cycles); the eight
 // warps' results are added in index order.  All threads call it; sm holds 8 * 16 doubles.
+// The lanes that hold the same value all store it: with the store under a condition on the lane, nvcc 13.0 lost
+// warp 0's share of a sum once a loop around this function was unrolled (up to four groups, the third with one vector).
 template <int N>
 __device__ __forceinline__ double cta_sums(double (&v)[16], double* sm) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -323,7 +325,7 @@ __device__ __forceinline__ double cta_sums(double (&v)[16], double* sm) {
     for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
     constexpr int kRep = 32 / N;  // lanes that hold the same value
     __syncthreads();
-    if (lane % kRep == 0) sm[16 * warp + lane / kRep] = v[0];
+    sm[16 * warp + lane / kRep] = v[0];
     __syncthreads();
     double t = 0.0;
     if (threadIdx.x < N) {
@@ -751,8 +753,6 @@ __global__ void __launch_bounds__(VEC_THREADS) k_om(const SysTab* __restrict__ t
         const long long p_of_q = (long long)(om_p(st, 0) - om_q(st, 0)) * st.n3p;  // from Q_s to P_s
         __syncthreads();
         double* part = st.partial + (long long)it.chunk * kRows;
-        // (not unrolled: nvcc 13.0's full unroll of these up to four groups lost warp 0's share of a sum
-        // once a third group had one vector; a barrier on either side of cta_sums also cured it)
 #pragma unroll 1
         for (int g0 = 0; g0 < max(1, nd); g0 += kGsGroup) {
             const int nn = min(kGsGroup, nd - g0), ng = max(0, min(kGsGroup, 1 + ngram - g0));  // (entry 0: (Q_1, Q_1))
@@ -1248,6 +1248,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 1) k_ortho_short(const SysTab* __
     for (int lo = 0; lo <= j; lo += bs, turn ^= 1) {
         const GsBlock B = gs_block_at(lo, bs, j);
         double* part = part2 + turn * gs_part_set(bs);
+#pragma unroll 1
         for (int g0 = 0; g0 < B.nd; g0 += kGsGroup) {
             double acc[16], ww = 0.0;
 #pragma unroll
