@@ -144,6 +144,8 @@ struct asm_ctx {
     long long n3p = 0;
     int nchunk = 0;
     DBuf d_ws, d_scal, d_ctl, d_partial;
+    int begin_ctl[C_NCTL] = {};  // what the solve in progress started from (copied without a wait: begin_solve)
+    double begin_tol = 0.0;
     SysTab tab{};
     DBuf d_tab1, d_vec1, d_row1, d_box1;
     int n_vec1 = 0, n_row1 = 0;
@@ -1509,17 +1511,18 @@ void begin_solve(asm_ctx* h, const double* b, int on_device, double rtol, int ma
     ensure_workspace(h);
     const ScalLayout SL = ScalLayout::make(h->ws_m);
     copy_in(h, h->d_ws.as<double>() + (long long)VB * h->n3p, b, sizeof(double) * 3 * (size_t)h->N, on_device);
-    int c[C_NCTL];
-    std::memset(c, 0, sizeof(c));
+    // The handle keeps the source of both copies until its next solve begins: a copy from pageable memory may be
+    // made any time before the next wait, and the first one is in the solve, not here (one per system).
+    int* c = h->begin_ctl;
+    std::memset(c, 0, sizeof(h->begin_ctl));
     c[C_PHASE] = PH_INIT;
     c[C_APPLY_IN] = -1;
     c[C_SPMV_IN] = -1;
     c[C_MAXIT] = max_iter;
     c[C_STATUS] = ASM_ERR_NOT_CONVERGED;
-    ck(cudaMemcpyAsync(h->d_ctl.p, c, sizeof(c), cudaMemcpyHostToDevice, h->stream));
-    double tol = rtol;
-    // (copies from pageable memory return once the source is staged: c and tol may go out of scope)
-    ck(cudaMemcpyAsync(h->d_scal.as<double>() + SL.tol, &tol, sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    ck(cudaMemcpyAsync(h->d_ctl.p, c, sizeof(h->begin_ctl), cudaMemcpyHostToDevice, h->stream));
+    h->begin_tol = rtol;
+    ck(cudaMemcpyAsync(h->d_scal.as<double>() + SL.tol, &h->begin_tol, sizeof(double), cudaMemcpyHostToDevice, h->stream));
 }
 
 // x and the result of a finished (or abandoned) system; c = its control words
