@@ -400,7 +400,8 @@ typedef struct {
 
 typedef struct {
     long long submitted, admitted, completed, steps, reuse_hits, structure_builds, evictions;
-    long long resident_bytes, budget_bytes;
+    long long resident_bytes, budget_bytes; /* (the account behind the budget also holds, for each system, the
+                                             * second layout of its factors, which a later step may upload) */
     int active, pending;
     /* where the host time goes (wall clock, ms, cumulative): structure analysis on the worker
      * thread; admission (every call of it), of which building new systems (allocation, structure

@@ -118,6 +118,7 @@ struct asm_ctx {
     DBuf d_lanes, d_ln_off_f, d_ln_src_f, d_ln_off_c, d_ln_src_c;
     long long ln_nf = 0, ln_nc = 0;
     bool lanes_ok = false, rows_ready = false, rows_packed = false;
+    size_t charged = 0;  // what the server's memory account holds for this system (charge, asm_server)
     int lanes_cap = 0, lanes_smem = 0;  // its largest chunk; the largest local vectors and zero row
     DBuf d_lv, d_rlists, d_y, d_corr_cells, d_corr, d_dev_err, d_gsum, d_r32;
     int n_group_items = 0;  // box_items[0 .. n_group_items): the cell-group sums (kind 2)
@@ -1751,6 +1752,14 @@ int handle_matrix_view(asm_ctx* h, MatrixView* out) {
 
 namespace {
 
+// device bytes of a structure's stream by rows and its pack lists
+size_t rows_bytes(const SysSym& S) {
+    size_t b = 0;
+    for (const SubSym& o : S.subs)
+        b += (o.stream.size() + 255) / 256 * 256 + (sizeof(long long) + sizeof(int)) * (o.pk_off_f.size() + o.pk_off_c.size());
+    return b;
+}
+
 size_t ctx_device_bytes(const asm_ctx* h) {
     const DBuf* bufs[] = {&h->d_ell_val, &h->d_ell_col, &h->d_ell_loc, &h->d_bsr_rp, &h->d_bsr_val, &h->d_bcell,
                           &h->d_cptr, &h->d_cloc, &h->d_cval, &h->d_boxsum, &h->d_slot, &h->d_dpiv, &h->d_aptr,
@@ -1892,14 +1901,32 @@ std::string structure_key(const asm_request& q, int prec) {
     return buf;
 }
 
+// The server's memory account: what a system holds, and what the stream by rows will take where it is not on the
+// device yet (any step may need it: build_batch).  A system leaves the account with what it came in with.
+void charge(asm_server* S, asm_ctx* h) {
+    h->charged = ctx_device_bytes(h) + (h->rows_ready ? 0 : rows_bytes(*h->sym));
+    S->resident += h->charged;
+}
+void discharge_and_destroy(asm_server* S, asm_ctx* h) {
+    S->resident -= h->charged;
+    asm_destroy(h);
+}
+// what the systems hold on the device now
+long long resident_now(const asm_server* S) {
+    size_t b = 0;
+    for (const Req* r : S->active)
+        if (r->h) b += ctx_device_bytes(r->h);
+    for (const auto& kv : S->idle) b += ctx_device_bytes(kv.second);
+    return (long long)b;
+}
+
 void evict_idle(asm_server* S, size_t need) {
     while (S->resident + need > S->budget && !S->lru.empty()) {
         const long long key = S->lru.front();
         S->lru.pop_front();
         asm_ctx* h = S->idle[key];
         S->idle.erase(key);
-        S->resident -= ctx_device_bytes(h);
-        asm_destroy(h);
+        discharge_and_destroy(S, h);
         S->st.evictions++;
     }
 }
@@ -1993,8 +2020,7 @@ void admit(asm_server* S) {
             const int st = rekey_ctx(h, r);
             S->st.rekey_ms += ms_since(t0);
             if (st) {
-                S->resident -= ctx_device_bytes(h);
-                asm_destroy(h);
+                discharge_and_destroy(S, h);
                 r->info.status = st;
                 r->state = 2;
                 it = S->pending.erase(it);
@@ -2025,7 +2051,9 @@ void admit(asm_server* S) {
                 it = S->pending.erase(it);
                 continue;
             }
-            const size_t need = (size_t)r->in.n_cells * 6144;  // ~6 KB per cell resident (FP32 factors, m = 30)
+            // ~6 KB per cell resident (FP32 factors, m = 30) with one stream of the factors, and the other one
+            size_t need = (size_t)r->in.n_cells * 6144;
+            if (wants_lanes(e->sym->g, S->sms)) need += rows_bytes(*e->sym);
             evict_idle(S, need);
             if (S->resident + need > S->budget && !S->active.empty()) {
                 ++it;  // no memory now: wait for systems to finish
@@ -2050,13 +2078,13 @@ void admit(asm_server* S) {
         if (st) {
             r->info.status = st;
             r->state = 2;
-            asm_destroy(h);
+            discharge_and_destroy(S, h);
             it = S->pending.erase(it);
             continue;
         }
         r->h = h;
         r->state = 1;
-        if (fresh) S->resident += ctx_device_bytes(h);
+        if (fresh) charge(S, h);
         if (key >= 0) S->key_busy[key] = true;
         S->active.push_back(r);
         S->dirty = true;
@@ -2087,14 +2115,12 @@ void retire(asm_server* S, Req* r, const int* c) {
         while ((int)S->idle.size() > S->opt.max_cached) {
             const long long k0 = S->lru.front();
             S->lru.pop_front();
-            S->resident -= ctx_device_bytes(S->idle[k0]);
-            asm_destroy(S->idle[k0]);
+            discharge_and_destroy(S, S->idle[k0]);
             S->idle.erase(k0);
             S->st.evictions++;
         }
     } else {
-        S->resident -= ctx_device_bytes(h);
-        asm_destroy(h);
+        discharge_and_destroy(S, h);
     }
     S->st.retire_ms += ms_since(t0);
 }
@@ -2985,7 +3011,6 @@ int asm_server_progress(asm_server_handle S, int max_steps, int* n_active, int* 
     }
     if (n_active) *n_active = (int)S->active.size();
     if (n_pending) *n_pending = (int)S->pending.size();
-    S->st.resident_bytes = (long long)S->resident;
     return ASM_OK;
 }
 
@@ -3006,7 +3031,7 @@ int asm_server_result(asm_server_handle S, long long ticket, double* x, asm_solv
 int asm_server_get_stats(asm_server_handle S, asm_server_stats* out) {
     if (!S || !out) return ASM_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lk(S->mu);  // the analysis thread adds to analysis_ms
-    S->st.resident_bytes = (long long)S->resident;
+    S->st.resident_bytes = resident_now(S);
     S->st.budget_bytes = (long long)S->budget;
     S->st.active = (int)S->active.size();
     S->st.pending = (int)S->pending.size();

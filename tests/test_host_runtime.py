@@ -63,3 +63,54 @@ def test_the_words_a_solve_starts_from_outlive_their_copies(fake):
     assert fake.fk_late_stack_copies() == 0
     for sol in sols:
         sol.close()
+
+
+def serve(srv, tickets):
+    """Runs the server until every ticket has its result; the largest number of systems in flight."""
+    most, left = 0, list(tickets)
+    for _ in range(10000):
+        most = max(most, srv.progress(1)[0])
+        left = [t for t in left if srv.result(t) is None]
+        if not left:
+            return most
+    raise AssertionError("requests did not finish")
+
+
+@pytest.mark.parametrize("kept", [0, 1, 2])
+def test_server_accounts_for_factor_streams_uploaded_after_admission(fake, kept):
+    """On 2 SMs one system of four subdomains applies by lane, two together by rows, whose stream is uploaded when
+    the second one joins.  What is resident at the end is what the kept systems hold on the device."""
+    fake.fk_reset(2)
+    systems = [synth.grid_jacobian(10, 10, 5, k) for k in range(4)]
+    empty = fake.fk_live_bytes()
+    srv = asm2.Server(precision="fp32", stream=0, max_cached=kept)
+    serve(srv, [srv.submit(s, s.b, partition=(2, 2, 1), max_iter=4, matrix_key=k) for k, s in enumerate(systems)])
+    assert fake.fk_calls(b"apply_rows") > 0
+    live, st = fake.fk_live_bytes() - empty, srv.stats()
+    srv.close()
+    assert st["completed"] == 4 and st["evictions"] == (4 - kept if kept else 0)
+    tables = 64 << 10  # the server's own work-item tables
+    assert live - tables <= st["resident_bytes"] <= live
+    assert fake.fk_live_bytes() == empty
+
+
+def test_server_admits_within_its_budget_when_streams_are_uploaded_later(fake):
+    """On 2 SMs two systems of four subdomains apply by lane and three by rows.  A budget for three with one stream
+    each, but not with both: two at a time."""
+    fake.fk_reset(2)
+    systems = [synth.grid_jacobian(20, 20, 8, k) for k in range(3)]
+
+    def resident(n, budget=0):
+        srv = asm2.Server(precision="fp32", stream=0, max_cached=n, hbm_budget=budget)
+        most = serve(srv, [srv.submit(s, s.b, partition=(2, 2, 1), max_iter=40, matrix_key=k)
+                           for k, s in enumerate(systems[:n])])
+        size = srv.stats()["resident_bytes"]
+        srv.close()
+        return most, size
+
+    (_, by_lane), (most, both) = resident(1), resident(3)
+    rows = both // 3 - by_lane
+    assert most == 3 and rows > 0
+    need = 3200 * 6144  # the server's estimate for a new system with one stream
+    assert resident(3, 2 * by_lane + need + rows // 2)[0] == 2
+    assert resident(3, both + need)[0] == 3
