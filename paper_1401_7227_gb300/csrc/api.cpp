@@ -112,12 +112,12 @@ struct asm_ctx {
     DBuf d_fp;  // factor program arrays (one allocation, see upload_factor_program)
     DBuf d_stream, d_pk_off_f, d_pk_src_f, d_pk_off_c, d_pk_src_c;
     // the factor stream by lane and its pack lists (packets.h); lanes_ok: every subdomain's chunks and
-    // local vectors fit a CTA's shared memory.  The other stream is then uploaded and packed only for
-    // a handle that is asked for one of its placements (rows_ready: uploaded; rows_packed: holds the current
-    // factors).
+    // local vectors fit a CTA's shared memory.  The other stream is then uploaded only for a handle that is asked
+    // for one of its placements (rows_ready).  A factorisation fills the stream that the last apply read
+    // (by_rows), and use_stream the other one when an apply needs it (*_packed: holds the current factors).
     DBuf d_lanes, d_ln_off_f, d_ln_src_f, d_ln_off_c, d_ln_src_c;
     long long ln_nf = 0, ln_nc = 0;
-    bool lanes_ok = false, rows_ready = false, rows_packed = false;
+    bool lanes_ok = false, lanes_packed = false, rows_ready = false, rows_packed = false, by_rows = false;
     size_t charged = 0;  // what the server's memory account holds for this system (charge, asm_server)
     int lanes_cap = 0, lanes_smem = 0;  // its largest chunk; the largest local vectors and zero row
     DBuf d_lv, d_rlists, d_y, d_corr_cells, d_corr, d_dev_err, d_gsum, d_r32;
@@ -597,6 +597,14 @@ void upload_rows(asm_ctx* h) {
     h->rows_ready = true;
     h->rows_packed = false;
 }
+void pack_lanes(asm_ctx* h) {
+    launch_pack_lanes(h->d_ln_off_f.as<long long>(), h->d_ln_src_f.as<int>(), h->ln_nf, h->prec,
+                      h->d_lanes.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
+    launch_pack_lanes(h->d_ln_off_c.as<long long>(), h->d_ln_src_c.as<int>(), h->ln_nc, h->lump32 ? 1 : 0,
+                      h->d_lanes.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
+    ck(cudaGetLastError());
+    h->lanes_packed = true;
+}
 void pack_rows(asm_ctx* h) {
     launch_pack(h->d_pk_off_f.as<long long>(), h->d_pk_src_f.as<int>(), h->pk_nf, h->prec, h->d_stream.as<unsigned char>(),
                 h->d_slot.as<double>(), h->stream);
@@ -607,9 +615,14 @@ void pack_rows(asm_ctx* h) {
 }
 // before a launch of configuration cfg: the stream it reads holds the current factors
 void use_stream(asm_ctx* h, const ApplyConfig& cfg) {
-    if (cfg.ymode == Y_PACKET || h->opt.local_solver == ASM_LOCAL_EXACT || is_nf(h)) return;
-    if (!h->rows_ready) upload_rows(h);
-    if (!h->rows_packed) pack_rows(h);
+    if (h->opt.local_solver == ASM_LOCAL_EXACT || is_nf(h)) return;
+    if (cfg.ymode == Y_PACKET) {
+        if (!h->lanes_packed) pack_lanes(h);
+    } else {
+        if (!h->rows_ready) upload_rows(h);
+        if (!h->rows_packed) pack_rows(h);
+    }
+    h->by_rows = cfg.ymode != Y_PACKET;  // (only now: an upload may have failed)
 }
 void upload_symbolic(asm_ctx* h) {
     SysSym& S = *h->sym;
@@ -719,7 +732,7 @@ void upload_symbolic(asm_ctx* h) {
     ck(cudaDeviceGetAttribute(&h->sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device));
     ck(cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, h->device));
     h->lanes_cap = h->lanes_smem = 0;
-    h->rows_ready = h->rows_packed = false;
+    h->rows_ready = h->rows_packed = h->lanes_packed = h->by_rows = false;
     h->d_stream.alloc(16);
     std::vector<long long> lane_base(K + 1, 0);
     bool lanes = K > 0;
@@ -1128,14 +1141,11 @@ int factor_numeric(asm_ctx* h) {
     } else {
         launch_factor(h->d_factdesc.as<FactDesc>(), (int)S.subs.size(), h->n_sms, h->d_err.as<FactErr>(), nullptr,
                       h->stream);
-        if (h->lanes_ok) {
-            launch_pack_lanes(h->d_ln_off_f.as<long long>(), h->d_ln_src_f.as<int>(), h->ln_nf, h->prec,
-                              h->d_lanes.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
-            launch_pack_lanes(h->d_ln_off_c.as<long long>(), h->d_ln_src_c.as<int>(), h->ln_nc, h->lump32 ? 1 : 0,
-                              h->d_lanes.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
-        }
-        h->rows_packed = false;
-        if (h->rows_ready) pack_rows(h);
+        h->lanes_packed = h->rows_packed = false;
+        if (h->lanes_ok && !h->by_rows)
+            pack_lanes(h);
+        else
+            pack_rows(h);
     }
     ck(cudaGetLastError());
     ck(cudaEventRecord(e1, h->stream));

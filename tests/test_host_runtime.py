@@ -114,3 +114,41 @@ def test_server_admits_within_its_budget_when_streams_are_uploaded_later(fake):
     need = 3200 * 6144  # the server's estimate for a new system with one stream
     assert resident(3, 2 * by_lane + need + rows // 2)[0] == 2
     assert resident(3, both + need)[0] == 3
+
+
+def test_a_new_factorisation_packs_the_one_stream_in_use(fake):
+    """On 2 SMs one system applies by lane and three together by rows.  Each factorisation fills the stream that the
+    last apply read; the other is filled when an apply needs it again, once."""
+    fake.fk_reset(2)
+    systems = [synth.grid_jacobian(10, 10, 5, k) for k in range(3)]
+    sols = [make_solver(s, (2, 2, 1), precision="fp32") for s in systems]
+
+    def packs():
+        by_rows, by_lane = fake.fk_calls(b"pack"), fake.fk_calls(b"pack_lanes")
+        fake.fk_reset(2)
+        return by_rows, by_lane
+
+    def new_values():
+        for s, sol in zip(systems, sols):
+            sol.update_values(s.vals)
+            sol.factor()
+
+    def batch():
+        asm2.solve_batch(sols, [s.b for s in systems], max_iter=3)
+
+    # (two launches fill a stream: fine rows, lump rows)
+    assert packs() == (0, 6)                       # new systems: by lane
+    batch()
+    assert fake.fk_calls(b"apply_rows") > 0 and packs() == (6, 0)
+    new_values()
+    batch()
+    assert packs() == (6, 0)
+    sols[0].solve(systems[0].b, max_iter=3)
+    assert fake.fk_calls(b"apply_lanes") > 0 and packs() == (0, 2)
+    sols[0].solve(systems[0].b, max_iter=3)
+    batch()
+    assert packs() == (0, 0)                       # both hold the current factors
+    new_values()
+    assert packs() == (6, 0)
+    for sol in sols:
+        sol.close()
