@@ -7,6 +7,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <map>
+#include <mutex>
+#include <utility>
+
 namespace asm2 {
 
 // ---------------------------------------------------------------------------------------------
@@ -256,6 +260,18 @@ struct NFDesc {
 // ---------------------------------------------------------------------------------------------
 // Kernel launchers (kernels.cu)
 // ---------------------------------------------------------------------------------------------
+// Lets launches of a kernel use that much dynamic shared memory.  The limit belongs to the function on a device, not
+// to a launch, so it only grows: a handle on another thread may be between its own call and its launch.
+inline void allow_dynamic_smem(const void* kernel, int bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, int> allowed;
+    int device = 0;
+    cudaGetDevice(&device);
+    std::lock_guard<std::mutex> lk(mu);
+    int& most = allowed[{device, kernel}];
+    if (most < bytes && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess)
+        most = bytes;
+}
 // slot values of the local matrices from the array-of-blocks copy of A (lists of BSR block indices,
 // ~index for a subtracted block); slots whose lists hold kLongAssembly or more blocks are
 // summed by a warp each (long_slots, nlong; null: every slot by the per-element kernel)

@@ -890,7 +890,7 @@ __global__ void __launch_bounds__(64) k_nf_apply(const SysTab* __restrict__ tab,
 
 template <typename T, int SLOTS>
 void nf_apply_t(const SysTab* tab, const NFDesc* descs, int ndesc, size_t smem, cudaStream_t st) {
-    cudaFuncSetAttribute(k_nf_apply<T, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem((const void*)k_nf_apply<T, SLOTS>, (int)smem);
     k_nf_apply<T, SLOTS><<<ndesc, 64, smem, st>>>(tab, descs);
 }
 
@@ -934,7 +934,7 @@ void nf_factor_t(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec,
     // against 1,008 and 672 here) and its plane vectors do
     const int stages = nf_factor_smem(bz_max, prec, 2) <= (size_t)dev_smem - 1024 ? 2 : 1;
     const size_t smem = nf_factor_smem(bz_max, prec, stages);
-    cudaFuncSetAttribute(k_nf_factor<TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem((const void*)k_nf_factor<TC>, (int)smem);
     k_nf_gather<TC><<<ggrid, 128, 0, st>>>(descs);
     k_nf_factor<TC><<<ndesc, kNfThreads, smem, st>>>(descs, stages, err);
     k_nf_pack<TC><<<grid, 128, 0, st>>>(descs);

@@ -1093,11 +1093,7 @@ ApplyConfig apply_local_vectors(int nsub, int all_bytes, int lump_bytes, int sme
 namespace {
 template <typename TF, typename TL, int YM, int SLOTS>
 void launch_apply_t(const SysTab* tab, const SubDesc* subs, int nsub, int smem, cudaStream_t st, int* occ) {
-    static int configured = -1;
-    if (configured < smem) {
-        cudaFuncSetAttribute(k_apply<TF, TL, YM, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        configured = smem;
-    }
+    allow_dynamic_smem((const void*)k_apply<TF, TL, YM, SLOTS>, smem);
     const int threads = YM == Y_SMEM ? 256 : kApplyThreadsDev;
     if (occ != nullptr) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k_apply<TF, TL, YM, SLOTS>, threads, smem) != cudaSuccess)
@@ -1117,12 +1113,8 @@ void launch_apply_s(const SysTab* tab, const SubDesc* subs, int nsub, int smem, 
 }
 template <typename TF>
 void launch_apply_packets(const SysTab* tab, const SubDesc* subs, int nsub, ApplyConfig cfg, cudaStream_t st, int* occ) {
-    static int configured = -1;
     const int smem = (int)apply_ring_bytes(cfg.slots, cfg.chunk) + cfg.smem;
-    if (configured < smem) {
-        cudaFuncSetAttribute(k_apply_packets<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        configured = smem;
-    }
+    allow_dynamic_smem((const void*)k_apply_packets<TF>, smem);
     if (occ != nullptr) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k_apply_packets<TF>, 32 * kPkWarps, smem) != cudaSuccess) *occ = 0;
         return;
