@@ -857,11 +857,15 @@ __global__ void __launch_bounds__(VEC_THREADS) k_om(const SysTab* __restrict__ t
         double* gram = st.scal + SL.gram;  // entry (slot, distance): the product with the direction that much older
         if (b == 0 && i >= 1 && i < nd) gram[dir(1) * kB + i] = tot[nd + i];
         __syncwarp();
-        double c = i < nd ? tot[i] : 0.0;
-        const double inv = i < nd ? 1.0 / st.scal[SL.om_qq + dir(lo + i)] : 0.0;
+        // One reciprocal per lane, not a division per link of the chain.  1 / (Q_l, Q_l) overflows below 2^-1024 (a
+        // right-hand side of 1e-150, eight digits later), so a small (Q_l, Q_l) and the products that its
+        // reciprocal multiplies are scaled by a power of two, which leaves their bits alone.
+        const double qq = i < nd ? st.scal[SL.om_qq + dir(lo + i)] : 1.0, sc = qq < 0x1p-1000 ? 0x1p600 : 1.0;
+        const double inv = i < nd ? 1.0 / (qq * sc) : 0.0;
+        double c = i < nd ? tot[i] * sc : 0.0;
         for (int k = 0; k + 1 < nd; k++) {
             const double beta = __shfl_sync(0xffffffffu, c * inv, k);
-            if (i > k && i < nd) c = fma(-gram[dir(lo + k) * kB + i - k], beta, c);
+            if (i > k && i < nd) c = fma(-(gram[dir(lo + k) * kB + i - k] * sc), beta, c);
         }
         if (i < nd) st.scal[SL.om_beta + lo - 1 + i] = c * inv;
     } else if (ph == PH_INIT || ph == PH_OM_FINAL) {
