@@ -119,8 +119,8 @@ __global__ void __launch_bounds__(VEC_THREADS) k_coarse_prolong(const SysTab* __
     const SysTab& st = tab[it.sys];
     if (st.cmode == 0 || st.ctl[C_APPLY_IN] < 0) return;
     double* z = st.ws + (long long)st.ctl[C_APPLY_OUT] * st.n3p;
-    const long long e0 = (long long)it.chunk * VEC_CHUNK;
-    for (int i = threadIdx.x; i < VEC_CHUNK; i += blockDim.x) {
+    const long long e0 = (long long)it.chunk * st.vchunk;
+    for (int i = threadIdx.x; i < st.vchunk; i += blockDim.x) {
         const long long e = e0 + i;
         if (e >= st.n3) break;
         const long long cell = e / 3;
