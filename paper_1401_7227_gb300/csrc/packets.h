@@ -71,6 +71,11 @@ inline void build_packets(const std::vector<unsigned char>& stream, const std::v
         size_t bytes;
     };
     P = Packets();
+    P.stream.reserve(stream.size() / 2 * 3);
+    P.off_f.reserve(src_f.size());
+    P.src_f.reserve(src_f.size());
+    P.off_c.reserve(src_c.size());
+    P.src_c.reserve(src_c.size());
     size_t kf = 0, kc = 0;
     std::vector<Row> rows;
     std::vector<Pk> pks;

@@ -121,6 +121,34 @@ struct Ctx {
     std::vector<long long> ckey;  // sorted unique far-box pair keys of C
 };
 
+// std::stable_sort of T, whose rows are 0 .. n - 1: distributed over the rows, which are short, then each row sorted
+// (one sort of all entries was a quarter of the analysis of 128 x 128 x 32 cells, 2.17 s on one thread; now 2.00).
+void sort_entries(std::vector<Tup>& T, int n) {
+    std::vector<size_t> at((size_t)n + 1, 0);
+    for (const Tup& t : T) at[t.p + 1]++;
+    for (int p = 0; p < n; p++) at[p + 1] += at[p];
+    std::vector<Tup> by_row(T.size());
+    {
+        std::vector<size_t> fill(at.begin(), at.end() - 1);
+        for (const Tup& t : T) by_row[fill[t.p]++] = t;
+    }
+    for (int p = 0; p < n; p++) {
+        Tup* r = by_row.data() + at[p];
+        const size_t len = at[p + 1] - at[p];
+        if (len > 32) {
+            std::stable_sort(r, r + len);
+            continue;
+        }
+        for (size_t i = 1; i < len; i++) {
+            const Tup t = r[i];
+            size_t k = i;
+            for (; k > 0 && t < r[k - 1]; k--) r[k] = r[k - 1];
+            r[k] = t;
+        }
+    }
+    T.swap(by_row);
+}
+
 std::string build_sub(const Ctx& X, int s, SubSym& o) {
     const Geom& g = X.g;
     const Pattern& A = X.A;
@@ -253,7 +281,7 @@ std::string build_sub(const Ctx& X, int s, SubSym& o) {
             if (S.cptr[c + 1] - S.cptr[c] > e2) T.push_back({flump[J], flump[Jp], c, 2});
         }
     }
-    std::stable_sort(T.begin(), T.end());
+    sort_entries(T, idx);
 
     // slots
     o.prp.assign(n + 1, 0);
