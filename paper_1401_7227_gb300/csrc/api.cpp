@@ -541,7 +541,11 @@ void choose_ring(asm_ctx* h) {
 // vectors in device memory (four), so launches of more than two waves keep those: 128x128x32 in 256
 // subdomains, 1.7 waves, one apply: 490 against 612 us in FP64, 231 / 245 in FP32, 227 / 231 in FP16; 128x128x64 in
 // 512, 3.4 waves: 1055 / 957, 479 / 367, 485 / 341.
-int lane_slots(const asm_ctx* h, int nsub, int smem, int chunk) {
+// In FP32 and FP16 a second wave of single CTAs loses against the stream by rows (rows: the configuration it would
+// have) where that runs every subdomain at once from shared memory: an apply of 128x128x32 in 256 subdomains of
+// overlap 1 in FP32 265 against 229 us, 105x105x31 in 169 248 / 215, in FP16 271 / 241; with a row of 80 blocks at
+// 96x96x16 in 256, whose chunks by lane are large, 192 / 163.  In FP64 it does not (96x96x16: 269 / 273).
+int lane_slots(const asm_ctx* h, int nsub, int smem, int chunk, const ApplyConfig& rows) {
     const int sms = std::max(1, h->n_sms), most = h->prec == 0 ? 1 : 2;
     const auto fits = [&](int sl, int ctas) {
         const size_t cta = (size_t)smem + apply_ring_bytes(sl, chunk) + 1024;
@@ -549,10 +553,17 @@ int lane_slots(const asm_ctx* h, int nsub, int smem, int chunk) {
     };
     for (int c = std::min(most, (nsub + sms - 1) / sms); c >= 1; c--) {
         if (nsub > 2LL * c * sms) break;
+        if (c < most && nsub > sms && rows.ymode == Y_SMEM) return 0;
         for (int sl = kMaxPacketSlots; sl >= 3; sl--)
             if (fits(sl, c)) return sl;
     }
     return nsub <= 2LL * sms && fits(2, 1) ? 2 : 0;
+}
+
+// the by-rows configuration of a launch of a handle's subdomains, place as ASM_TUNE_APPLY_SMEM stores it (0 automatic)
+ApplyConfig single_rows_config(const asm_ctx* h, int place) {
+    return apply_local_vectors((int)h->sym->subs.size(), h->apply_smem, h->apply_lump_smem, h->apply_slots, h->chunk_cap,
+                               h->sm_smem, h->n_sms, place, other_slots(h));
 }
 
 // f(s) for every subdomain s, on several threads when there are that many items (f does not throw)
@@ -755,6 +766,14 @@ void upload_symbolic(asm_ctx* h) {
     ck(cudaDeviceGetAttribute(&h->dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     ck(cudaDeviceGetAttribute(&h->sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device));
     ck(cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, h->device));
+    h->apply_smem_need = h->apply_lump_smem = 0;
+    h->chunk_cap = kStreamChunkMin;
+    for (const SubSym& o : S.subs) {
+        h->apply_smem_need = std::max(h->apply_smem_need, (int)apply_smem_bytes(o.nf, o.n - o.nf, S.prec, S.lump32));
+        h->apply_lump_smem = std::max(h->apply_lump_smem, (int)apply_lump_bytes(o.n - o.nf, S.prec, S.lump32));
+        h->chunk_cap = std::max(h->chunk_cap, o.chunk_cap);
+    }
+    choose_ring(h);
     h->lanes_cap = h->lanes_smem = 0;
     h->rows_ready = h->rows_packed = h->lanes_packed = h->by_rows = false;
     h->d_stream.alloc(16);
@@ -767,7 +786,8 @@ void upload_symbolic(asm_ctx* h) {
         h->lanes_cap = std::max(h->lanes_cap, (o.pk.cap + 127) / 128 * 128);
         h->lanes_smem = std::max(h->lanes_smem, (int)apply_smem_bytes(o.nf, o.n - o.nf, S.prec, S.lump32) + 32);
     }
-    h->lanes_ok = lanes && lane_slots(h, 1, h->lanes_smem, h->lanes_cap) > 0;
+    // (for the handle's own launch: what it does not take there it would only carry)
+    h->lanes_ok = lanes && lane_slots(h, K, h->lanes_smem, h->lanes_cap, single_rows_config(h, 0)) > 0;
     h->d_rlists.alloc((size_t)std::max<long long>(2, rl_base[K]) * 4);
     std::vector<BoxItem> corr_items;
     std::vector<int> corr_cells;
@@ -804,10 +824,6 @@ void upload_symbolic(asm_ctx* h) {
     }
     h->sub_desc.assign(K, SubDesc{});
     h->sub_cost.assign(K, 0.0);
-    h->apply_smem = 0;
-    h->apply_smem_need = 0;
-    h->apply_lump_smem = 0;
-    h->chunk_cap = kStreamChunkMin;
     h->tuned_ymode = -1;
     for (int s = 0; s < K; s++) {
         const SubSym& o = S.subs[s];
@@ -835,7 +851,6 @@ void upload_symbolic(asm_ctx* h) {
         sd.n_long = (int)o.clong.size();
         sd.corr0 = corr_base;
         sd.chunk_cap = o.chunk_cap;
-        h->chunk_cap = std::max(h->chunk_cap, o.chunk_cap);
         sd.pk_cap = (o.pk.cap + 127) / 128 * 128;
         sd.pk_stream = h->d_lanes.as<unsigned char>() + lane_base[s];
         sd.y = h->d_y.as<double>() + h->y_base[s];
@@ -870,8 +885,6 @@ void upload_symbolic(asm_ctx* h) {
         sd.clong = put(o.clong);
         sd.own_pos = put(o.own_pos);
         sd.own_cell = put(o.own_cell);
-        h->apply_smem_need = std::max<int>(h->apply_smem_need, (int)apply_smem_bytes(o.nf, o.n - o.nf, S.prec, S.lump32));
-        h->apply_lump_smem = std::max<int>(h->apply_lump_smem, (int)apply_lump_bytes(o.n - o.nf, S.prec, S.lump32));
         for (size_t k = 0; k + 1 < o.corr_ptr.size(); k++)
             corr_items.push_back(BoxItem{0, corr_base + (int)k, (int)corr_cells.size() + o.corr_ptr[k],
                                          (int)corr_cells.size() + o.corr_ptr[k + 1], 1, 0, nullptr});
@@ -1327,12 +1340,12 @@ void build_batch(Batch& B, cudaStream_t st) {
         lanes_smem = std::max(lanes_smem, h->lanes_smem);
         lanes_cap = std::max(lanes_cap, h->lanes_cap);
     }
-    const int ls = lanes ? lane_slots(B.hs[0], B.nsub, lanes_smem, lanes_cap) : 0;
-    if (ls > 0)
-        B.apply = ApplyConfig{Y_PACKET, lanes_smem, ls, lanes_cap};
-    else if (!B.hs.empty())
+    if (!B.hs.empty()) {
         B.apply = apply_local_vectors(B.nsub, all_bytes, lump_bytes, B.slots, B.chunk, B.hs[0]->sm_smem,
                                       B.hs[0]->n_sms, B.hs[0]->apply_place, other_slots(B.hs[0]));
+        const int ls = lanes ? lane_slots(B.hs[0], B.nsub, lanes_smem, lanes_cap, B.apply) : 0;
+        if (ls > 0) B.apply = ApplyConfig{Y_PACKET, lanes_smem, ls, lanes_cap};
+    }
     for (asm_ctx* h : B.hs) use_stream(h, B.apply);  // (may move a handle's descriptors: before they are copied)
 
     sd = longest_first(B.hs);
@@ -2384,11 +2397,10 @@ int placement_code(int ymode) { return ymode == Y_SMEM || ymode == Y_PACKET ? 3 
 // the placement of a single-system apply: `place` as ASM_TUNE_APPLY_SMEM stores it (0 automatic)
 ApplyConfig single_apply_config(const asm_ctx* h, int place) {
     if (place == 0 && h->lanes_ok && h->slots_force == 0) {
-        const int ls = lane_slots(h, (int)h->sub_desc.size(), h->lanes_smem, h->lanes_cap);
+        const int ls = lane_slots(h, (int)h->sub_desc.size(), h->lanes_smem, h->lanes_cap, single_rows_config(h, 0));
         if (ls > 0) return ApplyConfig{Y_PACKET, h->lanes_smem, ls, h->lanes_cap};
     }
-    return apply_local_vectors((int)h->sub_desc.size(), h->apply_smem, h->apply_lump_smem, h->apply_slots,
-                               h->chunk_cap, h->sm_smem, h->n_sms, place, other_slots(h));
+    return single_rows_config(h, place);
 }
 
 // R_i r and the fused ILU sweeps of every subdomain (after k_sums), single-system tables

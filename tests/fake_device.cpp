@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <pthread.h>
 
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 #include <map>
@@ -104,7 +105,11 @@ namespace asm2 {
 size_t apply_ring_bytes(int slots, int chunk) { return (size_t)slots * chunk + 128; }
 size_t apply_smem_bytes(int nf, int nc, int prec, bool lump32) { return y_layout(nf, nc, prec, lump32).total; }
 size_t apply_lump_bytes(int nf, int nc, bool mirror) { return y_layout(nf, nc, 0, false).fine * (mirror ? 2 : 1); }
-ApplyConfig apply_local_vectors(int, int, int, int, int chunk, int, int, int, int) { return {Y_DEVICE, 0, 2, chunk}; }
+ApplyConfig apply_local_vectors(int nsub, int all, int, int slots, int chunk, int sm_smem, int n_sms, int force, int) {
+    const int fit = all > 0 ? std::min(2, sm_smem / (all + (int)apply_ring_bytes(slots, chunk) + 1024)) : 0;
+    if (force == 0 && fit >= 1 && nsub <= fit * n_sms) return {Y_SMEM, all, slots, chunk};
+    return {Y_DEVICE, 0, 2, chunk};
+}
 int ortho_coop_grid(int, int, int) { return 0; }
 int noalloc_prepare(int) { return 0; }
 

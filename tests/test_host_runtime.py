@@ -152,3 +152,20 @@ def test_a_new_factorisation_packs_the_one_stream_in_use(fake):
     assert packs() == (6, 0)
     for sol in sols:
         sol.close()
+
+
+@pytest.mark.parametrize("precision,nz,form", [("fp32", 8, "lanes"),    # two CTAs per SM: one wave
+                                               ("fp32", 40, "rows"),    # one by lane, two by rows
+                                               ("fp16s", 44, "rows"),
+                                               ("fp32", 64, "lanes"),   # one either way
+                                               ("fp64", 40, "lanes")])
+def test_a_second_wave_by_lane_gives_way_to_one_by_rows(fake, precision, nz, form):
+    """Four subdomains on 3 SMs, with more local rows the taller the boxes."""
+    fake.fk_reset(3)
+    s = synth.grid_jacobian(18, 18, nz, 1)
+    sol = make_solver(s, (2, 2, 1), precision=precision)
+    sol.solve(s.b, max_iter=3)
+    other = "rows" if form == "lanes" else "lanes"
+    assert fake.fk_calls(f"apply_{form}".encode()) > 0 and fake.fk_calls(f"apply_{other}".encode()) == 0
+    assert fake.fk_calls(b"pack_lanes") == (2 if form == "lanes" else 0)
+    sol.close()
