@@ -116,7 +116,7 @@ struct asm_ctx {
     DBuf d_slot, d_dpiv, d_aptr, d_aloc, d_acs, d_along;
     int n_along = 0;  // slots whose assembly lists are summed by a warp each
     DBuf d_fp;  // factor program arrays (one allocation, see upload_factor_program)
-    DBuf d_stream, d_pk_off_f, d_pk_src_f, d_pk_off_c, d_pk_src_c;
+    DBuf d_stream;  // the factor stream by rows, then its pack lists: offsets (fine rows, lump rows), slots (the same)
     // the factor stream by lane and its pack lists (packets.h); lanes_ok: every subdomain's chunks and
     // local vectors fit a CTA's shared memory.  The other stream is then uploaded only for a handle that is asked
     // for one of its placements (rows_ready).  A factorisation fills the stream that the last apply read
@@ -566,15 +566,15 @@ ApplyConfig single_rows_config(const asm_ctx* h, int place) {
                                h->sm_smem, h->n_sms, place, other_slots(h));
 }
 
-// f(s) for every subdomain s, on several threads when there are that many items (f does not throw)
+// f(0) .. f(n - 1), on several threads when they make up that many items (f does not throw)
 template <class F>
-void for_subdomains(int K, size_t items, F f) {
+void for_each_task(int n, size_t items, F f) {
     std::atomic<int> next{0};
     const auto work = [&] {
-        for (int s = next++; s < K; s = next++) f(s);
+        for (int t = next++; t < n; t = next++) f(t);
     };
     std::vector<std::thread> pool;
-    const int threads = items < (1 << 17) ? 0 : std::min(K, (int)std::thread::hardware_concurrency()) - 1;
+    const int threads = items < (1 << 17) ? 0 : std::min(n, (int)std::thread::hardware_concurrency()) - 1;
     pool.reserve(std::max(0, threads));
     try {
         for (int t = 0; t < threads; t++) pool.emplace_back(work);
@@ -599,38 +599,107 @@ void upload_sub_tables(asm_ctx* h) {
     sync(h);
 }
 
-// The factor stream by rows and its pack lists onto the device, for the launches that take it (use_rows)
-void upload_rows(asm_ctx* h) {
-    const SysSym& S = *h->sym;
-    cudaStream_t st = h->stream;
-    const int K = (int)S.subs.size();
-    std::vector<long long> offf, offc;
-    std::vector<int> srcf, srcc;
-    h->d_stream.alloc((size_t)h->stream_base[K]);
-    for (int s = 0; s < K; s++) {
-        const SubSym& o = S.subs[s];
-        if (!o.stream.empty())
-            ck(cudaMemcpyAsync(h->d_stream.as<unsigned char>() + h->stream_base[s], o.stream.data(), o.stream.size(),
-                               cudaMemcpyHostToDevice, st));
+// The factor streams by rows and their pack lists onto the device, for the launches that take them (use_stream).  Of a
+// stream only the indices go there, a sixteenth of it; its values come from the factors.  The lists -- twelve bytes a
+// block of the local matrices -- and the indices are written by several threads over the subdomains of all the
+// systems into untouched memory, and each system has one allocation and one copy.  The first solve of a batch of 56
+// systems (654 subdomains, FP64, 316 MB of streams) takes 40 ms with ~10 of these; with whole streams, growing vectors
+// and an allocation per list 71 with 41.
+void upload_rows(const std::vector<asm_ctx*>& hs) {
+    struct Part {  // of one subdomain: first entries in its system's lists, pieces and index bytes; then their numbers
+        int sys, sub;
+        size_t f0, c0, p0, b0, pieces, bytes;
+    };
+    struct Image {  // what a system's allocation holds behind the stream
+        asm_ctx* h;
+        size_t nf, nc, pieces, bytes;
+        std::unique_ptr<unsigned char[]> host;
+        std::vector<SubDesc> ordered;
+        long long* off_f() const { return reinterpret_cast<long long*>(host.get()); }
+        long long* off_c() const { return off_f() + nf; }
+        int* src_f() const { return reinterpret_cast<int*>(off_c() + nc); }
+        int* src_c() const { return src_f() + nf; }
+        size_t piece0() const { return (sizeof(long long) + sizeof(int)) * (nf + nc); }
+        size_t byte0() const { return (piece0() + sizeof(PkPiece) * pieces + 15) & ~(size_t)15; }
+        size_t size() const { return byte0() + bytes; }
+    };
+    std::vector<Image> images;
+    std::vector<Part> parts;
+    size_t items = 0;
+    for (asm_ctx* h : hs) {
+        const int K = (int)h->sym->subs.size();
+        for (int s = 0; s < K; s++) {
+            parts.push_back(Part{(int)images.size(), s, 0, 0, 0, 0, 0, 0});
+            items += h->sym->subs[s].pk_off_f.size() + h->sym->subs[s].pk_off_c.size();
+        }
+        images.push_back(Image{h, 0, 0, 0, 0, nullptr, {}});
+    }
+    const auto each_piece = [&](const Part& q, auto add) {
+        const asm_ctx* h = images[q.sys].h;
+        const SubSym& o = h->sym->subs[q.sub];
+        rows_index_pieces(o.stream, o.chunk_off, o.n_fwd_chunks, h->prec, add);
+    };
+    for_each_task((int)parts.size(), items, [&](int t) {
+        each_piece(parts[t], [&](long long, size_t n) {
+            parts[t].pieces++;
+            parts[t].bytes += n;
+        });
+    });
+    for (Part& q : parts) {
+        Image& im = images[q.sys];
+        const SubSym& o = im.h->sym->subs[q.sub];
+        q.f0 = im.nf, q.c0 = im.nc, q.p0 = im.pieces, q.b0 = im.bytes;
+        im.nf += o.pk_off_f.size(), im.nc += o.pk_off_c.size(), im.pieces += q.pieces, im.bytes += q.bytes;
+    }
+    for (Image& im : images) im.host.reset(new unsigned char[im.size() + 16]);
+    for_each_task((int)parts.size(), items, [&](int t) {
+        const Part& q = parts[t];
+        const Image& im = images[q.sys];
+        const SubSym& o = im.h->sym->subs[q.sub];
+        const long long stream0 = im.h->stream_base[q.sub], slot0 = im.h->slot_base[q.sub];
         for (size_t i = 0; i < o.pk_off_f.size(); i++) {
-            offf.push_back(h->stream_base[s] + o.pk_off_f[i]);
-            srcf.push_back((int)(h->slot_base[s] + o.pk_src_f[i]));
+            im.off_f()[q.f0 + i] = stream0 + o.pk_off_f[i];
+            im.src_f()[q.f0 + i] = (int)(slot0 + o.pk_src_f[i]);
         }
         for (size_t i = 0; i < o.pk_off_c.size(); i++) {
-            offc.push_back(h->stream_base[s] + o.pk_off_c[i]);
-            srcc.push_back((int)(h->slot_base[s] + o.pk_src_c[i]));
+            im.off_c()[q.c0 + i] = stream0 + o.pk_off_c[i];
+            im.src_c()[q.c0 + i] = (int)(slot0 + o.pk_src_c[i]);
         }
+        PkPiece* piece = reinterpret_cast<PkPiece*>(im.host.get() + im.piece0()) + q.p0;
+        size_t at = q.b0;
+        each_piece(q, [&](long long off, size_t n) {
+            *piece++ = PkPiece{(int)((stream0 + off) / 16), (int)(at / 16), (int)(n / 16)};
+            std::memcpy(im.host.get() + im.byte0() + at, o.stream.data() + off, n);
+            at += n;
+        });
+    });
+    struct Wait {  // the images outlive their copies, also when an allocation fails
+        const std::vector<asm_ctx*>& hs;
+        ~Wait() {
+            for (asm_ctx* h : hs) cudaStreamSynchronize(h->stream);
+        }
+    } wait{hs};
+    for (Image& im : images) {
+        asm_ctx* h = im.h;
+        const int K = (int)h->sym->subs.size();
+        const size_t stream = (size_t)h->stream_base[K];
+        h->d_stream.alloc(stream + im.size());
+        unsigned char* base = h->d_stream.as<unsigned char>();
+        ck(cudaMemsetAsync(base, 0, stream, h->stream));
+        ck(cudaMemcpyAsync(base + stream, im.host.get(), im.size(), cudaMemcpyHostToDevice, h->stream));
+        launch_place(reinterpret_cast<const PkPiece*>(base + stream + im.piece0()), (int)im.pieces, base + stream + im.byte0(),
+                     base, h->stream);
+        ck(cudaGetLastError());
+        h->pk_nf = (long long)im.nf;
+        h->pk_nc = (long long)im.nc;
+        for (int s = 0; s < K; s++) h->sub_desc[s].stream = base + h->stream_base[s];
+        if (h->d_subdesc_single.p) {  // (not yet there while a structure is set up: upload_sub_tables)
+            im.ordered = longest_first({h});
+            h->d_subdesc_single.upload_reuse(im.ordered, h->stream);
+        }
+        h->rows_ready = true;
+        h->rows_packed = false;
     }
-    h->pk_nf = (long long)offf.size();
-    h->pk_nc = (long long)offc.size();
-    h->d_pk_off_f.upload(offf, st);
-    h->d_pk_src_f.upload(srcf, st);
-    h->d_pk_off_c.upload(offc, st);
-    h->d_pk_src_c.upload(srcc, st);
-    for (int s = 0; s < K; s++) h->sub_desc[s].stream = h->d_stream.as<unsigned char>() + h->stream_base[s];
-    upload_sub_tables(h);
-    h->rows_ready = true;
-    h->rows_packed = false;
 }
 void pack_lanes(asm_ctx* h) {
     launch_pack_lanes(h->d_ln_off_f.as<long long>(), h->d_ln_src_f.as<int>(), h->ln_nf, h->prec,
@@ -641,23 +710,28 @@ void pack_lanes(asm_ctx* h) {
     h->lanes_packed = true;
 }
 void pack_rows(asm_ctx* h) {
-    launch_pack(h->d_pk_off_f.as<long long>(), h->d_pk_src_f.as<int>(), h->pk_nf, h->prec, h->d_stream.as<unsigned char>(),
-                h->d_slot.as<double>(), h->stream);
-    launch_pack(h->d_pk_off_c.as<long long>(), h->d_pk_src_c.as<int>(), h->pk_nc, h->lump32 ? 1 : 0,
-                h->d_stream.as<unsigned char>(), h->d_slot.as<double>(), h->stream);
+    unsigned char* stream = h->d_stream.as<unsigned char>();
+    const long long* off_f = reinterpret_cast<const long long*>(stream + h->stream_base[h->sym->subs.size()]);
+    const long long* off_c = off_f + h->pk_nf;
+    const int* src_f = reinterpret_cast<const int*>(off_c + h->pk_nc);
+    launch_pack(off_f, src_f, h->pk_nf, h->prec, stream, h->d_slot.as<double>(), h->stream);
+    launch_pack(off_c, src_f + h->pk_nf, h->pk_nc, h->lump32 ? 1 : 0, stream, h->d_slot.as<double>(), h->stream);
     ck(cudaGetLastError());
     h->rows_packed = true;
 }
-// before a launch of configuration cfg: the stream it reads holds the current factors
-void use_stream(asm_ctx* h, const ApplyConfig& cfg) {
-    if (h->opt.local_solver == ASM_LOCAL_EXACT || is_nf(h)) return;
-    if (cfg.ymode == Y_PACKET) {
-        if (!h->lanes_packed) pack_lanes(h);
-    } else {
-        if (!h->rows_ready) upload_rows(h);
-        if (!h->rows_packed) pack_rows(h);
+// before a launch of configuration cfg: the streams it reads hold the current factors
+void use_stream(const std::vector<asm_ctx*>& hs, const ApplyConfig& cfg) {
+    if (hs.empty() || hs[0]->opt.local_solver == ASM_LOCAL_EXACT || is_nf(hs[0])) return;
+    const bool by_rows = cfg.ymode != Y_PACKET;
+    std::vector<asm_ctx*> without;
+    for (asm_ctx* h : hs)
+        if (by_rows && !h->rows_ready) without.push_back(h);
+    if (!without.empty()) upload_rows(without);
+    for (asm_ctx* h : hs) {
+        if (by_rows && !h->rows_packed) pack_rows(h);
+        if (!by_rows && !h->lanes_packed) pack_lanes(h);
+        h->by_rows = by_rows;  // (only now: an upload may have failed)
     }
-    h->by_rows = cfg.ymode != Y_PACKET;  // (only now: an upload may have failed)
 }
 void upload_symbolic(asm_ctx* h) {
     SysSym& S = *h->sym;
@@ -776,7 +850,7 @@ void upload_symbolic(asm_ctx* h) {
     choose_ring(h);
     h->lanes_cap = h->lanes_smem = 0;
     h->rows_ready = h->rows_packed = h->lanes_packed = h->by_rows = false;
-    h->d_stream.alloc(16);
+    h->d_stream.release();
     std::vector<long long> lane_base(K + 1, 0);
     bool lanes = K > 0;
     for (int s = 0; s < K; s++) {
@@ -806,7 +880,7 @@ void upload_symbolic(asm_ctx* h) {
             const size_t n = first[K];
             const std::unique_ptr<long long[]> off(new long long[n + 1]);
             const std::unique_ptr<int[]> src(new int[n + 1]);
-            for_subdomains(K, n, [&](int s) {
+            for_each_task(K, n, [&](int s) {
                 const Packets& k = S.subs[s].pk;
                 const std::vector<long long>& o = group == 0 ? k.off_f : k.off_c;
                 const std::vector<int>& r = group == 0 ? k.src_f : k.src_c;
@@ -929,8 +1003,9 @@ void upload_symbolic(asm_ctx* h) {
         h->box_items.push_back(it);
     }
     choose_ring(h);
+    h->d_subdesc_single.release();
+    if (!h->lanes_ok && h->opt.local_solver != ASM_LOCAL_EXACT && !is_nf(h)) upload_rows({h});
     upload_sub_tables(h);
-    if (!h->lanes_ok && h->opt.local_solver != ASM_LOCAL_EXACT && !is_nf(h)) upload_rows(h);
     h->d_err.alloc(sizeof(FactErr));
     sync(h);
 }
@@ -1346,7 +1421,7 @@ void build_batch(Batch& B, cudaStream_t st) {
         const int ls = lanes ? lane_slots(B.hs[0], B.nsub, lanes_smem, lanes_cap, B.apply) : 0;
         if (ls > 0) B.apply = ApplyConfig{Y_PACKET, lanes_smem, ls, lanes_cap};
     }
-    for (asm_ctx* h : B.hs) use_stream(h, B.apply);  // (may move a handle's descriptors: before they are copied)
+    use_stream(B.hs, B.apply);  // (may move a handle's descriptors: before they are copied)
 
     sd = longest_first(B.hs);
     B.exact = !B.hs.empty() && B.hs[0]->opt.local_solver == ASM_LOCAL_EXACT;
@@ -1806,19 +1881,21 @@ int handle_matrix_view(asm_ctx* h, MatrixView* out) {
 
 namespace {
 
-// device bytes of a structure's stream by rows and its pack lists
+// device bytes of a structure's stream by rows and what upload_rows puts behind it
 size_t rows_bytes(const SysSym& S) {
-    size_t b = 0;
-    for (const SubSym& o : S.subs)
+    size_t b = 16;
+    for (const SubSym& o : S.subs) {
         b += (o.stream.size() + 255) / 256 * 256 + (sizeof(long long) + sizeof(int)) * (o.pk_off_f.size() + o.pk_off_c.size());
+        rows_index_pieces(o.stream, o.chunk_off, o.n_fwd_chunks, S.prec, [&](long long, size_t n) { b += n + sizeof(PkPiece); });
+    }
     return b;
 }
 
 size_t ctx_device_bytes(const asm_ctx* h) {
     const DBuf* bufs[] = {&h->d_ell_val, &h->d_ell_col, &h->d_ell_loc, &h->d_bsr_rp, &h->d_bsr_val, &h->d_bcell,
                           &h->d_cptr, &h->d_cloc, &h->d_cval, &h->d_boxsum, &h->d_slot, &h->d_dpiv, &h->d_aptr,
-                          &h->d_aloc, &h->d_acs, &h->d_along, &h->d_fp, &h->d_stream, &h->d_pk_off_f, &h->d_pk_src_f,
-                          &h->d_pk_off_c, &h->d_pk_src_c, &h->d_lanes, &h->d_ln_off_f, &h->d_ln_src_f, &h->d_ln_off_c, &h->d_ln_src_c, &h->d_lv, &h->d_rlists, &h->d_y, &h->d_corr_cells,
+                          &h->d_aloc, &h->d_acs, &h->d_along, &h->d_fp, &h->d_stream,
+                          &h->d_lanes, &h->d_ln_off_f, &h->d_ln_src_f, &h->d_ln_off_c, &h->d_ln_src_c, &h->d_lv, &h->d_rlists, &h->d_y, &h->d_corr_cells,
                           &h->d_corr, &h->d_dev_err, &h->d_gsum, &h->d_r32, &h->d_factdesc, &h->d_subdesc_single,
                           &h->d_err, &h->d_ws,
                           &h->d_scal, &h->d_ctl, &h->d_partial, &h->d_tab1, &h->d_vec1, &h->d_row1, &h->d_box1,
@@ -2405,7 +2482,7 @@ ApplyConfig single_apply_config(const asm_ctx* h, int place) {
 
 // R_i r and the fused ILU sweeps of every subdomain (after k_sums), single-system tables
 void launch_ilu_local_solves(asm_ctx* h, const ApplyConfig& cfg) {
-    use_stream(h, cfg);
+    use_stream({h}, cfg);
     if (cfg.ymode != Y_PACKET)  // (the apply by lane forms R_i r itself)
         launch_restrict(h->d_tab1.as<SysTab>(), h->d_subdesc_single.as<SubDesc>(), h->d_ritems1.as<int2>(), h->n_ritems1,
                         h->prec, h->lump32, h->stream);
@@ -2472,7 +2549,7 @@ int asm_tune_tiling(asm_handle h, int reps, asm_tiling_report* out) {
             ensure_workspace(h);
             set_ctl(h, VU, VZ, -1, -1, -1);
             const ApplyConfig cfg = single_apply_config(h, place);
-            use_stream(h, cfg);
+            use_stream({h}, cfg);
             std::vector<float> t;
             for (int k = 0; k < reps + 2; k++) {
                 ck(cudaEventRecord(e0, h->stream));

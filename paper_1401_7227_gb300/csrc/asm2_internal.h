@@ -286,6 +286,9 @@ void launch_pack(const long long* off, const int* src, long long n, int prec, un
 // the same blocks into the streams by lane (packets.h: off holds ~offset for the blocks of a long lump row)
 void launch_pack_lanes(const long long* off, const int* src, long long n, int prec, unsigned char* stream_base,
                        const double* slot_base, cudaStream_t st);
+// the parts of src to their places in dst (packets.h)
+struct PkPiece;
+void launch_place(const PkPiece* pieces, int n, const void* src, void* dst, cudaStream_t st);
 void launch_ell_fill(const double* bsr_vals, const int* row_ptr, int n, int ell_w, double* ell_val, int rows_pad,
                      cudaStream_t st);
 

@@ -4,6 +4,7 @@
 #include <cuda_fp16.h>
 
 #include "asm2_internal.h"
+#include "packets.h"
 
 namespace asm2 {
 
@@ -391,6 +392,15 @@ __global__ void k_pack_lanes(const long long* __restrict__ off, const int* __res
     }
 }
 
+// a warp per part (a few hundred bytes; a few MB in all, once per structure)
+__global__ void __launch_bounds__(256) k_place(const PkPiece* __restrict__ pieces, int n, const int4* __restrict__ src,
+                                               int4* __restrict__ dst) {
+    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (i >= n) return;
+    const PkPiece p = pieces[i];
+    for (int k = threadIdx.x & 31; k < p.n; k += 32) dst[(long long)p.dst + k] = src[(long long)p.src + k];
+}
+
 inline unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
 }  // namespace
@@ -443,6 +453,11 @@ void launch_pack(const long long* off, const int* src, long long n, int prec, un
         k_pack<float><<<g, 256, 0, st>>>(off, src, n, stream_base, slot_base);
     else
         k_pack<__half><<<g, 256, 0, st>>>(off, src, n, stream_base, slot_base);
+}
+
+void launch_place(const PkPiece* pieces, int n, const void* src, void* dst, cudaStream_t st) {
+    if (n <= 0) return;
+    k_place<<<blocks_for(32LL * n, 256), 256, 0, st>>>(pieces, n, static_cast<const int4*>(src), static_cast<int4*>(dst));
 }
 
 void launch_pack_lanes(const long long* off, const int* src, long long n, int prec, unsigned char* stream_base,

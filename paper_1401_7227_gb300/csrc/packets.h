@@ -38,6 +38,28 @@ __host__ __device__ inline int pk_issued_end(int ci, int slots, int n) {
     return end < n ? end : n;
 }
 
+// A part of a stream, in units of 16 bytes: its place in the stream and in the bytes that hold such parts back to back.
+struct PkPiece {
+    int dst, src, n;
+};
+
+// The parts of a subdomain's stream by rows that are not values (symbolic.h): of each chunk the header with the fine
+// rows' pointers and columns, and the lump rows' pointers and columns.  add(byte offset, bytes) for each.
+template <class F>
+void rows_index_pieces(const std::vector<unsigned char>& stream, const std::vector<long long>& chunk_off, int n_fwd, int prec,
+                       F add) {
+    const auto a16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+    const size_t fbb = prec == 0 ? 72 : (prec == 1 ? 36 : 20);
+    for (size_t i = 0; i < chunk_off.size(); i++) {
+        int h[8];
+        std::memcpy(h, stream.data() + chunk_off[i], sizeof(h));
+        const size_t nf = (size_t)h[1], nc = (size_t)h[3], ef = (size_t)h[4], ec = (size_t)h[5];
+        const size_t fine = 32 + a16(4 * (nf + 1)) + a16(4 * ef), values = a16(fbb * ef) + ((int)i < n_fwd ? 0 : a16(fbb * nf));
+        add(chunk_off[i], fine);
+        add(chunk_off[i] + (long long)(fine + values), a16(4 * (nc + 1)) + a16(4 * ec));
+    }
+}
+
 struct Packets {
     std::vector<unsigned char> stream;  // out and idx filled in, values zero
     std::vector<long long> chunk_off;

@@ -23,7 +23,7 @@ namespace {
 std::mutex mu;
 std::map<void*, size_t> live;
 std::map<std::string, long long> calls;
-size_t live_bytes = 0;
+size_t live_bytes = 0, h2d_bytes = 0;
 int sms = 152, stack_copies = 0, late_stack_copies = 0;
 
 void count(const char* name) {
@@ -52,10 +52,12 @@ extern "C" {
 void fk_reset(int n_sms) {
     sms = n_sms;
     calls.clear();
+    h2d_bytes = 0;
     stack_copies = late_stack_copies = 0;
 }
 long long fk_calls(const char* name) { return calls[name]; }
 long long fk_live_bytes() { return (long long)live_bytes; }
+long long fk_h2d_bytes() { return (long long)h2d_bytes; }
 int fk_late_stack_copies() { return late_stack_copies; }
 
 int asm_residual_noalloc(void*, const double*, const double*, double*, double*) { return 6; }
@@ -78,7 +80,10 @@ cudaError_t cudaMallocHost(void** p, size_t n) { return *p = std::calloc(1, n), 
 cudaError_t cudaFreeHost(void* p) { return std::free(p), cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind kind, cudaStream_t) {
     count("cudaMemcpyAsync");
-    if (kind == cudaMemcpyHostToDevice && on_stack(s)) stack_copies++;
+    if (kind == cudaMemcpyHostToDevice) {
+        h2d_bytes += n;
+        if (on_stack(s)) stack_copies++;
+    }
     std::memcpy(d, s, n);
     return cudaSuccess;
 }
@@ -133,6 +138,11 @@ void launch_init(const SysTab*, const VecItem*, int, cudaStream_t) { kernel("ini
 void launch_pack(const long long*, const int*, long long, int, unsigned char*, const double*, cudaStream_t) { kernel("pack"); }
 void launch_pack_lanes(const long long*, const int*, long long, int, unsigned char*, const double*, cudaStream_t) {
     kernel("pack_lanes");
+}
+void launch_place(const PkPiece* p, int n, const void* src, void* dst, cudaStream_t) {
+    kernel("place");
+    for (int i = 0; i < n; i++)
+        std::memcpy(static_cast<char*>(dst) + 16LL * p[i].dst, static_cast<const char*>(src) + 16LL * p[i].src, 16LL * p[i].n);
 }
 void launch_post(const SysTab*, const VecItem*, int, cudaStream_t) { kernel("post"); }
 void launch_prep(const SysTab*, const VecItem*, int, cudaStream_t) { kernel("prep"); }

@@ -131,6 +131,38 @@ std::string check_sub(const SubSym& o, int prec, bool lump32) {
 
 }  // namespace
 
+namespace {
+
+// the stream by rows is its index parts over zeros (the values are not filled in on the host)
+std::string check_rows_pieces(const SubSym& o, int prec) {
+    std::vector<unsigned char> out(o.stream.size(), 0);
+    std::string e;
+    size_t bytes = 0;
+    rows_index_pieces(o.stream, o.chunk_off, o.n_fwd_chunks, prec, [&](long long at, size_t n) {
+        if (at < 0 || at % 16 != 0 || n % 16 != 0 || n == 0 || at + n > out.size()) {
+            e = "piece range";
+            return;
+        }
+        std::memcpy(out.data() + at, o.stream.data() + at, n);
+        bytes += n;
+    });
+    if (!e.empty()) return e;
+    // and none of it is a value's place: every block's bytes lie outside the parts
+    std::vector<char> index(o.stream.size(), 0);
+    rows_index_pieces(o.stream, o.chunk_off, o.n_fwd_chunks, prec,
+                      [&](long long at, size_t n) { std::memset(index.data() + at, 1, n); });
+    const size_t fbb = prec == 0 ? 72 : (prec == 1 ? 36 : 20), lbb = prec == 0 ? 72 : 36;
+    for (long long at : o.pk_off_f)
+        for (size_t k = 0; k < fbb; k++)
+            if (index[at + k]) return "a value in a part";
+    for (long long at : o.pk_off_c)
+        for (size_t k = 0; k < lbb; k++)
+            if (index[at + k]) return "a value in a part";
+    return out == o.stream && bytes < o.stream.size() ? "" : "parts";
+}
+
+}  // namespace
+
 // geo as in host_symbolic_shim.cpp; 0, or 1 with the first difference in err
 extern "C" int pk_check(const int* geo, int n, int nnzb, const int* rp, const int* ci, int prec, int chunk_force, char* err,
                         int errlen) {
@@ -143,6 +175,7 @@ extern "C" int pk_check(const int* geo, int n, int nnzb, const int* rp, const in
     const bool lump32 = prec != 0;
     std::string e = build_pattern(n, rp, ci, nnzb, P);
     if (e.empty()) e = build_symbolic(g, P, prec, lump32, 1, S, 0, chunk_force, true);
+    for (size_t s = 0; e.empty() && s < S.subs.size(); s++) e = check_rows_pieces(S.subs[s], prec);
     for (size_t s = 0; e.empty() && s < S.subs.size(); s++) e = check_sub(S.subs[s], prec, lump32);
     std::strncpy(err, e.c_str(), (size_t)errlen - 1);
     err[errlen - 1] = 0;

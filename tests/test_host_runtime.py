@@ -32,7 +32,7 @@ def fake_path(tmp_path_factory):
 def fake(fake_path, monkeypatch):
     """The package's classes on the fake device; its counters are reset."""
     lib = C.CDLL(fake_path, mode=os.RTLD_LAZY)
-    lib.fk_calls.restype = lib.fk_live_bytes.restype = C.c_longlong
+    lib.fk_calls.restype = lib.fk_live_bytes.restype = lib.fk_h2d_bytes.restype = C.c_longlong
     monkeypatch.setattr(asm2._build, "LIB", fake_path)
     monkeypatch.setattr(asm2, "_lib", None)
     monkeypatch.setattr(asm2.C, "CDLL", lambda path: lib)
@@ -169,3 +169,26 @@ def test_a_second_wave_by_lane_gives_way_to_one_by_rows(fake, precision, nz, for
     assert fake.fk_calls(f"apply_{form}".encode()) > 0 and fake.fk_calls(f"apply_{other}".encode()) == 0
     assert fake.fk_calls(b"pack_lanes") == (2 if form == "lanes" else 0)
     sol.close()
+
+
+def test_a_stream_uploaded_in_a_solve_goes_without_its_values(fake):
+    """On 2 SMs three systems of four subdomains apply by rows, which no one of them does alone: the first solve
+    uploads their streams and pack lists, the second nothing of the kind."""
+    fake.fk_reset(2)
+    systems = [synth.grid_jacobian(16, 16, 8, k) for k in range(3)]
+    sols = [make_solver(s, (2, 2, 1)) for s in systems]
+    sent = []
+    for _ in range(2):
+        fake.fk_reset(2)
+        asm2.solve_batch(sols, [s.b for s in systems], max_iter=3)
+        sent.append(fake.fk_h2d_bytes())
+    assert fake.fk_calls(b"apply_rows") > 0
+    stats = sols[0].stats()
+    lists, streams = 3 * 12 * stats["local_blocks"], 3 * stats["factor_bytes"]
+    assert lists < sent[0] - sent[1] < lists + streams // 4
+    sols.append(make_solver(systems[0], (2, 2, 1)))
+    fake.fk_reset(2)
+    asm2.solve_batch(sols, [s.b for s in systems] + [systems[0].b], max_iter=3)
+    assert fake.fk_calls(b"place") == 1  # (one system had no stream by rows yet)
+    for sol in sols:
+        sol.close()
