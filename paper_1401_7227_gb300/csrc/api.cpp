@@ -2821,6 +2821,10 @@ int asm_get_stats(asm_handle h, asm_stats* st) {
         const ApplyConfig cfg = single_apply_config(h, place);
         st->apply_placement = placement_code(cfg.ymode);
         st->apply_slots = cfg.slots;
+        if (cfg.ymode == Y_PACKET) {  // (factor_bytes above: the stream by rows)
+            st->factor_bytes = 0;
+            for (const SubSym& o : h->sym->subs) st->factor_bytes += (long long)o.pk.stream.size();
+        }
         const ApplyConfig& l = h->last_solve_apply;
         st->last_solve_placement = l.ymode < 0 ? -1 : placement_code(l.ymode);
         st->last_solve_slots = l.ymode < 0 ? 0 : l.slots;

@@ -192,3 +192,14 @@ def test_a_stream_uploaded_in_a_solve_goes_without_its_values(fake):
     assert fake.fk_calls(b"place") == 1  # (one system had no stream by rows yet)
     for sol in sols:
         sol.close()
+
+
+def test_factor_bytes_are_those_of_the_stream_the_apply_reads(fake):
+    """By lane every packet has ten positions and a table entry, so that stream is the larger one."""
+    s = synth.grid_jacobian(16, 16, 8, 1)
+    sol = make_solver(s, (2, 2, 1), precision="fp64")
+    by_lane = sol.stats()["factor_bytes"]
+    sol.set_tuning(apply_smem=0)
+    by_rows = sol.stats()["factor_bytes"]
+    assert by_rows > 72 * sol.stats()["local_blocks"] and by_lane > 1.05 * by_rows
+    sol.close()
