@@ -85,9 +85,6 @@ struct DBuf {
 
 }  // namespace
 
-// whether the factor stream by lane is built for a system: a launch of its subdomains alone may take it (lane_slots)
-static bool wants_lanes(const Geom& g, int sms) { return g.n_sub() <= 2LL * sms; }
-
 struct Batch;
 
 struct asm_ctx {
@@ -1943,7 +1940,7 @@ unsigned long long fnv1a(const void* p, size_t n, unsigned long long h) {
 
 struct asm_server {
     asm_server_options opt{};
-    int sms = 1;
+    int sms = 1, dev_smem = 0;
     cudaStream_t stream = nullptr;
     size_t budget = 0, resident = 0;
     long long next_ticket = 1;
@@ -2007,7 +2004,7 @@ void sym_worker(asm_server* S) {
                 g.far_mode = q.far_mode;
                 e.sym = std::make_shared<SysSym>();
                 e.err = build_symbolic(g, e.pat, S->opt.precision, S->opt.lump_precision == ASM_LUMP_FP32 ? 1 : 0, 1, *e.sym, 0, 0,
-                                       wants_lanes(g, S->sms));
+                                       wants_lanes(g, S->opt.precision, S->sms, S->dev_smem));
             }
         } catch (const std::exception& ex) {
             e.sym.reset();
@@ -2184,7 +2181,7 @@ void admit(asm_server* S) {
             }
             // ~6 KB per cell resident (FP32 factors, m = 30) with one stream of the factors, and the other one
             size_t need = (size_t)r->in.n_cells * 6144;
-            if (wants_lanes(e->sym->g, S->sms)) need += rows_bytes(*e->sym);
+            if (wants_lanes(e->sym->g, S->opt.precision, S->sms, S->dev_smem)) need += rows_bytes(*e->sym);
             evict_idle(S, need);
             if (S->resident + need > S->budget && !S->active.empty()) {
                 ++it;  // no memory now: wait for systems to finish
@@ -2448,11 +2445,12 @@ int asm_factor(asm_handle h) {
         if (!h->sym_valid) {
             auto t0 = std::chrono::steady_clock::now();
             h->sym = std::make_shared<SysSym>();
-            if (h->n_sms <= 1) ck(cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, h->device));
+            ck(cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, h->device));
+            ck(cudaDeviceGetAttribute(&h->dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
             std::string e = build_symbolic(h->geom, h->pat, h->prec, h->lump32 ? 1 : 0,
                                            h->opt.local_solver == ASM_LOCAL_BILU0_COLSUM ? 1 : 0,
                                            *h->sym, 0, h->chunk_force,
-                                           h->opt.local_solver <= ASM_LOCAL_BILU0 && wants_lanes(h->geom, h->n_sms));
+                                           h->opt.local_solver <= ASM_LOCAL_BILU0 && wants_lanes(h->geom, h->prec, h->n_sms, h->dev_smem));
             if (!e.empty()) {
                 h->last_error = e;
                 h->sym.reset();
@@ -3028,7 +3026,8 @@ int asm_server_create(asm_server_handle* out, const asm_server_options* opt, voi
         delete S;
         return ASM_ERR_CUDA;
     }
-    if (cudaDeviceGetAttribute(&S->sms, cudaDevAttrMultiProcessorCount, o.device) != cudaSuccess) {
+    if (cudaDeviceGetAttribute(&S->sms, cudaDevAttrMultiProcessorCount, o.device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&S->dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, o.device) != cudaSuccess) {
         cudaGetLastError();
         delete S;
         return ASM_ERR_CUDA;

@@ -5,6 +5,7 @@
 // iteration, the structure is not).
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -101,6 +102,23 @@ struct SysSym {
 // narrower fine rows).
 std::string build_symbolic(const Geom& g, const Pattern& A, int prec, int lump32, int colsum, SysSym& out,
                            int threads, int chunk_force = 0, bool packets = false);
+
+// Whether the factor stream by lane is built for a system on a device of so many SMs and so much shared memory per
+// CTA: a launch of its subdomains alone may take it (two waves of CTAs at most), and the fine rows of the largest
+// box fit a CTA.  128 x 128 x 64 cells in 64 boxes of up to 25,920: an analysis of 0.78 s, with the packets that
+// could never be read 0.81, and 616 MB of host memory.
+inline bool wants_lanes(const Geom& g, int prec, int sms, int smem) {
+    const auto widest = [&](int n, int p) {
+        long long w = 0;
+        for (int t = 0; t < p; t++) {
+            const long long a = (long long)n * t / p - g.ov, b = (long long)n * (t + 1) / p + g.ov;
+            w = std::max(w, std::min<long long>(n, b) - std::max<long long>(0, a));
+        }
+        return w;
+    };
+    return g.n_sub() <= 2LL * sms &&
+           widest(g.nx, g.px) * widest(g.ny, g.py) * widest(g.nz, g.pz) * (prec == 0 ? 24 : 16) <= smem;
+}
 
 // Aligned 2 x 2 x 2 cell groups: group of a cell, group count, and a group's cells in the grid
 // (x, y, z each in {2 g, 2 g + 1} within the grid; z fastest, as cells are numbered)

@@ -182,6 +182,21 @@ extern "C" int pk_check(const int* geo, int n, int nnzb, const int* rp, const in
     return e.empty() ? 0 : 1;
 }
 
+// wants_lanes of a geometry; in *fits whether every subdomain's local vectors and the row of zeros fit smem bytes
+extern "C" int pk_wanted(const int* geo, int n, int nnzb, const int* rp, const int* ci, int prec, int sms, int smem, int* fits) {
+    Geom g;
+    g.nx = geo[0], g.ny = geo[1], g.nz = geo[2], g.px = geo[3], g.py = geo[4], g.pz = geo[5], g.ov = geo[6], g.nw = geo[7];
+    for (int d = 0; d < 3; d++) g.cn[d] = geo[8 + d], g.cf[d] = geo[12 + d];
+    g.far_mode = geo[11];
+    Pattern P;
+    SysSym S;
+    if (!build_pattern(n, rp, ci, nnzb, P).empty() || !build_symbolic(g, P, prec, prec != 0, 1, S, 0).empty()) return -1;
+    *fits = 1;
+    for (const SubSym& o : S.subs)
+        if ((long long)y_layout(o.nf, o.n - o.nf, prec, prec != 0).total + 32 > smem) *fits = 0;
+    return wants_lanes(g, prec, sms, smem);
+}
+
 // The ring of k_apply_packets step by step: the wait for chunk `expire` runs out.  0 if the chunks expire ..
 // pk_issued_end - 1 are just those whose copies were issued and not waited for.
 extern "C" int pk_drain_check(int slots, int n, int expire) {

@@ -74,3 +74,24 @@ def test_an_expired_wait_drains_the_copies_in_flight_and_no_others(lib, slots):
     for n in (1, 2, 3, 7, 20):
         for expire in range(n):
             assert lib.pk_drain_check(slots, n, expire) == 0, (n, expire)
+
+
+@pytest.mark.parametrize("name", GEOMS)
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_no_packets_where_the_rows_cannot_fit_a_cta(lib, name, prec):
+    """The rule that spares the analysis the packets of boxes too large for a CTA's shared memory leaves out no system
+    whose subdomains fit, whatever the limit, and keeps none whose largest box alone does not."""
+    g = GEOMS[name]
+    s = synth.grid_jacobian(g.nx, g.ny, g.nz, 3)
+    geo = np.array([g.nx, g.ny, g.nz, g.px, g.py, g.pz, g.ov, g.near_width, *g.cnear, g.far_mode, *g.cfar], dtype=np.int32)
+    rp, ci = (np.ascontiguousarray(a, dtype=np.int32) for a in (s.row_ptr, s.col_idx))
+    fits, row = C.c_int(), 24 if prec == 0 else 16
+    p = lambda a: a.ctypes.data_as(C.c_void_p)
+    spans = [max(min(n, n * (t + 1) // q + g.ov) - max(0, n * t // q - g.ov) for t in range(q))
+             for n, q in ((g.nx, g.px), (g.ny, g.py), (g.nz, g.pz))]
+    box = int(np.prod(spans)) * row
+    for smem in (box - 1, box, box + 32, 2 * box, 40 * box, 232448):
+        want = lib.pk_wanted(p(geo), s.n_cells, s.nnzb, p(rp), p(ci), prec, 152, smem, C.byref(fits))
+        assert want == (1 if smem >= box else 0)
+        assert want == 1 or fits.value == 0
+    assert lib.pk_wanted(p(geo), s.n_cells, s.nnzb, p(rp), p(ci), prec, (g.px * g.py * g.pz - 1) // 2, 232448, C.byref(fits)) == 0
