@@ -858,14 +858,24 @@ __global__ void __launch_bounds__(VEC_THREADS) k_om(const SysTab* __restrict__ t
         if (b == 0 && i >= 1 && i < nd) gram[dir(1) * kB + i] = tot[nd + i];
         __syncwarp();
         // One reciprocal per lane, not a division per link of the chain.  1 / (Q_l, Q_l) overflows below 2^-1024 (a
-        // right-hand side of 1e-150, eight digits later), so a small (Q_l, Q_l) and the products that its
-        // reciprocal multiplies are scaled by a power of two, which leaves their bits alone.
-        const double qq = i < nd ? st.scal[SL.om_qq + dir(lo + i)] : 1.0, sc = qq < 0x1p-1000 ? 0x1p600 : 1.0;
-        const double inv = i < nd ? 1.0 / (qq * sc) : 0.0;
-        double c = i < nd ? tot[i] * sc : 0.0;
-        for (int k = 0; k + 1 < nd; k++) {
-            const double beta = __shfl_sync(0xffffffffu, c * inv, k);
-            if (i > k && i < nd) c = fma(-(gram[dir(lo + k) * kB + i - k] * sc), beta, c);
+        // right-hand side of 1e-150, eight digits later), so where a (Q_l, Q_l) is small it and the products that
+        // its reciprocal multiplies are scaled by a power of two, which leaves their bits alone.  (A chain of its own:
+        // one chain for both cases took 1.3 us a step longer at 30 x 30 x 9, k = 30.)
+        const double qq = i < nd ? st.scal[SL.om_qq + dir(lo + i)] : 1.0;
+        double c = i < nd ? tot[i] : 0.0, inv = i < nd ? 1.0 / qq : 0.0;
+        if (__any_sync(0xffffffffu, qq < 0x1p-1000)) {
+            const double sc = qq < 0x1p-1000 ? 0x1p600 : 1.0;
+            c *= sc;
+            inv = i < nd ? 1.0 / (qq * sc) : 0.0;
+            for (int k = 0; k + 1 < nd; k++) {
+                const double beta = __shfl_sync(0xffffffffu, c * inv, k);
+                if (i > k && i < nd) c = fma(-(gram[dir(lo + k) * kB + i - k] * sc), beta, c);
+            }
+        } else {
+            for (int k = 0; k + 1 < nd; k++) {
+                const double beta = __shfl_sync(0xffffffffu, c * inv, k);
+                if (i > k && i < nd) c = fma(-gram[dir(lo + k) * kB + i - k], beta, c);
+            }
         }
         if (i < nd) st.scal[SL.om_beta + lo - 1 + i] = c * inv;
     } else if (ph == PH_INIT || ph == PH_OM_FINAL) {
