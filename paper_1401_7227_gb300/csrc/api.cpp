@@ -1252,7 +1252,7 @@ int factor_numeric(asm_ctx* h) {
     } else if (is_nf(h)) {
         int nmax = 0;
         for (const NFDesc& d : h->nf_desc) nmax = std::max(nmax, d.n);
-        launch_nf_factor(h->d_nfdesc1.as<NFDesc>(), (int)h->nf_desc.size(), nmax, h->nf_bz_max, h->prec, h->dev_smem,
+        launch_nf_factor(h->d_nfdesc1.as<NFDesc>(), (int)h->nf_desc.size(), nmax, h->nf_bz_max, h->prec, h->dev_smem, h->n_sms,
                          h->d_err.as<FactErr>(), h->stream);
     } else {
         launch_factor(h->d_factdesc.as<FactDesc>(), (int)S.subs.size(), h->n_sms, h->d_err.as<FactErr>(), nullptr,

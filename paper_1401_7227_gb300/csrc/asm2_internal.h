@@ -371,8 +371,8 @@ size_t nf_plane_bytes(int S, int prec);  // one plane of the apply's y (stride o
 size_t nf_apply_smem(int bx, int bz, int prec, int slots);
 // ring slots of the apply (2..4) for ndesc subdomains of at most bx_max x bz_max planes
 int nf_apply_slots(int ndesc, int bx_max, int bz_max, int prec, int sm_smem, int sms, int dev_smem);
-// nmax cells and lines of bz_max cells at most; dev_smem: the device's shared memory per CTA
-void launch_nf_factor(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec, int dev_smem, FactErr* err,
+// nmax cells and lines of bz_max cells at most; dev_smem: the device's shared memory per CTA; sms: its SMs
+void launch_nf_factor(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec, int dev_smem, int sms, FactErr* err,
                       cudaStream_t st);
 void launch_nf_apply(const SysTab* tab, const NFDesc* descs, int ndesc, int prec, int slots, size_t smem,
                      cudaStream_t st);

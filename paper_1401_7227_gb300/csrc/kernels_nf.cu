@@ -178,10 +178,8 @@ __device__ __forceinline__ TC prod(const TC* a, const TC* b, int r, int c) {
 // memory, 64 boxes of 12 x 12 x 32 cells with column sums took 8.4 ms (FP32; FP64 15.5, FP32 boxes of
 // 4 x 3 x 150 1.77), now 2.6 (9.8, 0.55), the same FP32 bits; half of what is left is G's recurrence.
 // `stages` 2, or 1 (no overlap of the fetch) for lines whose two stages do not fit.
-constexpr int kNfThreads = 256;
-
-template <typename TC>
-__global__ void __launch_bounds__(kNfThreads) k_nf_factor(const NFDesc* __restrict__ descs, int stages, FactErr* err) {
+template <typename TC, int T>
+__global__ void __launch_bounds__(T, T == 128 ? 4 : 2) k_nf_factor(const NFDesc* __restrict__ descs, int stages, FactErr* err) {
     constexpr int BS = LayF<TC>::BS, RS = LayF<TC>::RS;
     extern __shared__ __align__(16) unsigned char nf_smem[];
     __shared__ bool bad;
@@ -243,7 +241,7 @@ __global__ void __launch_bounds__(kNfThreads) k_nf_factor(const NFDesc* __restri
         else
             meanwhile();
         __syncthreads();
-        elements<TC>(bz, 0, kNfThreads, [&](int, int q, int r, int c, int o) { W[o] = prod(v + BS * q, GI + BS * q, r, c); });
+        elements<TC>(bz, 0, T, [&](int, int q, int r, int c, int o) { W[o] = prod(v + BS * q, GI + BS * q, r, c); });
         __syncthreads();
         if (seq) chain_rows(W, K, 0, W, bz, bz - 1, -1, lane);
         __syncthreads();
@@ -252,13 +250,13 @@ __global__ void __launch_bounds__(kNfThreads) k_nf_factor(const NFDesc* __restri
     for (int j = 0; j < by; j++) {
         const bool plane_term = d.colsum && j > 0;
         if (plane_term) {
-            stage_plane(j, 0, 0, 0, kNfThreads);
+            stage_plane(j, 0, 0, 0, T);
             __syncthreads();
             for (int i = 0; i < 2 * bx - 1; i++) {
                 const int b = stages == 2 ? i & 1 : 0, l = i < bx ? i : 2 * bx - 2 - i;
                 TC *rhs = fix(NB_RHS), *W = fix(NB_W);
                 const TC *src = st(b, ST_SRC), *mx = st(b, ST_MX), *post = st(b, ST_POST);
-                elements<TC>(bz, 0, kNfThreads, [&](int t, int q, int r, int c, int o) {
+                elements<TC>(bz, 0, T, [&](int t, int q, int r, int c, int o) {
                     TC v = src[o];
                     if (i > 0) v -= prod(W + BS * q, mx + BS * q, r, c);
                     rhs[o] = v;
@@ -266,33 +264,33 @@ __global__ void __launch_bounds__(kNfThreads) k_nf_factor(const NFDesc* __restri
                 });
                 __syncthreads();
                 line_solve(rhs, st(b, ST_N), st(b, ST_K), st(b, ST_GI), [&] {
-                    if (stages == 2 && i + 1 < 2 * bx - 1) stage_plane(j, i + 1, b ^ 1, 32, kNfThreads - 32);
+                    if (stages == 2 && i + 1 < 2 * bx - 1) stage_plane(j, i + 1, b ^ 1, 32, T - 32);
                 });
                 if (i >= bx - 1)
-                    elements<TC>(bz, 0, kNfThreads, [&](int t, int q, int r, int c, int) {
+                    elements<TC>(bz, 0, T, [&](int t, int q, int r, int c, int) {
                         cs3[9 * l * bz + t] = prod(W + BS * q, post + BS * q, r, c);
                     });
                 if (stages != 2 && i + 1 < 2 * bx - 1) {
                     __syncthreads();
-                    stage_plane(j, i + 1, 0, 0, kNfThreads);
+                    stage_plane(j, i + 1, 0, 0, T);
                     __syncthreads();
                 }
             }
             __syncthreads();
         }
-        stage_line(j, 0, 0, false, plane_term, 0, kNfThreads);
+        stage_line(j, 0, 0, false, plane_term, 0, T);
         __syncthreads();
         for (int l = 0; l < bx; l++) {
             const int b = stages == 2 ? l & 1 : 0, p0 = j * S + l * bz;
             const bool line_term = d.colsum && l > 0;
             const auto next = [&] {
-                if (stages == 2 && l + 1 < bx) stage_line(j, l + 1, b ^ 1, d.colsum, plane_term, 32, kNfThreads - 32);
+                if (stages == 2 && l + 1 < bx) stage_line(j, l + 1, b ^ 1, d.colsum, plane_term, 32, T - 32);
             };
             TC *cs2 = fix(NB_CS2), *G = fix(NB_G), *GI = fix(NB_GI);
             if (line_term) {
                 line_solve(st(b, ST_SRC), fix(NB_N), fix(NB_K), GI, next);
                 const TC *W = fix(NB_W), *post = st(b, ST_POST);
-                elements<TC>(bz, 0, kNfThreads,
+                elements<TC>(bz, 0, T,
                              [&](int, int q, int r, int c, int o) { cs2[o] = prod(W + BS * q, post + BS * q, r, c); });
                 __syncthreads();
             }
@@ -341,7 +339,7 @@ __global__ void __launch_bounds__(kNfThreads) k_nf_factor(const NFDesc* __restri
             // G, G^{-1} and, for the line and plane solves, N_q and K_q
             TC *N = fix(NB_N), *K = fix(NB_K);
             const TC *L1 = st(b, ST_L1), *U1 = st(b, ST_U1);
-            elements<TC>(bz, 0, kNfThreads, [&](int t, int q, int r, int c, int o) {
+            elements<TC>(bz, 0, T, [&](int t, int q, int r, int c, int o) {
                 const long long at = 9LL * p0 + t;
                 const TC n = prod(GI + BS * q, U1 + BS * q, r, c);
                 const TC k = q + 1 < bz ? prod(L1 + BS * (q + 1), GI + BS * q, r, c) : TC(0), gi = GI[o];
@@ -355,7 +353,7 @@ __global__ void __launch_bounds__(kNfThreads) k_nf_factor(const NFDesc* __restri
             });
             __syncthreads();
             if (stages != 2 && l + 1 < bx) {
-                stage_line(j, l + 1, 0, d.colsum, plane_term, 0, kNfThreads);
+                stage_line(j, l + 1, 0, d.colsum, plane_term, 0, T);
                 __syncthreads();
             }
         }
@@ -927,27 +925,37 @@ size_t nf_factor_smem(int bz, int prec, int stages) {
 }
 
 template <typename TC>
-void nf_factor_t(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec, int dev_smem, FactErr* err, cudaStream_t st) {
+void nf_factor_t(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec, int dev_smem, int sms, FactErr* err,
+                 cudaStream_t st) {
     const dim3 ggrid((unsigned)((BD_N * nmax + 127) / 128), (unsigned)ndesc);
     const dim3 grid((unsigned)((nmax + 127) / 128), (unsigned)ndesc);
     // one stage always fits where the apply's two ring slots (1,056 bytes a cell in FP64 and 720 in FP32,
     // against 1,008 and 672 here) and its plane vectors do
     const int stages = nf_factor_smem(bz_max, prec, 2) <= (size_t)dev_smem - 1024 ? 2 : 1;
     const size_t smem = nf_factor_smem(bz_max, prec, stages);
-    allow_dynamic_smem((const void*)k_nf_factor<TC>, (int)smem);
     k_nf_gather<TC><<<ggrid, 128, 0, st>>>(descs);
-    k_nf_factor<TC><<<ndesc, kNfThreads, smem, st>>>(descs, stages, err);
+    // CTAs of 256 threads fit an SM twice (registers); where that does not hold the launch and shared memory has room
+    // for more, CTAs of 128, up to four: a re-factor of 128 x 128 x 64 cells in 512 boxes, FP64 24.5 -> 14.4 ms (22.5
+    // with one warp per box), FP32 8.6 -> 6.6; 128 x 128 x 32 in 320, 15.4 -> 10.8 and 4.9 -> 4.0.
+    const auto factor = [&](auto kernel, int threads) {
+        allow_dynamic_smem((const void*)kernel, (int)smem);
+        kernel<<<ndesc, threads, smem, st>>>(descs, stages, err);
+    };
+    if (ndesc <= 2 * sms || 3 * (smem + 1024) > (size_t)dev_smem)
+        factor(k_nf_factor<TC, 256>, 256);
+    else
+        factor(k_nf_factor<TC, 128>, 128);
     k_nf_pack<TC><<<grid, 128, 0, st>>>(descs);
 }
 }  // namespace
 
-void launch_nf_factor(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec, int dev_smem, FactErr* err,
+void launch_nf_factor(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec, int dev_smem, int sms, FactErr* err,
                       cudaStream_t st) {
     if (ndesc <= 0) return;
     if (prec == 0)
-        nf_factor_t<double>(descs, ndesc, nmax, bz_max, prec, dev_smem, err, st);
+        nf_factor_t<double>(descs, ndesc, nmax, bz_max, prec, dev_smem, sms, err, st);
     else
-        nf_factor_t<float>(descs, ndesc, nmax, bz_max, prec, dev_smem, err, st);
+        nf_factor_t<float>(descs, ndesc, nmax, bz_max, prec, dev_smem, sms, err, st);
 }
 
 void launch_nf_apply(const SysTab* tab, const NFDesc* descs, int ndesc, int prec, int slots, size_t smem,
