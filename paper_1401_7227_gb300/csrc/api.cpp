@@ -1534,7 +1534,7 @@ int local_solve_launches(const Batch& B) { return B.nf || (!B.exact && B.apply.y
 // A_i^{-1} R_i r, or the nested-factorisation sweeps
 void launch_local_solves(Batch& B, const SysTab* tab, cudaStream_t st) {
     if (B.nf) {
-        launch_nf_apply(tab, B.d_nf.as<NFDesc>(), B.nnf, B.prec, B.nf_slots, B.nf_smem, st);
+        launch_nf_apply(tab, B.d_nf.as<NFDesc>(), B.nnf, B.prec, B.nf_slots, B.nf_smem, B.hs[0]->n_sms, st);
     } else if (B.exact) {
         launch_dense_restrict(tab, B.d_sub.as<SubDesc>(), B.nsub, st);
         launch_dense_apply(tab, B.d_sub.as<SubDesc>(), B.d_dense.as<int2>(), B.ndense, st);
@@ -2503,7 +2503,7 @@ int asm_apply_precond(asm_handle h, const double* r, double* z, int on_device) {
         bool by_lane = false;
         if (is_nf(h)) {
             launch_nf_apply(h->d_tab1.as<SysTab>(), h->d_nfdesc1.as<NFDesc>(), (int)h->nf_desc.size(), h->prec,
-                            h->nf_slots, h->nf_smem, h->stream);
+                            h->nf_slots, h->nf_smem, h->n_sms, h->stream);
         } else if (h->opt.local_solver == ASM_LOCAL_EXACT) {
             launch_dense_restrict(h->d_tab1.as<SysTab>(), h->d_subdesc_single.as<SubDesc>(), (int)h->sub_desc.size(),
                                   h->stream);

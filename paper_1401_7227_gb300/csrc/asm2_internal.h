@@ -375,7 +375,7 @@ int nf_apply_slots(int ndesc, int bx_max, int bz_max, int prec, int sm_smem, int
 void launch_nf_factor(const NFDesc* descs, int ndesc, int nmax, int bz_max, int prec, int dev_smem, int sms, FactErr* err,
                       cudaStream_t st);
 void launch_nf_apply(const SysTab* tab, const NFDesc* descs, int ndesc, int prec, int slots, size_t smem,
-                     cudaStream_t st);
+                     int sms, cudaStream_t st);
 // ORTHOMIN(k): pass 0 .. number of projection blocks of the direction in progress (pass 0 also reduces
 // ||r|| of initial systems and ||b - A x|| of finishing ones), then x += alpha p, r -= alpha q.
 void launch_om(const SysTab* tab, const VecItem* items, int nitems, int pass, cudaStream_t st);

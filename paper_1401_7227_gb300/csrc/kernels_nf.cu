@@ -664,11 +664,18 @@ __device__ __forceinline__ T to_compute(double v) {
 }
 
 // B_i^{-1} R_i r for one subdomain per CTA, owned cells written to the apply output.  Warp 0 solves the lines;
-// warp 1 issues the copies, a slot's next line as soon as warp 0 has released it.  What bounds the kernel is the
-// serial path of warp 0, ~3,600 cycles a line of 32 cells in FP32 (the two recurrences 850 each at 16 steps,
+// warp 1 issues the copies, a slot's next line as soon as warp 0 has released it (SPREAD may exchange them).  What
+// bounds the kernel is the serial path of warp 0, ~3,600 cycles a line of 32 cells in FP32 (the two recurrences 850
+// each at 16 steps,
 // G^{-1} u 460, the wait 300, the other passes 240 - 410): addresses and copies of the next line, and the
 // conversion of r, are off it (64 boxes of 12 x 12 x 32 cells, an apply as called: FP32 1,084 -> 985 us, FP64
 // 4,360 -> 4,160).
+// SPREAD, for launches of more than two CTAs per SM: which of its two warps solves, a CTA takes from its place in the SM
+// (%warpid, read once; any value is right), so that the solving warps of four CTAs are in four sub-partitions.  The first
+// warps of every other CTA share one, and two line recurrences then take each other's issue slots.  512 boxes
+// (128 x 128 x 64), an apply as called, FP32: 1,452 us with first warps, 1,220 spread (1,222 with one warp per CTA), FP64
+// 4,953 and 4,918; 320 boxes 1,057 and 918.  With one or two CTAs per SM first warps are apart, and this form is 1 %
+// slower (64 boxes: 964 and 974).
 // Shared memory: SLOTS + 1 pairs of mbarriers (16 bytes: a slot is full | is free; y_j has come | the producer's
 // two words) | SLOTS packet slots | SLOTS slots for the
 // line's part of r (FP64) | plane vector pv [VS S] | y_j of a backward plane [VS S] | line vector
@@ -677,7 +684,7 @@ __device__ __forceinline__ T to_compute(double v) {
 // value of a line before it overwrites it.  y_j goes to device memory (yv, one plane every
 // nf_plane_bytes) when its forward plane is done, and comes back by a bulk copy issued at the start
 // of its backward plane.
-template <typename T, int SLOTS>
+template <typename T, int SLOTS, bool SPREAD>
 __global__ void __launch_bounds__(64) k_nf_apply(const SysTab* __restrict__ tab, const NFDesc* __restrict__ descs) {
     constexpr int BS = 3 * Lay<T>::RS, VS = Lay<T>::VS;
     extern __shared__ __align__(16) unsigned char nf_smem[];
@@ -753,10 +760,20 @@ __global__ void __launch_bounds__(64) k_nf_apply(const SysTab* __restrict__ tab,
         }
         tma::mbar_init(ybar, 1);
         *stop = 0;
+        if constexpr (SPREAD) {
+            unsigned slot;
+            asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+            *issued = (int)(slot >> 2) & 1;
+        }
         tma::fence_mbar_init();
     }
     __syncthreads();
-    if (threadIdx.x >= 32) {
+    bool solver = threadIdx.x < 32;
+    if constexpr (SPREAD) {
+        solver = (int)(threadIdx.x >> 5) == *issued;
+        __syncthreads();
+    }
+    if (!solver) {
         if (lane == 0) {
             LineStep nx;  // the next line solve to issue
             nx.set(bx, by);
@@ -887,19 +904,25 @@ __global__ void __launch_bounds__(64) k_nf_apply(const SysTab* __restrict__ tab,
 }
 
 template <typename T, int SLOTS>
-void nf_apply_t(const SysTab* tab, const NFDesc* descs, int ndesc, size_t smem, cudaStream_t st) {
-    allow_dynamic_smem((const void*)k_nf_apply<T, SLOTS>, (int)smem);
-    k_nf_apply<T, SLOTS><<<ndesc, 64, smem, st>>>(tab, descs);
+void nf_apply_t(const SysTab* tab, const NFDesc* descs, int ndesc, size_t smem, int sms, cudaStream_t st) {
+    const auto apply = [&](auto kernel) {
+        allow_dynamic_smem((const void*)kernel, (int)smem);
+        kernel<<<ndesc, 64, smem, st>>>(tab, descs);
+    };
+    if (ndesc <= 2 * sms)
+        apply(k_nf_apply<T, SLOTS, false>);
+    else
+        apply(k_nf_apply<T, SLOTS, true>);
 }
 
 template <typename T>
-void nf_apply_s(const SysTab* tab, const NFDesc* descs, int ndesc, int slots, size_t smem, cudaStream_t st) {
+void nf_apply_s(const SysTab* tab, const NFDesc* descs, int ndesc, int slots, size_t smem, int sms, cudaStream_t st) {
     if (slots >= 4)
-        nf_apply_t<T, 4>(tab, descs, ndesc, smem, st);
+        nf_apply_t<T, 4>(tab, descs, ndesc, smem, sms, st);
     else if (slots == 3)
-        nf_apply_t<T, 3>(tab, descs, ndesc, smem, st);
+        nf_apply_t<T, 3>(tab, descs, ndesc, smem, sms, st);
     else
-        nf_apply_t<T, 2>(tab, descs, ndesc, smem, st);
+        nf_apply_t<T, 2>(tab, descs, ndesc, smem, sms, st);
 }
 
 }  // namespace
@@ -959,12 +982,12 @@ void launch_nf_factor(const NFDesc* descs, int ndesc, int nmax, int bz_max, int 
 }
 
 void launch_nf_apply(const SysTab* tab, const NFDesc* descs, int ndesc, int prec, int slots, size_t smem,
-                     cudaStream_t st) {
+                     int sms, cudaStream_t st) {
     if (ndesc <= 0) return;
     if (prec == 0)
-        nf_apply_s<double>(tab, descs, ndesc, slots, smem, st);
+        nf_apply_s<double>(tab, descs, ndesc, slots, smem, sms, st);
     else
-        nf_apply_s<float>(tab, descs, ndesc, slots, smem, st);
+        nf_apply_s<float>(tab, descs, ndesc, slots, smem, sms, st);
 }
 
 int nf_apply_slots(int ndesc, int bx_max, int bz_max, int prec, int sm_smem, int sms, int dev_smem) {
