@@ -1599,7 +1599,7 @@ void launch_step_om(Batch& B, int kmax, cudaStream_t st, StepEvents* ev) {
     }
     launch_spmv(tab, B.d_row.as<RowItem>(), B.nrow, st);
     if (ev) ck(cudaEventRecord(ev->e[4], st));
-    for (int l = 0; l <= kmax; l++) launch_om(tab, vi, B.nvec, l, st);
+    for (int l = 0; l <= kmax; l++) launch_om(tab, vi, B.nvec, l, B.hs[0]->n_sms, st);
     launch_om_update(tab, vi, B.nvec, st);
     if (ev) ck(cudaEventRecord(ev->e[5], st));
     ck(cudaGetLastError());
@@ -1694,7 +1694,7 @@ int run_krylov(std::vector<asm_ctx*>& hs, const double* const* b, double* const*
         const VecItem* vi = B.d_vec.as<VecItem>();
         launch_init(tab, vi, B.nvec, st);
         if (om) {
-            launch_om(tab, vi, B.nvec, 0, st);
+            launch_om(tab, vi, B.nvec, 0, hs[0]->n_sms, st);
         } else if (B.coop_grid > 0) {
             ck(launch_ortho_coop(tab, hs[0]->d_partial.as<double>(), B.coop_grid, hs[0]->tab.ortho, hs[0]->tab.n3, st));
         } else {

@@ -378,7 +378,7 @@ void launch_nf_apply(const SysTab* tab, const NFDesc* descs, int ndesc, int prec
                      int sms, cudaStream_t st);
 // ORTHOMIN(k): pass 0 .. number of projection blocks of the direction in progress (pass 0 also reduces
 // ||r|| of initial systems and ||b - A x|| of finishing ones), then x += alpha p, r -= alpha q.
-void launch_om(const SysTab* tab, const VecItem* items, int nitems, int pass, cudaStream_t st);
+void launch_om(const SysTab* tab, const VecItem* items, int nitems, int pass, int sms, cudaStream_t st);
 void launch_om_update(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st);
 // Coarse-grid correction: [A_C | I] from the box-pair blocks, then in-place Gauss-Jordan (one
 // cooperative launch; *err = 1 + column of a zero pivot); and the per-apply kernels

@@ -720,8 +720,14 @@ __device__ void om_state(const SysTab& st, int ph, double nrm) {
 // block apart are kept: the newest direction's are taken in pass 0 of the step after its own, in the sweep that
 // reads the same vectors.  What bounded a step was its serial launches: at 30x30x9, k = 30, up to 31 of 15 us are
 // now three, and a solve of 29 steps takes 5.1 ms instead of 9.2.
-__global__ void __launch_bounds__(VEC_THREADS) k_om(const SysTab* __restrict__ tab, const VecItem* __restrict__ items,
-                                                    int b) {
+// MINB: CTAs per SM that the registers are limited for (0: no limit, 156 registers).  Launches of more CTAs than SMs
+// take two (128 registers, a few bytes spilled outside the sweeps): they are bound by the FP64 unit, which eight warps
+// alone do not keep busy.  128 x 128 x 64 FP32, a solve with k = 5: 79.5 ms with one, 71.2 with two (77.5 with a launch per
+// direction); k = 30 76.9 and 65.5; two systems of 64 x 64 x 48, k = 30 17.0 and 15.3.  Where one CTA per SM is all
+// there is, the limit costs: 64 x 64 x 48 alone 11.6 and 12.2.
+template <int MINB>
+__global__ void __launch_bounds__(VEC_THREADS, MINB) k_om(const SysTab* __restrict__ tab,
+                                                          const VecItem* __restrict__ items, int b) {
     const VecItem it = items[blockIdx.x];
     const SysTab& st = tab[it.sys];
     if (st.krylov != 1) return;
@@ -1485,8 +1491,12 @@ cudaError_t launch_ortho_coop(const SysTab* tab, double* part2, int grid, int or
     return cudaLaunchCooperativeKernel(ortho_kernel(ortho, n3), dim3(grid), dim3(VEC_THREADS), args, 0, st);
 }
 
-void launch_om(const SysTab* tab, const VecItem* items, int nitems, int pass, cudaStream_t st) {
-    if (nitems > 0) k_om<<<nitems, VEC_THREADS, 0, st>>>(tab, items, pass);
+void launch_om(const SysTab* tab, const VecItem* items, int nitems, int pass, int sms, cudaStream_t st) {
+    if (nitems <= 0) return;
+    if (nitems <= sms)
+        k_om<0><<<nitems, VEC_THREADS, 0, st>>>(tab, items, pass);
+    else
+        k_om<2><<<nitems, VEC_THREADS, 0, st>>>(tab, items, pass);
 }
 void launch_om_update(const SysTab* tab, const VecItem* items, int nitems, cudaStream_t st) {
     if (nitems > 0) k_om_update<<<nitems, VEC_THREADS, 0, st>>>(tab, items);
