@@ -593,11 +593,12 @@ def spmv_roofline(res, system, steps: int):
 
 def ortho_roofline(res, system, steps: int, m: int):
     """Modified Gram-Schmidt (k_ortho_long, one cooperative launch per Arnoldi step; the timer also
-    holds the small per-step control kernels).  Step j of a cycle makes j + 2 fused passes over
-    the 3N-vector w, each 2 FP64 FMAs per element (w -= h v_prev; dot with the next v, or the
-    norm), and one scaling pass: 4 * 3N * (j + 2) + 3N flops.  It reads v_0..v_j, w once and writes
-    v_{j+1}: 8 * 3N * (j + 3) algorithmic bytes (w stays in L2 between passes).  Bound: the FP64
-    pipe, against the nominal 1.25 TFLOP/s."""
+    holds the small per-step control kernels).  Counted are the method's own operations: for step j of
+    a cycle j + 1 dots and j + 1 subtractions with the 3N-vector w, ||w|| before and after, each an
+    FP64 FMA per element, and one scaling: 4 * 3N * (j + 2) + 3N flops; and v_0..v_j, w read once and
+    v_{j+1} written: 8 * 3N * (j + 3) bytes.  The kernel does more: it takes the vectors in blocks, each
+    read once for its dots (and, in the block of v_j, its products with v_j: a third FMA) and again for
+    its subtractions.  Bound: the FP64 pipe, against the nominal 1.25 TFLOP/s."""
     info = res["info"]
     n3 = 3.0 * system.n_cells
     flops = byt = 0.0

@@ -258,11 +258,13 @@ int asm_solve_batch(asm_handle* hs, int n, const double* const* b, double* const
 int asm_get_stats(asm_handle h, asm_stats* st);
 
 /* Tuning switches of the kernels (none changes the arithmetic of a fine row; results are bitwise
- * the same, except where ASM_TUNE_CHUNK_KB says otherwise):
+ * the same, except where ASM_TUNE_COOP_ORTHO and ASM_TUNE_CHUNK_KB say otherwise):
  *   ASM_TUNE_APPLY_SMEM  where the apply keeps each subdomain's local vectors.  1 (default):
  *                        all in shared memory with the factor stream laid out by lane (512-thread
- *                        CTAs; not for FP64 lump rows under narrower fine rows) when the launch is at
- *                        most two waves of CTAs and every subdomain fits; else all in shared memory
+ *                        CTAs; not for FP64 lump rows under narrower fine rows, nor for rows of more
+ *                        than 255 blocks on a side of the diagonal) when the launch is at most two
+ *                        waves of CTAs and every subdomain fits (in FP32 and FP16S not where it would
+ *                        take a second wave that the next form does not); else all in shared memory
  *                        (256-thread CTAs) when every subdomain CTA of the
  *                        launch then runs at once; else the lump vector in shared memory and the
  *                        fine-row vector in device memory when that fits; else all in device memory
@@ -271,7 +273,9 @@ int asm_get_stats(asm_handle h, asm_stats* st);
  *                        not fit).  The first launch of a handle that leaves the stream by lane
  *                        uploads the other stream;
  *   ASM_TUNE_COOP_ORTHO  1 (default) runs the Gram-Schmidt step of a single-system solve in one
- *                        cooperative launch, 0 in one launch per block of basis vectors.
+ *                        cooperative launch, 0 in one launch per block of basis vectors.  The two add
+ *                        the partial sums in another order and, above 131,072 unknowns, take blocks of
+ *                        four and of eight vectors, so their iterates agree to rounding only;
  * Errors: INVALID_ARG for an unknown key or value. */
 typedef enum {
     ASM_TUNE_APPLY_SMEM = 0,
@@ -279,7 +283,9 @@ typedef enum {
     ASM_TUNE_AUTOTUNE = 2, /* 1 (default): a solve's first apply steps try every placement of the
                               local vectors that fits (a warm-up round, then a timed round) and
                               keep the fastest; remembered per handle for single-system solves.
-                              Placements give bitwise equal results.  0: the placement rule only. */
+                              Placements give bitwise equal results.  Launches that take the factor
+                              stream by lane (ASM_TUNE_APPLY_SMEM) are not timed: they keep it.
+                              0: the placement rule only. */
     ASM_TUNE_GRAPHS = 3,   /* 1 (default): batched solves replay each Krylov step as a captured
                               CUDA graph (one per projection count); 0: plain launches */
     ASM_TUNE_WAIT_LIMIT = 4, /* failure-detection hook (0..30, default 22): the apply kernels (ILU
@@ -300,7 +306,8 @@ typedef enum {
                               are chosen per chunk) */
     ASM_TUNE_APPLY_SLOTS = 6 /* ring slots of the apply: 0 (default) with all local vectors in
                               shared memory as many as keep two CTAs per SM, else 4, and 2 with the
-                              other placements; 2, 3 or 4 for every placement */
+                              other placements; 2, 3 or 4 for every placement (the
+                              automatic one then leaves the stream by lane) */
 } asm_tune_key;
 int asm_set_tuning(asm_handle h, int key, int value);
 
@@ -309,8 +316,9 @@ int asm_set_tuning(asm_handle h, int key, int value);
  * preconditioner apply under every stream-chunk capacity (ASM_TUNE_CHUNK_KB: the rule, 8, 12, 16,
  * 20, 24 KB; capacities that give every subdomain the same chunks as an earlier one are skipped)
  * crossed with every placement of the local vectors that fits (all in shared memory, lumps in
- * shared memory, all in device memory) and 2, 3 or 4 ring slots, each as the median of `reps` timed
- * applies after two untimed ones.  It then leaves the fastest in place (ASM_TUNE_CHUNK_KB,
+ * shared memory, all in device memory) and 2, 3 or 4 ring slots, and with the factor stream by lane
+ * where the rule takes it (ASM_TUNE_APPLY_SMEM), each as the median of `reps` timed applies after two
+ * untimed ones.  It then leaves the fastest in place (ASM_TUNE_CHUNK_KB,
  * ASM_TUNE_APPLY_SLOTS and ASM_TUNE_APPLY_SMEM set, the online placement tuner off) with the
  * handle factored again, and reports every measurement.  Each capacity costs one symbolic rebuild
  * and factorisation, so this is a set-up step to run once per structure.  The handle's values are
@@ -322,7 +330,7 @@ typedef struct {
     int chunk_max_kb;  /* the largest capacity the subdomains got (a ring slot's size) */
     long long chunks;  /* stream chunks of all subdomains, both sweeps */
     int placement;     /* ASM_TUNE_APPLY_SMEM value: 3 all in shared memory, 2 lumps, 0 device */
-    int slots;         /* ring slots */
+    int slots;         /* ring slots (up to 8 with the stream by lane) */
     int ctas_per_sm;   /* apply CTAs resident per SM */
     double apply_ms;   /* median time of one preconditioner apply (all its kernels) */
 } asm_tiling_entry;

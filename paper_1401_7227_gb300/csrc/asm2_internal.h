@@ -20,7 +20,9 @@ namespace asm2 {
 constexpr int VEC_CHUNK = 4096;   // vectors are padded to whole chunks of this many elements
 // Elements per vector work item (one CTA of 256 threads): a quarter of a chunk for short vectors, so
 // that a few of them fill the chip, a whole one where the partial sums of a long vector would
-// otherwise outnumber what the last CTA adds up quickly.
+// otherwise outnumber what the last CTA adds up quickly.  A solve of two FP32 systems of n3 unknowns, and ORTHOMIN(30)
+// of one, ms, with a quarter | a whole: n3 = 40k 5.7 | 7.4 and 4.8 | 6.6; 120k 6.8 | 8.2 and 5.8 | 8.0; 263k 10.1 | 10.4
+// and 8.3 | 9.5; 395k 12.8 | 12.6 and 10.7 | 10.9; 590k 15.8 | 13.8 and 12.8 | 11.6; 1.6M 37.2 | 32.5 and 25.0 | 21.8.
 inline int vec_item_len(long long n3) { return n3 <= 400000 ? VEC_CHUNK / 4 : VEC_CHUNK; }
 // Basis vectors per reduction of the blocked modified Gram-Schmidt, and per sweep over the vectors
 constexpr int kGsMaxBlock = 32, kGsGroup = 8, kGsLong = 4;
@@ -131,7 +133,8 @@ struct SysTab {
     int gs_block;        // basis vectors per Gram-Schmidt reduction (kGsGroup or kGsMaxBlock)
     double* scal;        // scalars (ScalLayout)
     int* ctl;            // control words (Ctl)
-    double* partial;     // [nchunk * (2 gs_block + 1)] chunk partial sums
+    double* partial;     // chunk partial sums: 2 gs_block + 1 a chunk (ORTHOMIN 2 kGsMaxBlock + 1), or those of
+                         // the cooperative Gram-Schmidt's CTAs (ensure_workspace)
     // A in ELL form: slot w, element t of row r at ell_val[(w*9 + t) * rows_pad + r]
     const double* ell_val;
     const int* ell_col;  // [w * rows_pad + r]; padding slots point at r with zero values

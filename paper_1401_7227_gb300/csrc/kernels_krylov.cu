@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kSpmvThreads, 6) k_spmv(const SysTab* __restri
 }
 
 // ------------------------------------------------------------------------------------------
-// GMRES vector kernels.  A chunk is VEC_CHUNK elements of one system; reductions write one
+// GMRES vector kernels.  A chunk is a work item of one system (vec_item_len elements); reductions write one
 // partial per chunk and the last chunk to arrive sums the partials in index order, so every
 // result is independent of scheduling and of the other systems in the launch.
 // ------------------------------------------------------------------------------------------
@@ -721,7 +721,7 @@ __device__ void om_state(const SysTab& st, int ph, double nrm) {
 // reads the same vectors.  What bounded a step was its serial launches: at 30x30x9, k = 30, up to 31 of 15 us are
 // now three, and a solve of 29 steps takes 5.1 ms instead of 9.2.
 // MINB: CTAs per SM that the registers are limited for (0: no limit, 156 registers).  Launches of more CTAs than SMs
-// take two (128 registers, a few bytes spilled outside the sweeps): they are bound by the FP64 unit, which eight warps
+// take two (128 registers, 32 bytes spilled): they are bound by the FP64 unit, which eight warps
 // alone do not keep busy.  128 x 128 x 64 FP32, a solve with k = 5: 79.5 ms with one, 71.2 with two (77.5 with a launch per
 // direction); k = 30 76.9 and 65.5; two systems of 64 x 64 x 48, k = 30 17.0 and 15.3.  Where one CTA per SM is all
 // there is, the limit costs: 64 x 64 x 48 alone 11.6 and 12.2.
@@ -1246,7 +1246,7 @@ __device__ __forceinline__ double ortho_beta(const SysTab& st, double* part2, co
     return sqrt(gs_grid_sum(s0, part2, grid));
 }
 
-// Short vectors (st.gs_block = kGsMaxBlock: up to 862 elements per SM): a handful of elements per thread, so
+// Short vectors (st.gs_block = kGsMaxBlock: up to 131,072 values, 862 per SM): a handful of elements per thread, so
 // what counts is the number of barriers and of dependent FP64 operations.
 __global__ void __launch_bounds__(VEC_THREADS, 1) k_ortho_short(const SysTab* __restrict__ tab, double* __restrict__ part2) {
     namespace cg = cooperative_groups;

@@ -9,11 +9,11 @@
 // depends on the previous line of its plane, every plane on the previous plane.  So one CTA takes
 // one subdomain: in the factorisation one of its warps runs the recurrences of a line (FP64 and the
 // 3x3 block algebra of G: lane 3 r + c holds element (r, c) of a block), the others fetch the next
-// line's operands, and all share the independent per-cell products.  The apply (one warp) streams one
-// packet per line -- G^{-1}, G^{-1} L1, G^{-1} U1, their two-step products, L2, L3, U3, U2 of the line's
+// line's operands, and all share the independent per-cell products.  The apply (one warp that solves, one
+// that issues the copies) streams one packet per line -- G^{-1}, G^{-1} L1, G^{-1} U1, their two-step products, L2, L3, U3, U2 of the line's
 // cells, packed after the factorisation -- through a shared-memory ring of 2-4 slots by bulk copies,
 // ahead of the line being solved.  The products that do not depend on the line recurrences run on
-// all lanes; the two recurrences of T^{-1}, with one level of recursive doubling, run from shared
+// all lanes of the first warp; the two recurrences of T^{-1}, with one level of recursive doubling, run from shared
 // memory on one lane (FP32) or three (FP64, one row each: an FP64 instruction costs the same for one
 // lane as for 32).
 #include <cuda_runtime.h>
